@@ -300,7 +300,8 @@ ligate_status ligate_plan_best_scores(const ligate_plan *plan, float *out, int s
  * Errors: INVALID, CUDA. */
 ligate_status ligate_plan_best_quantile(ligate_plan *plan, double frac, float *out, void *stream);
 ligate_status ligate_plan_set_cutoff(ligate_plan *plan, const float *cutoff);
-/* Kernel launches one run enqueues, and the shape in use. */
+/* Docking-kernel launches one run enqueues (after the kernel that builds the
+ * rows' clash tables), and the shape in use. */
 ligate_status ligate_plan_get_tile(const ligate_plan *plan, ligate_tile *tile_out,
                                    int *kernel_launches);
 /* Work done by one run, counted from the packed batch: unique poses

@@ -999,7 +999,7 @@ static void free_plan(ligate_plan *pl) {
   cudaFree(pl->sub_items); cudaFree(pl->sub_partial); cudaFree(pl->sub_count); cudaFree(pl->sub_lig_items);
   cudaFree(pl->sub_slot0); cudaFree(pl->rowmap); cudaFree(pl->sub_row_lig); cudaFree(pl->lig_by_cost);
   cudaFree(pl->lig_bucket);
-  cudaFree(pl->p.memo1);
+  cudaFree(pl->p.memo1); cudaFree(pl->p.tab);
   if (pl->exec) cudaGraphExecDestroy(pl->exec);
   if (pl->graph) cudaGraphDestroy(pl->graph);
   if (pl->cap_stream) cudaStreamDestroy(pl->cap_stream);
@@ -1046,6 +1046,10 @@ static void model_chunks(const BatchDev &B, const int32_t *sel, int n, int S, in
     chunks[b] = std::max(G, (int)chunk / G * G);
   }
 }
+
+// Most bytes a plan keeps for its rows' clash tables (clash_tables_kernel);
+// about 12 KB per ligand at S = 16 and 12 bonds.
+constexpr size_t TAB_BUDGET = (size_t)1 << 30;
 
 // Plan over all ligands of B (sel == NULL) or over the ligands sel[0..n_sel),
 // whose results fill output rows 0..n_sel-1 in that order.
@@ -1238,16 +1242,21 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
     free_plan(pl);
     return cuda_fail(e, "plan upload");
   }
-  {  // per resident warp: the clash tables of the pairs a single earlier bond separates
+  {  // clash tables: every row's, built once per run, while they stay within TAB_BUDGET;
+     // beyond it those of the pairs a single earlier bond separates, per resident warp
     int m1 = 0;
     for (int r = 0; r < n; ++r) {
       const LigDesc &ld = B->d.h_lig[sel ? sel[r] : r];
       m1 = std::max(m1, dock_memo1_tables(ld, B->d.h_bonds.data() + ld.bond_base, p.S));
     }
-    if (m1 > 0) {
+    p.m1max = m1;
+    const size_t stride = dock_tab_stride(p.S, p.rmax, m1);
+    if (n > 0 && p.rmax > 0 && stride * sizeof(float) * n <= TAB_BUDGET) {
+      if ((e = dmalloc(&p.tab, stride * n)) != cudaSuccess) { free_plan(pl); return cuda_fail(e, "plan allocation"); }
+      p.tab_stride = (int)stride;
+    } else if (m1 > 0) {
       const size_t floats = (size_t)pl->grid * t.warps_per_cta * m1 * p.S * p.S;
       if ((e = dmalloc(&p.memo1, floats)) != cudaSuccess) { free_plan(pl); return cuda_fail(e, "plan allocation"); }
-      p.m1max = m1;
     }
   }
   p.items = pl->items;
@@ -1293,6 +1302,7 @@ static ligate_status plan_capture(ligate_plan *pl) {
   CK(cudaStreamBeginCapture(pl->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
   cudaError_t e = cudaMemsetAsync(pl->counters, 0, pl->counter_bytes, pl->cap_stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(pl->stats, 0, N_STATS * sizeof(unsigned long long), pl->cap_stream);
+  if (e == cudaSuccess && pl->p.n_items > 0) e = launch_clash_tables(pl->p, pl->row_lig, pl->n_ligands, pl->cap_stream);
   if (e == cudaSuccess && pl->p.n_items > 0)
     e = launch_dock(pl->mode, pl->tile.reg_cap, pl->p, pl->grid, pl->block, pl->smem, pl->cap_stream);
   cudaGraph_t g = nullptr;
@@ -1517,7 +1527,8 @@ extern "C" ligate_status ligate_plan_run_subset(ligate_plan *pl, const int32_t *
     q.lig_items = pl->sub_lig_items;
     q.lig_slot0 = pl->sub_slot0;
     q.partial = pl->sub_partial;
-    if ((e = launch_dock(pl->mode, pl->tile.reg_cap, q, pl->grid, pl->block, pl->smem, s)) != cudaSuccess)
+    if ((e = launch_clash_tables(q, pl->sub_row_lig, n_sel, s)) != cudaSuccess ||
+        (e = launch_dock(pl->mode, pl->tile.reg_cap, q, pl->grid, pl->block, pl->smem, s)) != cudaSuccess)
       return cuda_fail(e, "plan_run_subset: docking kernel");
   }
   if (out && n_sel > 0) {
@@ -1564,6 +1575,7 @@ extern "C" void ligate_plan_destroy(ligate_plan *pl) { free_plan(pl); }
 static cudaError_t plan_launch(ligate_plan *pl, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(pl->counters, 0, pl->counter_bytes, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(pl->stats, 0, N_STATS * sizeof(unsigned long long), st);
+  if (e == cudaSuccess && pl->p.n_items > 0) e = launch_clash_tables(pl->p, pl->row_lig, pl->n_ligands, st);
   if (e == cudaSuccess && pl->p.n_items > 0)
     e = launch_dock(pl->mode, pl->tile.reg_cap, pl->p, pl->grid, pl->block, pl->smem, st);
   pl->rows = pl->n_ligands;

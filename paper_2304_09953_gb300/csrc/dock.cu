@@ -148,115 +148,150 @@ __device__ __forceinline__ float clash_sweep(const DockParams &p, const WarpSmem
   return ac;
 }
 
-// Clash sums of the first n_memo bonds' sweeps into w.memo: memo[k] for
-// bond 0 on the input conformation, memo[S + k0 S + k] for bond 1 after
-// bond 0 turned by step k0; and of each later bond b, the sums over its
-// first n_cand0 candidates on the input conformation, memo[memo_row0(S) +
-// (b - memo_bonds(S)) S + k]; and, when m1 is given, of each bond b >= 2
-// with pairs that bond e1 alone separates, the sums over those pairs after
-// e1 turned by step t, m1[(slot S + t) S + k] (e1 and slot packed in e1).
-// Conformations are posed by start 0's frame (the clash term is invariant
-// under the rigid move); group g takes k0 = g, g + G, ...  Warp-collective.
-__device__ void build_memo(const DockParams &p, const WarpSmem &w, float4 *pose, const LigDesc &d,
-                           int n_memo, float ck, float sk, int g, int k, int L, int G, int S,
-                           float *__restrict__ m1) {
-  unsigned n_test = 0, n_pair = 0;  // not counted: once per ligand
-  float R[9], T[3];
-  start_frame(p, 0, R, T);
-  if (m1) {
-    for (int b = 2; b < d.n_rot; ++b) {
-      BondRec bb = w.bonds[b];
-      if (bb.n_cand1 == 0) continue;  // warp-uniform
-      const int slot = bb.e1 >> 16;
-      const BondRec be = w.bonds[bb.e1 & 0xffff];
-      bb.cand_off += bb.n_cand0;
-      bb.n_cand = bb.n_cand1;
-      for (int r = 0; r < (S + G - 1) / G; ++r) {
-        const int te = min(r * G + g, S - 1);  // groups past S repeat the last step
-        for (int i = k; i < d.n_atoms; i += L) {
-          const float4 a = w.ref[i];
-          pose[i] = make_float4(fmaf(R[0], a.x, fmaf(R[1], a.y, fmaf(R[2], a.z, T[0]))),
-                                fmaf(R[3], a.x, fmaf(R[4], a.y, fmaf(R[5], a.z, T[1]))),
-                                fmaf(R[6], a.x, fmaf(R[7], a.y, fmaf(R[8], a.z, T[2]))), 0.f);
-        }
-        __syncwarp();
-        float ex, ey, ez;
-        const float4 ev = pose[be.v];
-        bond_axis(pose[be.u], ev, ex, ey, ez);
-        float ce, se;
-        step_cs(p, te, ce, se);
-        Rot re;
-        re.make(ce, se, ex, ey, ez, ev.x, ev.y, ev.z);
-        __syncwarp();
-        for (int i = be.v + 1 + k; i < be.end; i += L) {
-          float4 q = pose[i];
-          re.apply(q.x, q.y, q.z, q.x, q.y, q.z);
-          pose[i] = q;
-        }
-        __syncwarp();
-        float mx, my, mz;
-        const float4 qv = pose[bb.v];
-        bond_axis(pose[bb.u], qv, mx, my, mz);
-        const float a1 = clash_sweep(p, w, pose, d, bb, mx, my, mz, qv, ck, sk, g, k, L, G, n_test, n_pair);
-        if (r * G + g < S && k < S) {  // kept in L2 ahead of streaming data (evict-last policy)
-          uint64_t pol;
-          asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-          asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(m1 + (slot * S + te) * S + k), "f"(a1),
-                       "l"(pol) : "memory");
-        }
-        __syncwarp();
-      }
-    }
+// The input conformation posed by start 0's frame (R, T), where every clash
+// table is built (the clash term is invariant under the rigid move).
+__device__ __forceinline__ void pose_input(const WarpSmem &w, float4 *pose, const LigDesc &d, const float (&R)[9],
+                                           const float (&T)[3], int k, int L) {
+  for (int i = k; i < d.n_atoms; i += L) {
+    const float4 a = w.ref[i];
+    pose[i] = make_float4(fmaf(R[0], a.x, fmaf(R[1], a.y, fmaf(R[2], a.z, T[0]))),
+                          fmaf(R[3], a.x, fmaf(R[4], a.y, fmaf(R[5], a.z, T[1]))),
+                          fmaf(R[6], a.x, fmaf(R[7], a.y, fmaf(R[8], a.z, T[2]))), 0.f);
   }
-  const int rounds = n_memo == 2 ? (S + G - 1) / G : 0;
-  for (int r = -1; r < rounds; ++r) {  // r = -1: bond 0 on the input conformation
-    for (int i = k; i < d.n_atoms; i += L) {
-      const float4 a = w.ref[i];
-      pose[i] = make_float4(fmaf(R[0], a.x, fmaf(R[1], a.y, fmaf(R[2], a.z, T[0]))),
-                            fmaf(R[3], a.x, fmaf(R[4], a.y, fmaf(R[5], a.z, T[1]))),
-                            fmaf(R[6], a.x, fmaf(R[7], a.y, fmaf(R[8], a.z, T[2]))), 0.f);
-    }
+  __syncwarp();
+}
+
+// Clash sums of the swept candidates of bond bb at every step k after bond be
+// alone turned by each step t, out[t S + k]; group g takes t = g, g + G, ...
+// LAST: stored with an L2 evict-last policy (ahead of streaming data).
+// Warp-collective.
+template <bool LAST>
+__device__ void turn_table(const DockParams &p, const WarpSmem &w, float4 *pose, const LigDesc &d, const BondRec &be,
+                           const BondRec &bb, const float (&R)[9], const float (&T)[3], float ck, float sk, int g,
+                           int k, int L, int G, int S, float *out) {
+  unsigned n_test = 0, n_pair = 0;  // not counted: once per ligand
+  for (int r = 0; r < (S + G - 1) / G; ++r) {
+    const int te = min(r * G + g, S - 1);  // groups past S repeat the last step
+    pose_input(w, pose, d, R, T, k, L);
+    float ex, ey, ez;
+    const float4 ev = pose[be.v];
+    bond_axis(pose[be.u], ev, ex, ey, ez);
+    float ce, se;
+    step_cs(p, te, ce, se);
+    Rot re;
+    re.make(ce, se, ex, ey, ez, ev.x, ev.y, ev.z);
     __syncwarp();
-    const BondRec b0 = w.bonds[0];
-    float nx, ny, nz;
-    float4 pv = pose[b0.v];
-    bond_axis(pose[b0.u], pv, nx, ny, nz);
-    if (r < 0) {
-      const float ac = clash_sweep(p, w, pose, d, b0, nx, ny, nz, pv, ck, sk, g, k, L, G, n_test, n_pair);
-      if (g == 0 && k < S) w.memo[k] = ac;
-      __syncwarp();
-      for (int b = memo_bonds(S); b < d.n_rot; ++b) {  // the fixed-geometry pairs of later bonds
-        BondRec bb = w.bonds[b];
-        if (bb.n_cand0 == 0) continue;  // warp-uniform
-        bb.n_cand = bb.n_cand0;
-        float mx, my, mz;
-        const float4 qv = pose[bb.v];
-        bond_axis(pose[bb.u], qv, mx, my, mz);
-        const float a0 = clash_sweep(p, w, pose, d, bb, mx, my, mz, qv, ck, sk, g, k, L, G, n_test, n_pair);
-        if (g == 0 && k < S) w.memo[memo_row0(S) + (b - memo_bonds(S)) * S + k] = a0;
-        __syncwarp();
-      }
-      continue;
-    }
-    const int k0 = min(r * G + g, S - 1);  // groups past S repeat the last step
-    float c0, s0;
-    step_cs(p, k0, c0, s0);
-    Rot rb;
-    rb.make(c0, s0, nx, ny, nz, pv.x, pv.y, pv.z);
-    __syncwarp();
-    for (int i = b0.v + 1 + k; i < b0.end; i += L) {
+    for (int i = be.v + 1 + k; i < be.end; i += L) {
       float4 q = pose[i];
-      rb.apply(q.x, q.y, q.z, q.x, q.y, q.z);
+      re.apply(q.x, q.y, q.z, q.x, q.y, q.z);
       pose[i] = q;
     }
     __syncwarp();
-    const BondRec b1 = w.bonds[1];
-    pv = pose[b1.v];
-    bond_axis(pose[b1.u], pv, nx, ny, nz);
-    const float ac = clash_sweep(p, w, pose, d, b1, nx, ny, nz, pv, ck, sk, g, k, L, G, n_test, n_pair);
-    if (r * G + g < S && k < S) w.memo[S + k0 * S + k] = ac;
+    float mx, my, mz;
+    const float4 qv = pose[bb.v];
+    bond_axis(pose[bb.u], qv, mx, my, mz);
+    const float a1 = clash_sweep(p, w, pose, d, bb, mx, my, mz, qv, ck, sk, g, k, L, G, n_test, n_pair);
+    if (r * G + g < S && k < S) {
+      if (LAST) {
+        uint64_t pol;
+        asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+        asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(out + te * S + k), "f"(a1), "l"(pol) : "memory");
+      } else {
+        out[te * S + k] = a1;
+      }
+    }
     __syncwarp();
   }
+}
+
+// The pairs of bond b >= 2 that bond e1 alone separates, by e1's step.
+__device__ void single_table(const DockParams &p, const WarpSmem &w, float4 *pose, const LigDesc &d, BondRec bb,
+                             const float (&R)[9], const float (&T)[3], float ck, float sk, int g, int k, int L, int G,
+                             int S, float *m1) {
+  bb.cand_off += bb.n_cand0;
+  bb.n_cand = bb.n_cand1;
+  turn_table<true>(p, w, pose, d, w.bonds[bb.e1 & 0xffff], bb, R, T, ck, sk, g, k, L, G, S,
+                   m1 + (bb.e1 >> 16) * S * S);
+}
+
+// memo[k]: the sums of bond 0's sweep; memo[memo_row0(S) + (b - memo_bonds(S))
+// S + k]: of each later bond b, the sums over its first n_cand0 candidates;
+// all on the input conformation.
+__device__ void input_rows(const DockParams &p, const WarpSmem &w, float4 *pose, const LigDesc &d, const float (&R)[9],
+                           const float (&T)[3], float ck, float sk, int g, int k, int L, int G, int S, float *memo) {
+  unsigned n_test = 0, n_pair = 0;
+  pose_input(w, pose, d, R, T, k, L);
+  for (int b = 0; b < d.n_rot; b = b == 0 ? memo_bonds(S) : b + 1) {
+    BondRec bb = w.bonds[b];
+    if (b > 0) {
+      if (bb.n_cand0 == 0) continue;  // warp-uniform
+      bb.n_cand = bb.n_cand0;
+    }
+    float mx, my, mz;
+    const float4 qv = pose[bb.v];
+    bond_axis(pose[bb.u], qv, mx, my, mz);
+    const float a0 = clash_sweep(p, w, pose, d, bb, mx, my, mz, qv, ck, sk, g, k, L, G, n_test, n_pair);
+    if (g == 0 && k < S) memo[(b == 0 ? 0 : memo_row0(S) + (b - memo_bonds(S)) * S) + k] = a0;
+    __syncwarp();
+  }
+}
+
+// All clash tables of the loaded ligand by one warp: input_rows and bond 1's
+// sums after bond 0's step (memo[S + k0 S + k]) into w.memo, the single-
+// separator tables into m1 (if given).  For runs without clash_tables_kernel.
+__device__ __noinline__ void build_memo(const DockParams &p, const WarpSmem &w, float4 *pose, const LigDesc &d,
+                                        float ck, float sk, int g, int k, int L, int G, int S, float *m1) {
+  float R[9], T[3];
+  start_frame(p, 0, R, T);
+  if (m1)
+    for (int b = 2; b < d.n_rot; ++b) {
+      const BondRec bb = w.bonds[b];
+      if (bb.n_cand1 > 0) single_table(p, w, pose, d, bb, R, T, ck, sk, g, k, L, G, S, m1);
+    }
+  input_rows(p, w, pose, d, R, T, ck, sk, g, k, L, G, S, w.memo);
+  if (d.n_rot >= 2 && memo_bonds(S) == 2)
+    turn_table<false>(p, w, pose, d, w.bonds[0], w.bonds[1], R, T, ck, sk, g, k, L, G, S, w.memo + S);
+}
+
+// The clash tables of every row's ligand, once per run: one warp per (row,
+// table).  What a row's work items share is built here once instead of by
+// every item's warp, so items can be small (a batch that leaves few starts
+// per warp) without paying for the tables again, and a ligand's tables are
+// built in parallel.  The same device code builds the tables in the docking
+// kernel when the rows' tables do not fit the plan's budget.
+__global__ void __launch_bounds__(128) clash_tables_kernel(const DockParams p, const int32_t *__restrict__ row_lig,
+                                                           int rows) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const WarpSmem w = warp_smem(smem_raw + (size_t)warp * smem_bytes_per_warp(p.nmax, 0, p.G, 0), p.nmax, p.G);
+  const int tables = 2 + p.m1max, S = p.S, L = p.L, G = p.G;
+  const long long id = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
+  const int row = (int)(id / tables), t = (int)(id % tables);
+  if (row >= rows) return;
+  const int li = row_lig[row];
+  const LigDesc d = p.lig[li];
+  if (d.n_rot == 0 || (t == 1 && (d.n_rot < 2 || memo_bonds(S) < 2))) return;
+  int slot_bond = -1;
+  if (t >= 2) {  // the bond whose single-separator table has slot t - 2
+    bool mine = false;
+    if (lane >= 2 && lane < d.n_rot) {
+      const BondRec b = p.bonds[d.bond_base + lane];
+      mine = b.n_cand1 > 0 && (b.e1 >> 16) == t - 2;
+    }
+    slot_bond = __ffs(__ballot_sync(FULL, mine)) - 1;
+    if (slot_bond < 0) return;
+  }
+  load_coords(p, w, d, lane);
+  const int g = lane / L, k = lane - g * L;
+  float4 *pose = w.pose + (size_t)g * (p.nmax + 1);
+  float ck = 1.f, sk = 0.f;
+  if (k < S) step_cs(p, k, ck, sk);
+  float R[9], T[3];
+  start_frame(p, 0, R, T);
+  float *memo = p.tab + (size_t)row * p.tab_stride, *m1 = memo + memo_floats(S, p.rmax);
+  if (t == 0) input_rows(p, w, pose, d, R, T, ck, sk, g, k, L, G, S, memo);
+  else if (t == 1) turn_table<false>(p, w, pose, d, w.bonds[0], w.bonds[1], R, T, ck, sk, g, k, L, G, S, memo + S);
+  else single_table(p, w, pose, d, w.bonds[slot_bond], R, T, ck, sk, g, k, L, G, S, m1);
 }
 
 // Drops the L2 copies of the whole 128-byte lines inside [lo, hi) without
@@ -340,8 +375,10 @@ __global__ void __launch_bounds__(128, MINB) dock_kernel(const DockParams p) {
   if (k < S) step_cs(p, k, ck, sk);
   const int ts = type_stride(MODE, p.g);
   const float INF = __int_as_float(0x7f800000);
-  float *const m1 = p.memo1 ? p.memo1 + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * p.m1max * S * S
-                            : nullptr;
+  // single-separator tables: the row's (p.tab), or this warp's own scratch
+  float *const m1w = p.memo1 ? p.memo1 + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * p.m1max * S * S
+                             : nullptr;
+  const float *m1 = m1w;
 
   const int n_items = p.n_items_dev ? __ldcg(p.n_items_dev) : p.n_items;
   int cur = -1, n_memo = 0;
@@ -354,20 +391,27 @@ __global__ void __launch_bounds__(128, MINB) dock_kernel(const DockParams p) {
     if (lane == 0) it = atomicAdd(p.queue, 1);
     it = __shfl_sync(FULL, it, 0);
     if (it >= n_items) {
-      if (m1) {  // this warp's clash tables are dead: no write-back
+      if (m1w) {  // this warp's clash tables are dead: no write-back
         __syncwarp();
-        l2_discard(m1, m1 + (size_t)p.m1max * S * S, lane);
+        l2_discard(m1w, m1w + (size_t)p.m1max * S * S, lane);
       }
       break;
     }
     const Item item = p.items[it];
     if (item.ligand != cur) {
       __syncwarp();
-      if (m1 && cur >= 0) l2_discard(m1, m1 + (size_t)p.m1max * S * S, lane);  // the last ligand's tables
+      if (m1w && cur >= 0) l2_discard(m1w, m1w + (size_t)p.m1max * S * S, lane);  // the last ligand's tables
       clash_ref = load_ligand(p, w, item.ligand, d, lane);
       cur = item.ligand;
       n_memo = min(d.n_rot, memo_bonds(S));
-      if (n_memo > 0) build_memo(p, w, pose, d, n_memo, ck, sk, g, k, L, G, S, m1);
+      if (p.tab) {  // clash_tables_kernel's rows
+        const float4 *src = reinterpret_cast<const float4 *>(p.tab + (size_t)item.row * p.tab_stride);
+        const int nf = n_memo > 0 ? memo_floats(S, d.n_rot) / 4 : 0;
+        for (int q = lane; q < nf; q += 32) reinterpret_cast<float4 *>(w.memo)[q] = __ldg(src + q);
+        m1 = p.tab + (size_t)item.row * p.tab_stride + memo_floats(S, p.rmax);
+      } else if (n_memo > 0) {
+        build_memo(p, w, pose, d, ck, sk, g, k, L, G, S, m1w);
+      }
       bound_setup(p, w, d, lane);
     }
     top.clear();
@@ -595,7 +639,7 @@ __global__ void __launch_bounds__(128, MINB) dock_kernel(const DockParams p) {
 
     top.clear();
     const int slot0 = p.lig_slot0[item.row], nit = p.lig_items[item.row];
-    for (int c = 0; c < nit; ++c) {
+    for (int c = 0; c < nit; ++c) {  // each list ascends: past its first loser nothing enters
       const PoseOut *src = p.partial + (size_t)(slot0 + c) * K;
       float pe = INF;
       int ps = EMPTY_SID;
@@ -610,7 +654,7 @@ __global__ void __launch_bounds__(128, MINB) dock_kernel(const DockParams p) {
         const int cs = __shfl_sync(FULL, ps, j);
         const uint32_t c0 = __shfl_sync(FULL, q0, j), c1 = __shfl_sync(FULL, q1, j),
                        c2 = __shfl_sync(FULL, q2, j), c3 = __shfl_sync(FULL, q3, j);
-        if (cs != EMPTY_SID) top.insert(ce, cs, c0, c1, c2, c3, K, lane);
+        if (cs == EMPTY_SID || !top.insert(ce, cs, c0, c1, c2, c3, K, lane)) break;
       }
     }
     __syncwarp();  // the ligand's partial lists are merged and dead: no write-back
@@ -765,6 +809,19 @@ cudaError_t launch_dock(int mode, int reg_cap, const DockParams &p, int grid, in
   void *args[] = {(void *)&p};
   return cudaLaunchKernel(dock_fn(mode, reg_cap), dim3(grid), dim3(block), args, smem, s);
 }
+
+cudaError_t launch_clash_tables(const DockParams &p, const int32_t *row_lig, int rows, cudaStream_t s) {
+  if (rows <= 0 || !p.tab || p.rmax == 0) return cudaSuccess;
+  const int warps = 4;
+  const size_t smem = (size_t)warps * smem_bytes_per_warp(p.nmax, 0, p.G, 0);
+  cudaError_t e = cudaFuncSetAttribute(clash_tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e != cudaSuccess) return e;
+  const long long n = (long long)rows * (2 + p.m1max);
+  clash_tables_kernel<<<(unsigned)((n + warps - 1) / warps), 32 * warps, smem, s>>>(p, row_lig, rows);
+  return cudaGetLastError();
+}
+
+size_t dock_tab_stride(int S, int rmax, int m1max) { return (size_t)memo_floats(S, rmax) + ((size_t)m1max * S * S + 3) / 4 * 4; }
 
 size_t dock_kernel_local_bytes(int mode, int reg_cap) {
   cudaFuncAttributes a;

@@ -198,12 +198,13 @@ struct TopK {
   __device__ __forceinline__ void clear() {
     e = __int_as_float(0x7f800000); s = EMPTY_SID; t0 = t1 = t2 = t3 = 0;
   }
-  // Insert a warp-uniform candidate (all lanes pass the same values).
-  __device__ __forceinline__ void insert(float ce, int cs, uint32_t c0, uint32_t c1, uint32_t c2,
+  // Insert a warp-uniform candidate (all lanes pass the same values); false
+  // when it is not among the K smallest.
+  __device__ __forceinline__ bool insert(float ce, int cs, uint32_t c0, uint32_t c1, uint32_t c2,
                                          uint32_t c3, int K, int lane) {
     const float ke = __shfl_sync(FULL, e, K - 1);
     const int ks = __shfl_sync(FULL, s, K - 1);
-    if (!pose_less(ce, cs, ke, ks)) return;  // warp-uniform
+    if (!pose_less(ce, cs, ke, ks)) return false;  // warp-uniform
     const bool before = lane < K && pose_less(e, s, ce, cs);
     const int pos = __popc(__ballot_sync(FULL, before));
     const float ue = __shfl_up_sync(FULL, e, 1);
@@ -212,6 +213,7 @@ struct TopK {
                    u2 = __shfl_up_sync(FULL, t2, 1), u3 = __shfl_up_sync(FULL, t3, 1);
     if (lane > pos && lane < K) { e = ue; s = us; t0 = u0; t1 = u1; t2 = u2; t3 = u3; }
     if (lane == pos) { e = ce; s = cs; t0 = c0; t1 = c1; t2 = c2; t3 = c3; }
+    return true;
   }
 };
 
@@ -280,13 +282,9 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// Load ligand `li` into the warp's slot: reference coordinates centred on
-// their centroid, bond table, clash masks.  Returns the clash sum (without
-// the weight) of the input conformation, which every pose shares up to the
-// torsion-dependent part.
-__device__ inline float load_ligand(const DockParams &p, const WarpSmem &w, int li, LigDesc &d,
-                             int lane) {
-  d = p.lig[li];
+// Reference coordinates of ligand d centred on their centroid, and its bond
+// table, into the warp's slot.
+__device__ __forceinline__ void load_coords(const DockParams &p, const WarpSmem &w, const LigDesc &d, int lane) {
   float sx = 0.f, sy = 0.f, sz = 0.f;
   for (int i = lane; i < d.n_atoms; i += 32) {
     const float4 a = __ldg(p.atoms + d.atom_base + i);
@@ -304,6 +302,15 @@ __device__ inline float load_ligand(const DockParams &p, const WarpSmem &w, int 
   }
   for (int b = lane; b < d.n_rot; b += 32) w.bonds[b] = p.bonds[d.bond_base + b];
   __syncwarp();
+}
+
+// Load ligand `li` into the warp's slot: load_coords and the clash sum
+// (without the weight) of the input conformation, which every pose shares up
+// to the torsion-dependent part.
+__device__ inline float load_ligand(const DockParams &p, const WarpSmem &w, int li, LigDesc &d,
+                             int lane) {
+  d = p.lig[li];
+  load_coords(p, w, d, lane);
   float cl = 0.f;
   for (int i = lane; i < d.n_atoms; i += 32) {
     const float4 xi = w.ref[i];

@@ -207,7 +207,12 @@ struct DockParams {
   int rmax;                // rotatable bonds of the batch's largest ligand (memo rows)
   float *memo1;            // [resident warps][m1max][S][S] clash sums of the pairs one earlier bond
                            // separates, by that bond's step (null: those pairs are swept live)
-  int m1max;               // tables per warp (bonds with such pairs, largest ligand)
+  int m1max;               // such tables per ligand (bonds with such pairs, largest ligand)
+  // optional [rows][tab_stride]: every row's clash tables, built once per run
+  // by clash_tables_kernel (memo_floats(S, rmax) floats of the shared-memory
+  // memo, then m1max tables of S x S); null: built by the warps (memo1)
+  float *tab;
+  int tab_stride;
   // optional [n_anchor]: the order a work item visits each orientation's
   // anchors in (consecutive entries are spatially close anchors, so the
   // start groups of a warp sweep similar poses); null: anchor order (plans
@@ -279,6 +284,10 @@ size_t dock_smem_per_warp(int nmax, int S, int G, int rmax);
 int dock_memo1_tables(const LigDesc &d, const BondRec *bonds, int S);
 cudaError_t launch_dock(int mode, int reg_cap, const DockParams &p, int grid, int block, size_t smem,
                         cudaStream_t s);
+// Clash tables of the rows' ligands into p.tab (no-op without it), before the
+// docking kernel on the same stream; floats per row for S steps.
+cudaError_t launch_clash_tables(const DockParams &p, const int32_t *row_lig, int rows, cudaStream_t s);
+size_t dock_tab_stride(int S, int rmax, int m1max);
 cudaError_t launch_start_frames(const double *quat_unused, const float *quat_f32_dev,
                                 int n_orient, const float *anchors_dev, int n_anchor,
                                 const double origin[3], double h, float *rot_out,
