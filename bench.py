@@ -82,16 +82,17 @@ def algorithmic_flops(work, S, n_starts, total_atoms):
 # DRAM bytes (read + write) of one full-size launch of the chosen-form
 # kernel, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum),
 # valid only for the kernel revision it was captured on (sha1 prefix of
-# dock.cu + dock_device.cuh); any other revision reports null until it is
+# the docking kernel's files); any other revision reports null until it is
 # captured again.
 TRAFFIC_BYTES = {("cf4358d5f3d0", "batched", 10000): 104403456 + 24783104}
 
 
 def kernel_source_sha():
-    """sha1 prefix of the docking kernel's sources (dock.cu + dock_device.cuh)."""
+    """sha1 prefix of the docking kernel's sources (dock.cu, dock_kernel.cuh, dock_l16.cu,
+    dock_device.cuh)."""
     import hashlib
     h = hashlib.sha1()
-    for f in ("dock.cu", "dock_device.cuh"):
+    for f in ("dock.cu", "dock_kernel.cuh", "dock_l16.cu", "dock_device.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2304_09953_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:12]
 

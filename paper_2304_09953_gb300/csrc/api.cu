@@ -1129,7 +1129,7 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
     set_error("plan_create: %zu B shared memory per CTA exceeds 227 KB; use fewer warps", pl->smem);
     return LIGATE_ERR_UNSUPPORTED;
   }
-  const int occ = dock_kernel_max_ctas_per_sm(mode, t.reg_cap, pl->block, pl->smem);
+  const int occ = dock_kernel_max_ctas_per_sm(mode, t.reg_cap, p.L, pl->block, pl->smem);
   if (occ < 1) {
     free_plan(pl);
     set_error("plan_create: kernel cannot be resident with %d threads, %zu B shared memory",
@@ -2273,7 +2273,7 @@ extern "C" ligate_status ligate_model_tile(const ligate_pocket *P, const ligate_
   int best_res = 0;
   for (int cap = 1; cap <= 3; ++cap) {
     if (mode == MODE_F32_PLAIN && cap != 3) continue;
-    if (cap < 3 && dock_kernel_local_bytes(mode, cap) > 0) continue;  // spills: registers too tight
+    if (cap < 3 && dock_kernel_local_bytes(mode, cap, pow2ceil(S)) > 0) continue;  // spills: registers too tight
     const int minb = cap == 1 ? 6 : cap == 2 ? 5 : 4;  // CTAs of 128 threads the register cap allows
     for (int warps : {2, 4}) {
       const size_t cta_smem = per_warp * warps + 1024;  // + the per-CTA reserve

@@ -79,63 +79,119 @@ __device__ __forceinline__ float grid_eval(const void *__restrict__ maps, int to
 }
 
 
-// Two atoms at once with packed FP32 (FFMA2 / FADD2: per component the same
-// rounding as fmaf / the scalar add, so each value equals grid_eval's).
+// The sweep's interpolation: grid_eval's values with fewer instructions on
+// the half-rate ALU pipe (compares, minima, selects, shifts), which the
+// gathers' address arithmetic otherwise fills.
+//
+// The cell index is formed on the raw bit patterns of 2^23 + floor(u)
+// (modulo 2^32), and the constants' share is subtracted once per run, in the
+// offset each atom carries (cell_bias), not per evaluation.
+constexpr float CELL_M = 8388608.f;  // 2^23
+constexpr unsigned CELL_MB = 0x4B000000u;
+
+// Node or cell strides of a map: index (iz * A + iy) * B + ix.
 template <int MODE>
-__device__ __forceinline__ void load_corners(const void *__restrict__ maps, int toff, int ix, int iy, int iz,
-                                             const GridConst &g, float (&v)[8]) {
+__device__ __forceinline__ void map_strides(const GridConst &g, unsigned &A, unsigned &B) {
+  A = MODE == MODE_F32_PLAIN ? g.ny : g.ny - 1;
+  B = MODE == MODE_F32_PLAIN ? g.nx : g.nx - 1;
+}
+template <int MODE>
+__device__ __forceinline__ unsigned cell_bias(const GridConst &g) {
+  unsigned A, B;
+  map_strides<MODE>(g, A, B);
+  return 0u - CELL_MB * (A * B + B + 1u);
+}
+
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+// The 8 corners of the cell at index `cell` (plain: its first node).
+template <int MODE>
+__device__ __forceinline__ void load_corners(const void *__restrict__ maps, unsigned cell, const GridConst &g,
+                                             float (&v)[8]) {
   if (MODE == MODE_F32_PLAIN) {
-    const float *m = (const float *)maps + toff + (iz * g.ny + iy) * g.nx + ix;
+    const float *m = (const float *)maps + cell;
     const int sy = g.nx, sz = g.nx * g.ny;
     v[0] = __ldg(m); v[1] = __ldg(m + 1); v[2] = __ldg(m + sy); v[3] = __ldg(m + sy + 1);
     v[4] = __ldg(m + sz); v[5] = __ldg(m + sz + 1); v[6] = __ldg(m + sz + sy); v[7] = __ldg(m + sz + sy + 1);
+  } else if (MODE == MODE_F32_CORNER) {
+    const float4 *m = (const float4 *)maps + 2 * (size_t)cell;
+    const float4 a = __ldg(m), b = __ldg(m + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
   } else {
-    const int cell = toff + (iz * (g.ny - 1) + iy) * (g.nx - 1) + ix;
-    if (MODE == MODE_F32_CORNER) {
-      const float4 *m = (const float4 *)maps + 2 * cell;
-      const float4 a = __ldg(m), b = __ldg(m + 1);
-      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    const uint4 w = __ldg((const uint4 *)maps + cell);
+    if (MODE == MODE_BF16_CORNER) {
+      v[0] = __uint_as_float(w.x << 16); v[1] = __uint_as_float(w.x & 0xffff0000u);
+      v[2] = __uint_as_float(w.y << 16); v[3] = __uint_as_float(w.y & 0xffff0000u);
+      v[4] = __uint_as_float(w.z << 16); v[5] = __uint_as_float(w.z & 0xffff0000u);
+      v[6] = __uint_as_float(w.w << 16); v[7] = __uint_as_float(w.w & 0xffff0000u);
     } else {
-      const uint4 w = __ldg((const uint4 *)maps + cell);
-      if (MODE == MODE_BF16_CORNER) {
-        v[0] = __uint_as_float(w.x << 16); v[1] = __uint_as_float(w.x & 0xffff0000u);
-        v[2] = __uint_as_float(w.y << 16); v[3] = __uint_as_float(w.y & 0xffff0000u);
-        v[4] = __uint_as_float(w.z << 16); v[5] = __uint_as_float(w.z & 0xffff0000u);
-        v[6] = __uint_as_float(w.w << 16); v[7] = __uint_as_float(w.w & 0xffff0000u);
-      } else {
-        float2 f;
-        f = __half22float2(*reinterpret_cast<const __half2 *>(&w.x)); v[0] = f.x; v[1] = f.y;
-        f = __half22float2(*reinterpret_cast<const __half2 *>(&w.y)); v[2] = f.x; v[3] = f.y;
-        f = __half22float2(*reinterpret_cast<const __half2 *>(&w.z)); v[4] = f.x; v[5] = f.y;
-        f = __half22float2(*reinterpret_cast<const __half2 *>(&w.w)); v[6] = f.x; v[7] = f.y;
-      }
+      float2 f;
+      f = __half22float2(*reinterpret_cast<const __half2 *>(&w.x)); v[0] = f.x; v[1] = f.y;
+      f = __half22float2(*reinterpret_cast<const __half2 *>(&w.y)); v[2] = f.x; v[3] = f.y;
+      f = __half22float2(*reinterpret_cast<const __half2 *>(&w.z)); v[4] = f.x; v[5] = f.y;
+      f = __half22float2(*reinterpret_cast<const __half2 *>(&w.w)); v[6] = f.x; v[7] = f.y;
     }
   }
 }
 
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-
+// One atom; off = map offset + cell_bias.  Outside [0, n - 1] on any axis
+// (NaN coordinates included) it scores the penalty.
 template <int MODE>
-__device__ __forceinline__ float2 grid_eval2(const void *__restrict__ maps, int toffa, float ax, float ay, float az,
-                                             int toffb, float bx, float by, float bz, const GridConst &g) {
-  const bool ina = (ax >= 0.f) & (ax <= g.fx1) & (ay >= 0.f) & (ay <= g.fy1) & (az >= 0.f) & (az <= g.fz1);
-  const bool inb = (bx >= 0.f) & (bx <= g.fx1) & (by >= 0.f) & (by <= g.fy1) & (bz >= 0.f) & (bz <= g.fz1);
-  const float M23 = 8388608.f;
-  const float txa = fminf(__fadd_rd(ax, M23), g.cx), tya = fminf(__fadd_rd(ay, M23), g.cy),
-              tza = fminf(__fadd_rd(az, M23), g.cz);
-  const float txb = fminf(__fadd_rd(bx, M23), g.cx), tyb = fminf(__fadd_rd(by, M23), g.cy),
-              tzb = fminf(__fadd_rd(bz, M23), g.cz);
-  const int ixa = ina ? __float_as_int(txa) - 0x4B000000 : 0, iya = ina ? __float_as_int(tya) - 0x4B000000 : 0,
-            iza = ina ? __float_as_int(tza) - 0x4B000000 : 0;
-  const int ixb = inb ? __float_as_int(txb) - 0x4B000000 : 0, iyb = inb ? __float_as_int(tyb) - 0x4B000000 : 0,
-            izb = inb ? __float_as_int(tzb) - 0x4B000000 : 0;
-  const float2 m23 = make_float2(M23, M23);
-  const float2 fx = sub2(make_float2(ax, bx), sub2(make_float2(txa, txb), m23));
-  const float2 fy = sub2(make_float2(ay, by), sub2(make_float2(tya, tyb), m23));
-  const float2 fz = sub2(make_float2(az, bz), sub2(make_float2(tza, tzb), m23));
+__device__ __forceinline__ float sweep_eval(const void *__restrict__ maps, unsigned off, float ux, float uy, float uz,
+                                            const GridConst &g) {
+  unsigned A, B;
+  map_strides<MODE>(g, A, B);
+  const bool in = (min3_nan(ux, uy, uz) >= 0.f) & (max3_nan(ux - g.fx1, uy - g.fy1, uz - g.fz1) <= 0.f);
+  const float tx = fminf(__fadd_rd(ux, CELL_M), g.cx), ty = fminf(__fadd_rd(uy, CELL_M), g.cy),
+              tz = fminf(__fadd_rd(uz, CELL_M), g.cz);  // the upper face belongs to the last cell
+  const float fx = ux - (tx - CELL_M), fy = uy - (ty - CELL_M), fz = uz - (tz - CELL_M);
+  unsigned cell = off + (__float_as_uint(tz) * A + __float_as_uint(ty)) * B + __float_as_uint(tx);
+  cell = in ? cell : 0u;
+  float v[8];
+  load_corners<MODE>(maps, cell, g, v);
+  const float y0z0 = fmaf(fx, v[1] - v[0], v[0]);
+  const float y1z0 = fmaf(fx, v[3] - v[2], v[2]);
+  const float y0z1 = fmaf(fx, v[5] - v[4], v[4]);
+  const float y1z1 = fmaf(fx, v[7] - v[6], v[6]);
+  const float z0 = fmaf(fy, y1z0 - y0z0, y0z0);
+  const float z1 = fmaf(fy, y1z1 - y0z1, y0z1);
+  const float r = fmaf(fz, z1 - z0, z0);
+  return in ? r : g.penalty;
+}
+
+// Two atoms at once with packed FP32 (FFMA2 / FADD2: per component the same
+// rounding as fmaf / the scalar add, so each value equals sweep_eval's).
+template <int MODE>
+__device__ __forceinline__ float2 sweep_eval2(const void *__restrict__ maps, unsigned offa, unsigned offb, float2 ux,
+                                              float2 uy, float2 uz, const GridConst &g) {
+  unsigned A, B;
+  map_strides<MODE>(g, A, B);
+  const float2 dx = __fadd2_rn(ux, make_float2(-g.fx1, -g.fx1)), dy = __fadd2_rn(uy, make_float2(-g.fy1, -g.fy1)),
+               dz = __fadd2_rn(uz, make_float2(-g.fz1, -g.fz1));
+  const bool ina = (min3_nan(ux.x, uy.x, uz.x) >= 0.f) & (max3_nan(dx.x, dy.x, dz.x) <= 0.f);
+  const bool inb = (min3_nan(ux.y, uy.y, uz.y) >= 0.f) & (max3_nan(dx.y, dy.y, dz.y) <= 0.f);
+  const float2 tx = make_float2(fminf(__fadd_rd(ux.x, CELL_M), g.cx), fminf(__fadd_rd(ux.y, CELL_M), g.cx));
+  const float2 ty = make_float2(fminf(__fadd_rd(uy.x, CELL_M), g.cy), fminf(__fadd_rd(uy.y, CELL_M), g.cy));
+  const float2 tz = make_float2(fminf(__fadd_rd(uz.x, CELL_M), g.cz), fminf(__fadd_rd(uz.y, CELL_M), g.cz));
+  const float2 mm = make_float2(-CELL_M, -CELL_M);
+  const float2 fx = sub2(ux, __fadd2_rn(tx, mm)), fy = sub2(uy, __fadd2_rn(ty, mm)), fz = sub2(uz, __fadd2_rn(tz, mm));
+  unsigned ca = offa + (__float_as_uint(tz.x) * A + __float_as_uint(ty.x)) * B + __float_as_uint(tx.x);
+  unsigned cb = offb + (__float_as_uint(tz.y) * A + __float_as_uint(ty.y)) * B + __float_as_uint(tx.y);
+  ca = ina ? ca : 0u;
+  cb = inb ? cb : 0u;
   float va[8], vb[8];
-  load_corners<MODE>(maps, ina ? toffa : 0, ixa, iya, iza, g, va);
-  load_corners<MODE>(maps, inb ? toffb : 0, ixb, iyb, izb, g, vb);
+  load_corners<MODE>(maps, ca, g, va);
+  load_corners<MODE>(maps, cb, g, vb);
   const float2 v0 = make_float2(va[0], vb[0]), v1 = make_float2(va[1], vb[1]), v2 = make_float2(va[2], vb[2]),
                v3 = make_float2(va[3], vb[3]), v4 = make_float2(va[4], vb[4]), v5 = make_float2(va[5], vb[5]),
                v6 = make_float2(va[6], vb[6]), v7 = make_float2(va[7], vb[7]);
@@ -190,30 +246,29 @@ __device__ __forceinline__ bool pose_less(float e1, int s1, float e2, int s2) {
   return e1 < e2 || (e1 == e2 && s1 < s2);
 }
 
-// Warp-distributed sorted top-K list: lane j < K holds entry j.
-struct TopK {
+// Warp-distributed sorted top-K list: lane j < K holds entry j's energy, start
+// and the slot its torsion steps are kept in (in memory: an entry's four step
+// words are written once and stay out of the registers).
+struct TopSlots {
   float e;
-  int s;
-  uint32_t t0, t1, t2, t3;
-  __device__ __forceinline__ void clear() {
-    e = __int_as_float(0x7f800000); s = EMPTY_SID; t0 = t1 = t2 = t3 = 0;
+  int s, at;
+  __device__ __forceinline__ void clear(int lane) {
+    e = __int_as_float(0x7f800000); s = EMPTY_SID; at = lane;
   }
-  // Insert a warp-uniform candidate (all lanes pass the same values); false
-  // when it is not among the K smallest.
-  __device__ __forceinline__ bool insert(float ce, int cs, uint32_t c0, uint32_t c1, uint32_t c2,
-                                         uint32_t c3, int K, int lane) {
+  // Insert a warp-uniform candidate: the slot for its steps (the evicted
+  // entry's), or -1 when it is not among the K smallest.
+  __device__ __forceinline__ int insert(float ce, int cs, int K, int lane) {
     const float ke = __shfl_sync(FULL, e, K - 1);
     const int ks = __shfl_sync(FULL, s, K - 1);
-    if (!pose_less(ce, cs, ke, ks)) return false;  // warp-uniform
+    if (!pose_less(ce, cs, ke, ks)) return -1;  // warp-uniform
+    const int ka = __shfl_sync(FULL, at, K - 1);
     const bool before = lane < K && pose_less(e, s, ce, cs);
     const int pos = __popc(__ballot_sync(FULL, before));
     const float ue = __shfl_up_sync(FULL, e, 1);
-    const int us = __shfl_up_sync(FULL, s, 1);
-    const uint32_t u0 = __shfl_up_sync(FULL, t0, 1), u1 = __shfl_up_sync(FULL, t1, 1),
-                   u2 = __shfl_up_sync(FULL, t2, 1), u3 = __shfl_up_sync(FULL, t3, 1);
-    if (lane > pos && lane < K) { e = ue; s = us; t0 = u0; t1 = u1; t2 = u2; t3 = u3; }
-    if (lane == pos) { e = ce; s = cs; t0 = c0; t1 = c1; t2 = c2; t3 = c3; }
-    return true;
+    const int us = __shfl_up_sync(FULL, s, 1), ua = __shfl_up_sync(FULL, at, 1);
+    if (lane > pos && lane < K) { e = ue; s = us; at = ua; }
+    if (lane == pos) { e = ce; s = cs; at = ka; }
+    return ka;
   }
 };
 
@@ -224,18 +279,24 @@ struct WarpSmem {
   float4 *list;    // [PAIR_WARP] clash pairs that survive the circle bound of a bond
   float2 *cab;     // [G][nmax] (axial coordinate, radial distance) about the bond axis
   BondRec *bonds;  // [LIGATE_MAX_ROT]
-  float *lbc;      // [LBC_FLOATS] per sweep stage b: sum of the map minima of the atoms bonds >= b move
-  uint8_t *lastb;  // [nmax] 1 + the last bond that moves each atom (0: no bond moves it)
+  // the docking kernel's (S > 0) only:
+  float *lbc;      // [LIGATE_MAX_ROT + 1] per sweep stage b: sum of the map minima of the atoms bonds >= b move
+  uint32_t *fixm;  // [4] bit i: no bond moves atom i
+  unsigned *swept; // [LIGATE_MAX_ROT + 2] starts of the item pruned after b bonds; [MAX_ROT + 1]: swept to the end
+  uint8_t *steps;  // [G][LIGATE_MAX_ROT] chosen step of each bond of the start being swept
+  uint32_t *lastm; // [LIGATE_MAX_ROT][nmax / 32] per bond: bit q: it moves atom v + 1 + q for the last time
   float *memo;     // [memo_floats(S, rmax)] clash sums that every start shares
 };
 
-// floats of WarpSmem::lbc (LIGATE_MAX_ROT + 1 stages, padded to 16 bytes)
-constexpr int LBC_FLOATS = (LIGATE_MAX_ROT + 1 + 3) / 4 * 4;
+// words of lbc, fixm and swept together (padded to 16 bytes)
+constexpr int SWEEP_WORDS = (2 * LIGATE_MAX_ROT + 1 + 2 + 4 + 3) / 4 * 4;
 
 // Surviving clash pairs buffered per warp before they are evaluated for
-// every torsion step: 192 entries, 192 / G = 6 L per start group (the
-// buffer is flushed whenever a group may overflow).
-constexpr int PAIR_WARP = 192;
+// every torsion step: 188 entries, nearly 6 L per start group (the buffer is
+// flushed whenever a group may overflow).  With 188 entries five 4-warp CTAs
+// of a 64-atom, 12-bond batch stay within the 196 KB shared-memory
+// configuration, which leaves the map gathers 60 KB of L1.
+constexpr int PAIR_WARP = 188;
 
 // The clash term of a bond's sweep depends only on the ligand's internal
 // conformation, which before bond b is set by the steps chosen at bonds
@@ -258,8 +319,8 @@ __host__ __device__ inline int memo_floats(int S, int rmax) {
 // keep a histogram there, 0 for those that need neither).
 __host__ __device__ inline size_t smem_bytes_per_warp(int nmax, int S, int G, int rmax, int list = PAIR_WARP) {
   return (size_t)nmax * 16 + (size_t)G * (nmax + 1) * 16 + (size_t)list * 16 +
-         (size_t)G * nmax * 8 + sizeof(BondRec) * LIGATE_MAX_ROT + (size_t)LBC_FLOATS * 4 +
-         (size_t)((nmax + 15) & ~15) + (size_t)memo_floats(S, rmax) * 4;
+         (size_t)G * nmax * 8 + sizeof(BondRec) * LIGATE_MAX_ROT +
+         (S > 0 ? (size_t)(SWEEP_WORDS + LIGATE_MAX_ROT * (nmax / 32)) * 4 + (size_t)G * LIGATE_MAX_ROT : 0) + (size_t)memo_floats(S, rmax) * 4;
 }
 
 
@@ -271,8 +332,11 @@ __device__ __forceinline__ WarpSmem warp_smem(unsigned char *base, int nmax, int
   w.cab = reinterpret_cast<float2 *>(w.list + list);
   w.bonds = reinterpret_cast<BondRec *>(w.cab + (size_t)G * nmax);
   w.lbc = reinterpret_cast<float *>(w.bonds + LIGATE_MAX_ROT);
-  w.lastb = reinterpret_cast<uint8_t *>(w.lbc + LBC_FLOATS);
-  w.memo = reinterpret_cast<float *>(w.lastb + ((nmax + 15) & ~15));
+  w.fixm = reinterpret_cast<uint32_t *>(w.lbc + LIGATE_MAX_ROT + 1);
+  w.swept = w.fixm + 4;
+  w.steps = reinterpret_cast<uint8_t *>(w.lbc + SWEEP_WORDS);
+  w.lastm = reinterpret_cast<uint32_t *>(w.steps + G * LIGATE_MAX_ROT);
+  w.memo = reinterpret_cast<float *>(w.lastm + LIGATE_MAX_ROT * (nmax / 32));
   return w;
 }
 

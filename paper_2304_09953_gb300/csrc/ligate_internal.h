@@ -299,9 +299,11 @@ cudaError_t launch_score_poses(int mode, const DockParams &p, int n_poses, const
 // atoms in input order (order: the batch's DFS-to-input map).
 cudaError_t launch_pose_coords(const DockParams &p, const uint8_t *order, int n_poses, const int32_t *lig_idx,
                                const int32_t *start_id, const uint8_t *tors, float *out, cudaStream_t s);
-int dock_kernel_max_ctas_per_sm(int mode, int reg_cap, int block, size_t smem);
+int dock_kernel_max_ctas_per_sm(int mode, int reg_cap, int L, int block, size_t smem);
+// Kernel instance for 16 lanes per start (dock_l16.cu); minb 4 or 5.
+const void *dock_fn_l16(int mode, int minb);
 // Local (spill) memory per thread of a kernel instance, in bytes.
-size_t dock_kernel_local_bytes(int mode, int reg_cap);
+size_t dock_kernel_local_bytes(int mode, int reg_cap, int L);
 
 // Pocket kernels (pocket.cu).
 cudaError_t launch_corner_pack(const float *plain, int n_types, int nx, int ny, int nz,

@@ -227,7 +227,7 @@ extern "C" ligate_status ligate_dock_noalloc(const ligate_pocket *P, const ligat
   const size_t per_warp = dock_smem_per_warp(p.nmax, p.S, G, p.rmax);
   const int warps = (int)std::min<size_t>(4, std::max<size_t>(1, (size_t)(227 * 1024) / per_warp));
   const size_t smem = per_warp * warps;
-  const int occ = dock_kernel_max_ctas_per_sm(mode, 0, 32 * warps, smem);
+  const int occ = dock_kernel_max_ctas_per_sm(mode, 0, L, 32 * warps, smem);
   if (occ < 1) { set_error("dock_noalloc: kernel cannot be resident"); return LIGATE_ERR_UNSUPPORTED; }
   int sms = 0;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)

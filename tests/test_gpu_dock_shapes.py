@@ -1,0 +1,51 @@
+"""The docking kernel's instances and work-item shapes give the same bits:
+16-lane instances against the generic ones, small items against large ones,
+a plain-layout plan (which searches the pocket's FP32 corner copy) against
+one whose pocket has no copy, at torsion steps around the group sizes and
+list lengths from one to the limit; and the result is the oracle's."""
+import numpy as np
+import pytest
+
+from paper_2304_09953_gb300 import docking as D
+from paper_2304_09953_gb300 import native as N
+from paper_2304_09953_gb300.workload import Sampling
+from tests.parity import Stats, compare_ligand
+
+pytestmark = pytest.mark.gpu
+
+
+def tile(chunk=0, reg_cap=0, warps=0):
+    t = N.ligate_tile()
+    t.reg_cap, t.warps_per_cta = reg_cap, warps
+    for b in range(N.LIGATE_N_BUCKETS):
+        t.starts_per_item[b] = chunk
+    return t
+
+
+@pytest.mark.parametrize("S,K,orient,anchor", [(1, 1, 3, 5), (7, 4, 5, 7), (8, 32, 8, 8), (9, 5, 6, 11), (16, 16, 16, 8),
+                                               (16, 1, 1, 1), (17, 7, 4, 9), (32, 32, 9, 7)])
+def test_shapes_agree_and_match_the_oracle(batched_small, S, K, orient, anchor):
+    w = batched_small
+    idx = [i for i in range(w.ligands.n) if w.ligands.n_rot[i] in (0, 1, 2, 5, 12)][:10] + [1, 2, 3]
+    ligs = w.ligands.subset(idx)
+    samp = Sampling(w.sampling.quats[:orient], anchor, S, K)
+    full, plain = D.PocketHandle(w.pocket), D.PocketHandle(w.pocket, mask=0)
+    bh = D.BatchHandle(ligs)
+    try:
+        ref = D.Plan(full, bh, samp, mode="fp32").result()
+        for pocket, mode, t in ((full, "fp32", tile(chunk=8)), (full, "fp32", tile(chunk=4096, warps=1)),
+                                (full, "fp32", tile(reg_cap=1)), (full, "fp32c", tile(reg_cap=3)),
+                                (plain, "fp32", None), (plain, "fp32", tile(chunk=64, reg_cap=2))):
+            assert np.array_equal(D.Plan(pocket, bh, samp, mode=mode, tile=t).result(), ref)
+        bf = D.Plan(full, bh, samp, mode="bf16").result()
+        for t in (tile(chunk=8), tile(reg_cap=1), tile(reg_cap=3, warps=2)):
+            assert np.array_equal(D.Plan(full, bh, samp, mode="bf16", tile=t).result(), bf)
+    finally:
+        bh.close()
+        full.close()
+        plain.close()
+    st = Stats()
+    for r in range(0, len(idx), 4):
+        if K <= samp.n_starts:
+            compare_ligand(ligs.ligand(r), w.pocket, samp, ref[r], K=K, stats=st)
+    print(st.line())
