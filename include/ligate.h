@@ -577,7 +577,9 @@ ligate_status ligate_autotune(const ligate_pocket *pocket, const ligate_batch *b
  * 128-register instances: its eight scalar gathers per interpolation need
  * registers for loads in flight).  Chunk of size bucket b (the work model, also used by
  * every plan for zero chunk fields): starts_per_item[b] = W / (8 P c_b)
- * clamped to [128, 2048] and rounded down to the start group, with W the
+ * clamped to [lo, 2048] and rounded down to the start group, with lo = 32 (8
+ * to 32 for a run with fewer than 32 starts per resident warp; at least 2
+ * top_k), W the
  * run's total work (sum over ligands of starts x per-start cost atoms +
  * 0.35 clash pairs + 40), P the resident warps of the whole GPU and c_b the
  * bucket's mean per-start cost: the largest item stays under an eighth of a

@@ -1006,7 +1006,7 @@ static void free_plan(ligate_plan *pl) {
   cudaFree(pl->rot); cudaFree(pl->anc); cudaFree(pl->quat); cudaFree(pl->visit);
   cudaFree(pl->q_scores); cudaFree(pl->q_keys); cudaFree(pl->q_idx);
   cudaFree(pl->items); cudaFree(pl->lig_items); cudaFree(pl->lig_slot0);
-  cudaFree(pl->counters); cudaFree(pl->partial); cudaFree(pl->out); cudaFree(pl->stats);
+  cudaFree(pl->partial); cudaFree(pl->out); cudaFree(pl->stats);  // counters: inside stats
   cudaFree(pl->row_lig);
   delete pl;
 }
@@ -1019,15 +1019,25 @@ static void default_tile(ligate_tile *t) {
 }
 
 // Work model of the launch (paper Sec. 3.3: a batch shape per ligand size):
-// chunk of size bucket b = W / (8 P c_b) starts, clamped to [128, 2048] and
+// chunk of size bucket b = W / (8 P c_b) starts, clamped to [lo, 2048] and
 // rounded down to the start group, with W the run's total work (starts x
 // per-start cost atoms + 0.35 clash pairs + 40, the queue's own estimate),
 // P the warps resident on the whole GPU and c_b the bucket's mean per-start
 // cost: the largest item stays under an eighth of a warp's share (tail
-// balance) while still amortising the load of a ligand and its clash memo.
+// balance).  lo = 32 starts, or the starts per resident warp of a batch too
+// small to give every warp 32 (at least 8), but no fewer than 2 K: an item
+// pays for loading its ligand, and has no K-th best of its own to stop starts
+// with before its K-th start (measured, lo = 128, 64, 32, 16, 8: one 24-atom
+// ligand with 512 starts and K = 4 372, 213, 135, 99 and 88 us; 301 ligands
+// with 1,717 starts and K = 5 4.9, 3.44, 3.19, 3.49 and 3.62 ms; 8 P in the
+// model against 12 P and 16 P: 1,000 ligands 24.1, 24.5, 25.1 ms).
 // Buckets without ligands get 512.  Ligands: sel[0..n) or all of B.
+static double least_chunk(double starts, double P_warps, int K) {
+  return std::max(2.0 * K, std::min(32.0, std::max(8.0, starts / std::max(P_warps, 1.0))));
+}
+
 static void model_chunks(const BatchDev &B, const int32_t *sel, int n, int S, int n_starts, double P_warps,
-                         int G, int *chunks) {
+                         int G, int K, int *chunks) {
   double W = 0.0, cb[LIGATE_N_BUCKETS] = {0}, nb[LIGATE_N_BUCKETS] = {0};
   for (int r = 0; r < n; ++r) {
     const int i = sel ? sel[r] : r;
@@ -1042,7 +1052,7 @@ static void model_chunks(const BatchDev &B, const int32_t *sel, int n, int S, in
   for (int b = 0; b < LIGATE_N_BUCKETS; ++b) {
     double chunk = 512.0;
     if (nb[b] > 0) chunk = W / (8.0 * std::max(P_warps, 1.0) * (cb[b] / nb[b]));
-    chunk = std::min(2048.0, std::max(128.0, chunk));
+    chunk = std::min(2048.0, std::max(least_chunk((double)n * n_starts, P_warps, K), chunk));
     chunks[b] = std::max(G, (int)chunk / G * G);
   }
 }
@@ -1140,7 +1150,7 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
   pl->grid = sms * t.ctas_per_sm;
   {  // chunks not given: the work model for this batch and these resident warps
     int mc[LIGATE_N_BUCKETS];
-    model_chunks(B->d, sel, pl->n_ligands, p.S, p.n_starts, (double)pl->grid * t.warps_per_cta, p.G, mc);
+    model_chunks(B->d, sel, pl->n_ligands, p.S, p.n_starts, (double)pl->grid * t.warps_per_cta, p.G, p.K, mc);
     for (int b = 0; b < LIGATE_N_BUCKETS; ++b)
       if (t.starts_per_item[b] <= 0) t.starts_per_item[b] = mc[b];
   }
@@ -1223,14 +1233,11 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
   for (size_t i = 0; i < order.size(); ++i) sorted[i] = items[order[i]];
   const size_t ni = items.size();
   cudaError_t e;
-  pl->counter_bytes = sizeof(int) * (2 * (size_t)n + 1);  // queue, done[n], lig_thr[n]
-  if ((e = dmalloc(&pl->stats, N_STATS)) != cudaSuccess) {
-    free_plan(pl);
-    return cuda_fail(e, "plan allocation");
-  }
+  // stats (64-bit), queue, done[n], lig_thr[n]: one array, reset at once
+  pl->counter_bytes = sizeof(unsigned long long) * N_STATS + sizeof(int) * (2 * (size_t)n + 1);
   if ((e = dmalloc(&pl->items, ni)) != cudaSuccess || (e = dmalloc(&pl->lig_items, n)) != cudaSuccess ||
       (e = dmalloc(&pl->lig_slot0, n)) != cudaSuccess ||
-      (e = dmalloc(&pl->counters, 2 * (size_t)n + 1)) != cudaSuccess ||
+      (e = dmalloc(&pl->stats, pl->counter_bytes / sizeof(unsigned long long) + 1)) != cudaSuccess ||
       (e = dmalloc(&pl->partial, ni * p.K)) != cudaSuccess ||
       (e = dmalloc(&pl->out, (size_t)n * p.K)) != cudaSuccess) {
     free_plan(pl);
@@ -1259,6 +1266,7 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
       if ((e = dmalloc(&p.memo1, floats)) != cudaSuccess) { free_plan(pl); return cuda_fail(e, "plan allocation"); }
     }
   }
+  pl->counters = reinterpret_cast<int *>(pl->stats + N_STATS);
   p.items = pl->items;
   p.n_items = (int)ni;
   p.lig_items = pl->lig_items;
@@ -1300,8 +1308,7 @@ static ligate_status plan_capture(ligate_plan *pl) {
   if (pl->exec) return LIGATE_OK;
   CK(cudaStreamCreateWithFlags(&pl->cap_stream, cudaStreamNonBlocking), "capture stream");
   CK(cudaStreamBeginCapture(pl->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-  cudaError_t e = cudaMemsetAsync(pl->counters, 0, pl->counter_bytes, pl->cap_stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(pl->stats, 0, N_STATS * sizeof(unsigned long long), pl->cap_stream);
+  cudaError_t e = cudaMemsetAsync(pl->stats, 0, pl->counter_bytes, pl->cap_stream);
   if (e == cudaSuccess && pl->p.n_items > 0) e = launch_clash_tables(pl->p, pl->row_lig, pl->n_ligands, pl->cap_stream);
   if (e == cudaSuccess && pl->p.n_items > 0)
     e = launch_dock(pl->mode, pl->tile.reg_cap, pl->p, pl->grid, pl->block, pl->smem, pl->cap_stream);
@@ -1482,18 +1489,24 @@ extern "C" ligate_status ligate_plan_run_subset(ligate_plan *pl, const int32_t *
         (n && (e = cudaMemcpy(pl->lig_bucket, bucket.data(), (size_t)n, cudaMemcpyHostToDevice)) != cudaSuccess))
       return cuda_fail(e, "plan_run_subset: set-up");
   }
-  // chunks from the work model for a selection of n_sel average ligands
+  // chunks from the work model for a selection of m average ligands
   SubsetChunks ch;
-  int cmin = 2048;
   const double P_warps = std::max(1.0, (double)pl->grid * pl->tile.warps_per_cta);
-  for (int b = 0; b < LIGATE_N_BUCKETS; ++b) {
-    double chunk = 512.0;
-    if (pl->model_cb[b] > 0) chunk = pl->model_W * ((double)n_sel / std::max(n, 1)) / (8.0 * P_warps * pl->model_cb[b]);
-    chunk = std::min(2048.0, std::max(128.0, chunk));
-    ch.c[b] = std::max(p.G, (int)chunk / p.G * p.G);
-    cmin = std::min(cmin, ch.c[b]);
-  }
-  const size_t need = (size_t)n_sel * (size_t)((p.n_starts + cmin - 1) / cmin);
+  auto chunks = [&](int m) {  // into ch; the most items such a selection has
+    int cmin = 2048;
+    for (int b = 0; b < LIGATE_N_BUCKETS; ++b) {
+      double chunk = 512.0;
+      if (pl->model_cb[b] > 0) chunk = pl->model_W * ((double)m / std::max(n, 1)) / (8.0 * P_warps * pl->model_cb[b]);
+      chunk = std::min(2048.0, std::max(least_chunk((double)m * p.n_starts, P_warps, p.K), chunk));
+      ch.c[b] = std::max(p.G, (int)chunk / p.G * p.G);
+      cmin = std::min(cmin, ch.c[b]);
+    }
+    return (size_t)m * (size_t)((p.n_starts + cmin - 1) / cmin);
+  };
+  size_t need = chunks(n_sel);
+  if (need > pl->sub_cap)  // room for every smaller selection too: those have smaller chunks
+    for (int m = n_sel; m > 0; m -= std::max(1, m / 64)) need = std::max(need, chunks(m) + chunks(m) / 32);
+  chunks(n_sel);
   if (need > pl->sub_cap) {  // grows only
     cudaFree(pl->sub_items);
     cudaFree(pl->sub_partial);
@@ -1516,9 +1529,7 @@ extern "C" ligate_status ligate_plan_run_subset(ligate_plan *pl, const int32_t *
     subset_meta_kernel<<<blocks, 256, 0, s>>>(ligands, n_sel, B.n_ligands, pl->rowmap, pl->sub_row_lig, pl->out,
                                               p.K);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "plan_run_subset: selection");
-    if ((e = cudaMemsetAsync(pl->counters, 0, sizeof(int) * ((size_t)n_sel + 1), s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(pl->counters + 1 + n, 0, sizeof(int) * (size_t)n_sel, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(pl->stats, 0, N_STATS * sizeof(unsigned long long), s)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(pl->stats, 0, pl->counter_bytes, s)) != cudaSuccess)
       return cuda_fail(e, "plan_run_subset");
     DockParams q = p;
     q.items = pl->sub_items;
@@ -1573,8 +1584,7 @@ extern "C" void ligate_plan_destroy(ligate_plan *pl) { free_plan(pl); }
 
 // One docking run of a plan, launched directly on `st` (no graph).
 static cudaError_t plan_launch(ligate_plan *pl, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(pl->counters, 0, pl->counter_bytes, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(pl->stats, 0, N_STATS * sizeof(unsigned long long), st);
+  cudaError_t e = cudaMemsetAsync(pl->stats, 0, pl->counter_bytes, st);
   if (e == cudaSuccess && pl->p.n_items > 0) e = launch_clash_tables(pl->p, pl->row_lig, pl->n_ligands, st);
   if (e == cudaSuccess && pl->p.n_items > 0)
     e = launch_dock(pl->mode, pl->tile.reg_cap, pl->p, pl->grid, pl->block, pl->smem, st);
@@ -2289,7 +2299,7 @@ extern "C" ligate_status ligate_model_tile(const ligate_pocket *P, const ligate_
     return LIGATE_ERR_UNSUPPORTED;
   }
   model_chunks(B->d, nullptr, B->d.n_ligands, S, s->n_orient * s->n_anchor, (double)sms * best_res, G,
-               t.starts_per_item);
+               s->top_k, t.starts_per_item);
   *out = t;
   return LIGATE_OK;
 }
