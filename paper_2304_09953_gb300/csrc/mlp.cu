@@ -3,13 +3,14 @@
 //
 // MLP 256 -> 512 -> 512 -> 512 -> 1, ReLU on hidden layers.  Weights and
 // activations in BF16, products accumulated in FP32 by mma.sync m16n8k16,
-// FP32 master weights updated by Adam.  One tiled GEMM kernel serves the
-// three product shapes of a training step:
+// FP32 master weights updated by Adam.  Products of a training step:
 //   forward      H_l = relu(H_{l-1} W_l + b_l)        A row-major, B row-major
 //   data grad    dH_{l-1} = dZ_l W_l^T (then ReLU mask) A row-major, B = W^T
 //   weight grad  dW_l = H_{l-1}^T dZ_l                 A = H^T,      B row-major
-// Operand layouts are template flags; ldmatrix (.trans where the tile is
-// stored k-major) feeds the fragments.
+// The first two run on tcgen05 (mlp_tc05.cu) or, with LIGATE_MLP_GEMM=mma, on
+// gemm_kernel here; the weight gradients of all layers are one launch
+// (grads_kernel).  ldmatrix (.trans where the tile is stored k-major) feeds
+// the fragments.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -47,14 +48,14 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// C[M][N] = sum_k A(m,k) B(k,n).  A(m,k) = A[m*sAm + k*sAk], B(k,n) =
-// B[k*sBk + n*sBn]; the contiguous dimension (stride 1) is given by the
-// template flags and must be a multiple of 8 elements with 16 B aligned
+// C[M][N] = sum_k A(m,k) B(k,n).  A(m,k) = A[m*sAm + k], B(k,n) = B[k*sBk +
+// n*sBn]; B's contiguous dimension (stride 1) is given by the template flag;
+// contiguous dimensions must be multiples of 8 elements with 16 B aligned
 // rows; the other dimension is bounds-checked (zero fill).
-template <bool A_KCONTIG, bool B_KCONTIG, int EPI>
+template <bool B_KCONTIG, int EPI>
 __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
-  // A tile: [BM][BKT+PAD] if k-contiguous else [BKT][BM+PAD]; same for B with BN.
-  __shared__ __align__(16) __nv_bfloat16 As[A_KCONTIG ? BM * (BKT + PAD) : BKT * (BM + PAD)];
+  // B tile: [BN][BKT+PAD] if k-contiguous else [BKT][BN+PAD].
+  __shared__ __align__(16) __nv_bfloat16 As[BM * (BKT + PAD)];
   __shared__ __align__(16) __nv_bfloat16 Bs[B_KCONTIG ? BN * (BKT + PAD) : BKT * (BN + PAD)];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int wm = warp >> 2, wn = warp & 3;  // 2 x 4 warps, warp tile 64 x 32
@@ -74,16 +75,11 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
     for (int r = 0; r < 2; ++r) {
       const int c = tid + r * 256;  // 512 16-byte chunks per tile
       uint4 v = make_uint4(0, 0, 0, 0);
-      if (A_KCONTIG) {
+      {
         const int row = c >> 2, kc = (c & 3) * 8;
         const int m = m0 + row, k = k0 + kc;
         if (m < g.M && k < g.K) v = *reinterpret_cast<const uint4 *>(A + (size_t)m * g.sAm + k);
         *reinterpret_cast<uint4 *>(&As[row * (BKT + PAD) + kc]) = v;
-      } else {
-        const int krow = c >> 4, mc = (c & 15) * 8;
-        const int m = m0 + mc, k = k0 + krow;
-        if (k < g.K && m < g.M) v = *reinterpret_cast<const uint4 *>(A + (size_t)k * g.sAk + m);
-        *reinterpret_cast<uint4 *>(&As[krow * (BM + PAD) + mc]) = v;
       }
       uint4 w = make_uint4(0, 0, 0, 0);
       if (B_KCONTIG) {
@@ -106,14 +102,8 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int mb = wm * 64 + i * 16;
-        if (A_KCONTIG) {
-          const __nv_bfloat16 *p = &As[(mb + (lane & 15)) * (BKT + PAD) + ks + (lane >> 4) * 8];
-          ldsm_x4(af[i][0], af[i][1], af[i][2], af[i][3], p);
-        } else {
-          const int r = lane & 7, mi = (lane >> 3) & 1, ki = lane >> 4;
-          const __nv_bfloat16 *p = &As[(ks + ki * 8 + r) * (BM + PAD) + mb + mi * 8];
-          ldsm_x4_t(af[i][0], af[i][1], af[i][2], af[i][3], p);
-        }
+        const __nv_bfloat16 *p = &As[(mb + (lane & 15)) * (BKT + PAD) + ks + (lane >> 4) * 8];
+        ldsm_x4(af[i][0], af[i][1], af[i][2], af[i][3], p);
       }
 #pragma unroll
       for (int j = 0; j < 4; j += 2) {
@@ -151,30 +141,160 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
           v0 = fmaxf(v0 + g.bias[n], 0.f);
           v1 = fmaxf(v1 + g.bias[n + 1], 0.f);
           *reinterpret_cast<__nv_bfloat162 *>(g.Cb + (size_t)m * g.ldc + n) = __floats2bfloat162_rn(v0, v1);
-        } else if (EPI == EPI_RELU_MASK) {
+        } else {
           const __nv_bfloat162 hm = *reinterpret_cast<const __nv_bfloat162 *>(g.mask + (size_t)m * g.ldc + n);
           if (!(__bfloat162float(hm.x) > 0.f)) v0 = 0.f;
           if (!(__bfloat162float(hm.y) > 0.f)) v1 = 0.f;
           *reinterpret_cast<__nv_bfloat162 *>(g.Cb + (size_t)m * g.ldc + n) = __floats2bfloat162_rn(v0, v1);
-        } else {
-          *reinterpret_cast<float2 *>(g.Cf + (size_t)m * g.ldc + n) = make_float2(v0, v1);
         }
       }
 }
 
-template <bool AK, bool BKc, int EPI>
+template <bool BKc, int EPI>
 static cudaError_t gemm_t(const GemmArgs &g, cudaStream_t s) {
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
-  gemm_kernel<AK, BKc, EPI><<<grid, 256, 0, s>>>(g);
+  gemm_kernel<BKc, EPI><<<grid, 256, 0, s>>>(g);
   return cudaGetLastError();
 }
 
 cudaError_t gemm(int kind, const GemmArgs &g, cudaStream_t s) {
-  switch (kind) {
-    case GEMM_FWD: return gemm_t<true, false, EPI_BIAS_RELU>(g, s);
-    case GEMM_DGRAD: return gemm_t<true, true, EPI_RELU_MASK>(g, s);
-    default: return gemm_t<false, false, EPI_F32>(g, s);
+  return kind == GEMM_FWD ? gemm_t<false, EPI_BIAS_RELU>(g, s) : gemm_t<true, EPI_RELU_MASK>(g, s);
+}
+
+// ---------------------------------------------------------------------------
+// All parameter gradients of one training step in one launch: for each hidden
+// layer the weight gradient dW = H^T dZ (64 x 32 tiles, mma.sync m16n8k16,
+// rows as k) and the column sums of dZ (bias gradients), and the head's
+// gw4[k] = sum_b H3[b][k] dy[b] and gb4 = sum_b dy[b].  Rows stream through a
+// four-stage cp.async ring of 64-row slices.
+//
+// What bounds it: every sum runs over the rows in ascending order, so it is a
+// serial chain per output (the MMA steps of a tile; one addition per row of a
+// column sum); the launch is as wide as the outputs allow (320 tiles + 32
+// column CTAs, all resident at once) and the loads are off the chain.  Before,
+// the sums ran as launches of their own on 2 and 4 CTAs with every load on the
+// chain and the weight gradients on 8 to 16 CTAs without overlap: 87 + 3 x 61
+// + 3 x 37 us per step of 1,024 rows (serialised, cold), now 21.
+constexpr int GK = 64, GM = 64, GN = 32, GC = 64, GSTAGES = 4;  // rows per slice, tile, columns of a sum CTA
+constexpr int GA_LD = GM + 8, GB_LD = GN + 8, GC_LD = GC + 8;
+constexpr int G_STAGE = GK * (GA_LD + GB_LD);  // elements per stage (a sum CTA's slice is smaller)
+static_assert(GK * GC_LD <= G_STAGE, "column slices fit the stage");
+
+__device__ __forceinline__ void cp16(void *dst, const void *src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0)
+               : "memory");
+}
+// rows [k0, k0 + GK) x COLS columns from column c0 of src [rows][ld] into dst (zero past the last row)
+template <int COLS, int LD>
+__device__ __forceinline__ void load_slice(__nv_bfloat16 *dst, const __nv_bfloat16 *src, int ld, int c0, int k0,
+                                           int rows) {
+  constexpr int CH = COLS / 8;
+#pragma unroll
+  for (int c = threadIdx.x; c < GK * CH; c += 128) {
+    const int r = c / CH, q = c % CH * 8;
+    const bool in = k0 + r < rows;
+    cp16(dst + r * LD + q, src + (size_t)(in ? k0 + r : 0) * ld + c0 + q, in);
   }
+}
+
+__global__ void __launch_bounds__(128) grads_kernel(const GradArgs a) {
+  extern __shared__ __align__(16) unsigned char graw[];
+  __nv_bfloat16 *const ring = reinterpret_cast<__nv_bfloat16 *>(graw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int slices = (a.rows + GK - 1) / GK;
+  int t = blockIdx.x;
+  int layer = 0;
+  for (; layer < 3; ++layer) {  // a weight tile of this layer?
+    const int n = (a.fan_in[layer] / GM) * (512 / GN);
+    if (t < n) break;
+    t -= n;
+  }
+  if (layer < 3) {
+    const int m0 = t / (512 / GN) * GM, n0 = t % (512 / GN) * GN, mb = warp * 16;
+    auto load = [&](int s) {
+      __nv_bfloat16 *st = ring + (s % GSTAGES) * G_STAGE;
+      load_slice<GM, GA_LD>(st, a.in[layer], a.fan_in[layer], m0, s * GK, a.rows);
+      load_slice<GN, GB_LD>(st + GK * GA_LD, a.dz[layer], 512, n0, s * GK, a.rows);
+    };
+    float acc[4][4] = {};
+    for (int s = 0; s < GSTAGES - 1; ++s) {
+      if (s < slices) load(s);
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    for (int s = 0; s < slices; ++s) {
+      asm volatile("cp.async.wait_group %0;\n" ::"n"(GSTAGES - 2) : "memory");
+      __syncthreads();
+      if (s + GSTAGES - 1 < slices) load(s + GSTAGES - 1);  // the stage read in the last iteration
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      const __nv_bfloat16 *As = ring + (s % GSTAGES) * G_STAGE, *Bs = As + GK * GA_LD;
+      const int r = lane & 7, q1 = (lane >> 3) & 1, q2 = lane >> 4;
+#pragma unroll
+      for (int ks = 0; ks < GK; ks += 16) {
+        uint32_t af[4], bf[4][2];
+        ldsm_x4_t(af[0], af[1], af[2], af[3], As + (ks + q2 * 8 + r) * GA_LD + mb + q1 * 8);
+#pragma unroll
+        for (int j = 0; j < 4; j += 2)
+          ldsm_x4_t(bf[j][0], bf[j][1], bf[j + 1][0], bf[j + 1][1], Bs + (ks + q1 * 8 + r) * GB_LD + j * 8 + q2 * 8);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma_bf16(acc[j], af, bf[j][0], bf[j][1]);
+      }
+    }
+    float *dw = a.dw[layer];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int m = m0 + mb + (lane >> 2) + h * 8, n = n0 + j * 8 + (lane & 3) * 2;
+        *reinterpret_cast<float2 *>(dw + (size_t)m * 512 + n) = make_float2(acc[j][2 * h], acc[j][2 * h + 1]);
+      }
+    return;
+  }
+  // column sums: 3 x 8 CTAs of the bias gradients, then 8 of the head
+  const int what = t / (512 / GC), c0 = t % (512 / GC) * GC;
+  const bool head = what == 3;
+  const __nv_bfloat16 *src = head ? a.h3 : a.dz[what];
+  __shared__ float dys[GSTAGES][GK];
+  auto load = [&](int s) {
+    load_slice<GC, GC_LD>(ring + (s % GSTAGES) * G_STAGE, src, 512, c0, s * GK, a.rows);
+    if (head && tid < GK) dys[s % GSTAGES][tid] = s * GK + tid < a.rows ? a.dy[s * GK + tid] : 0.f;
+  };
+  float sum = 0.f;
+  for (int s = 0; s < GSTAGES - 1; ++s) {
+    if (s < slices) load(s);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  for (int s = 0; s < slices; ++s) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(GSTAGES - 2) : "memory");
+    __syncthreads();
+    if (s + GSTAGES - 1 < slices) load(s + GSTAGES - 1);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    const __nv_bfloat16 *col = ring + (s % GSTAGES) * G_STAGE + tid;
+    const float *dy = dys[s % GSTAGES];
+    if (tid < GC) {
+      if (head) {
+#pragma unroll 16
+        for (int r = 0; r < GK; ++r) sum = fmaf(__bfloat162float(col[r * GC_LD]), dy[r], sum);
+      } else {
+#pragma unroll 16
+        for (int r = 0; r < GK; ++r) sum += __bfloat162float(col[r * GC_LD]);
+      }
+    } else if (tid == GC && head && c0 == 0) {
+#pragma unroll 16
+      for (int r = 0; r < GK; ++r) sum += dy[r];
+    }
+  }
+  if (tid < GC) (head ? a.gw4 : a.db[what])[c0 + tid] = sum;
+  else if (tid == GC && head && c0 == 0) a.gb4[0] = sum;
+}
+
+cudaError_t grads(const GradArgs &a, cudaStream_t s) {
+  const int smem = GSTAGES * G_STAGE * 2;
+  cudaError_t e = cudaFuncSetAttribute(grads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  int ctas = 4 * (512 / GC);
+  for (int l = 0; l < 3; ++l) ctas += (a.fan_in[l] / GM) * (512 / GN);
+  grads_kernel<<<ctas, 128, smem, s>>>(a);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -197,12 +317,10 @@ __global__ void gather_std_kernel(const float *__restrict__ desc, const int *__r
 // Last layer y[b] = H3[b] . w4 + b4 (one warp per row); with targets, also
 // dy = 2 (y - t) / B, the squared error sum, and dZ3 = dy w4^T masked by
 // H3 > 0 (BF16).
-__global__ void head_kernel(const __nv_bfloat16 *__restrict__ h3, const __nv_bfloat16 *__restrict__ w4,
-                            const float *__restrict__ b4, int rows, const float *__restrict__ t,
-                            float *__restrict__ y, float *__restrict__ dy, float inv_b2,
-                            double *__restrict__ sse, __nv_bfloat16 *__restrict__ dz3) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= rows) return;
+__device__ __forceinline__ void head_row(const __nv_bfloat16 *__restrict__ h3, const __nv_bfloat16 *__restrict__ w4,
+                                         const float *__restrict__ b4, const float *__restrict__ t,
+                                         float *__restrict__ y, float *__restrict__ dy, float inv_b2,
+                                         __nv_bfloat16 *__restrict__ dz3, int warp, int lane, double *sq) {
   const __nv_bfloat16 *h = h3 + (size_t)warp * 512;
   float s = 0.f;
   for (int k = lane; k < 512; k += 32) s = fmaf(__bfloat162float(h[k]), __bfloat162float(w4[k]), s);
@@ -215,7 +333,7 @@ __global__ void head_kernel(const __nv_bfloat16 *__restrict__ h3, const __nv_bfl
   const float d = inv_b2 * e;  // 2 (y - t) / B
   if (lane == 0) {
     dy[warp] = d;
-    atomicAdd(sse, (double)e * e);
+    *sq = (double)e * e;
   }
   for (int k = lane; k < 512; k += 32) {
     const float hv = __bfloat162float(h[k]);
@@ -223,45 +341,79 @@ __global__ void head_kernel(const __nv_bfloat16 *__restrict__ h3, const __nv_bfl
   }
 }
 
-// Gradients of the last layer: gw4[k] = sum_b H3[b][k] dy[b], gb4 = sum_b dy[b].
-__global__ void head_grad_kernel(const __nv_bfloat16 *__restrict__ h3, const float *__restrict__ dy,
-                                 int rows, float *__restrict__ gw4, float *__restrict__ gb4) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < 512) {
-    float s = 0.f;
-    for (int b = 0; b < rows; ++b) s = fmaf(__bfloat162float(h3[(size_t)b * 512 + k]), dy[b], s);
-    gw4[k] = s;
-  }
-  if (k == 0) {
-    float s = 0.f;
-    for (int b = 0; b < rows; ++b) s += dy[b];
-    gb4[0] = s;
+__global__ void head_kernel(const __nv_bfloat16 *__restrict__ h3, const __nv_bfloat16 *__restrict__ w4,
+                            const float *__restrict__ b4, int rows, const float *__restrict__ t,
+                            float *__restrict__ y, float *__restrict__ dy, float inv_b2,
+                            double *__restrict__ sse, __nv_bfloat16 *__restrict__ dz3) {
+  __shared__ double sq[8];  // squared errors of the CTA's 8 rows: one atomic per CTA
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x < 8) sq[threadIdx.x] = 0.0;
+  __syncthreads();
+  if (warp < rows) head_row(h3, w4, b4, t, y, dy, inv_b2, dz3, warp, lane, &sq[threadIdx.x >> 5]);
+  if (!t) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double e2 = 0.0;
+    for (int q = 0; q < 8; ++q) e2 += sq[q];
+    atomicAdd(sse, e2);
   }
 }
+// Adam (Kingma & Ba, Algorithm 1) on FP32 master weights, then their BF16
+// copies: row-major wb and, for tcgen05, the transposed hidden weights wt.  A
+// CTA of 256 threads owns a 32 x 32 tile of a hidden weight matrix (transposed
+// through shared memory) or 1,024 of the remaining parameters; one launch in
+// place of an elementwise pass and three transposes that read the weights
+// again (6.2 + 10.6 us per step, serialised, to 6.3).
+struct AdamArgs {
+  float *w;
+  const float *g;
+  float *m, *v;
+  __nv_bfloat16 *wb, *wt;
+  int off[3], K[3], wt_off[3];  // hidden layers: weights at w + off, [K][512]
+  int rest0[4], rest1[4];       // the other parameters' ranges
+  float lr, b1, b2, eps, c1, c2;
+};
 
-// Column sums of BF16 dZ[rows][cols] (bias gradients).
-__global__ void colsum_kernel(const __nv_bfloat16 *__restrict__ dz, int rows, int cols,
-                              float *__restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int b = 0; b < rows; ++b) s += __bfloat162float(dz[(size_t)b * cols + c]);
-  out[c] = s;
+__device__ __forceinline__ __nv_bfloat16 adam_one(const AdamArgs &a, int i) {
+  const float gi = a.g[i];
+  // products and sums written out: the rounding does not depend on how a
+  // compiler contracts them
+  const float mi = fmaf(1.f - a.b1, gi, __fmul_rn(a.b1, a.m[i]));
+  const float vi = fmaf(__fmul_rn(1.f - a.b2, gi), gi, __fmul_rn(a.b2, a.v[i]));
+  a.m[i] = mi;
+  a.v[i] = vi;
+  const float wi = a.w[i] - a.lr * (mi * a.c1) / (sqrtf(vi * a.c2) + a.eps);
+  a.w[i] = wi;
+  const __nv_bfloat16 b = __float2bfloat16_rn(wi);
+  a.wb[i] = b;
+  return b;
 }
 
-// Adam (Kingma & Ba, Algorithm 1) on FP32 master weights, then the BF16 copy.
-__global__ void adam_kernel(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                            float *__restrict__ v, __nv_bfloat16 *__restrict__ wb, int n, float lr,
-                            float b1, float b2, float eps, float c1, float c2) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
-    w[i] = wi;
-    wb[i] = __float2bfloat16_rn(wi);
+__global__ void __launch_bounds__(256) adam_kernel(const AdamArgs a) {
+  __shared__ __nv_bfloat16 tile[32][34];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  int t = blockIdx.x;
+  for (int l = 0; l < 3; ++l) {
+    const int n = a.K[l] / 32 * 16;
+    if (t >= n) { t -= n; continue; }
+    const int k0 = t / 16 * 32, n0 = t % 16 * 32;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tile[ty + 8 * q][tx] = adam_one(a, a.off[l] + (k0 + ty + 8 * q) * 512 + n0 + tx);
+    if (!a.wt) return;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      a.wt[a.wt_off[l] + (size_t)(n0 + ty + 8 * q) * a.K[l] + k0 + tx] = tile[tx][ty + 8 * q];
+    return;
+  }
+  for (int r = 0; r < 4; ++r) {
+    const int n = (a.rest1[r] - a.rest0[r] + 1023) / 1024;
+    if (t >= n) { t -= n; continue; }
+    for (int q = threadIdx.x; q < 1024; q += 256) {
+      const int i = a.rest0[r] + t * 1024 + q;
+      if (i < a.rest1[r]) adam_one(a, i);
+    }
+    return;
   }
 }
 
@@ -410,19 +562,25 @@ cudaError_t head(const __nv_bfloat16 *h3, const __nv_bfloat16 *w4, const float *
   head_kernel<<<(rows * 32 + 255) / 256, 256, 0, s>>>(h3, w4, b4, rows, t, y, dy, inv_b2, sse, dz3);
   return cudaGetLastError();
 }
-cudaError_t head_grad(const __nv_bfloat16 *h3, const float *dy, int rows, float *gw4, float *gb4,
-                      cudaStream_t s) {
-  head_grad_kernel<<<2, 256, 0, s>>>(h3, dy, rows, gw4, gb4);
-  return cudaGetLastError();
-}
-cudaError_t colsum(const __nv_bfloat16 *dz, int rows, int cols, float *out, cudaStream_t s) {
-  colsum_kernel<<<(cols + 127) / 128, 128, 0, s>>>(dz, rows, cols, out);
-  return cudaGetLastError();
-}
-cudaError_t adam(float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb, int n, float lr,
+cudaError_t adam(float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb, __nv_bfloat16 *wt, float lr,
                  float b1, float b2, float eps, float c1, float c2, cudaStream_t s) {
-  adam_kernel<<<(n + 255) / 256 < 2048 ? (n + 255) / 256 : 2048, 256, 0, s>>>(w, g, m, v, wb, n, lr,
-                                                                               b1, b2, eps, c1, c2);
+  AdamArgs a;
+  a.w = w; a.g = g; a.m = m; a.v = v; a.wb = wb; a.wt = wt;
+  a.lr = lr; a.b1 = b1; a.b2 = b2; a.eps = eps; a.c1 = c1; a.c2 = c2;
+  int o = 0, tw = 0, ctas = 0;
+  for (int l = 0; l < 3; ++l) {  // W1 [256][512], W2, W3 [512][512], each followed by its bias
+    a.K[l] = l == 0 ? 256 : 512;
+    a.off[l] = o;
+    a.wt_off[l] = tw;
+    o += a.K[l] * 512;
+    tw += a.K[l] * 512;
+    a.rest0[l] = o;
+    a.rest1[l] = o += 512;
+    ctas += a.K[l] / 32 * 16 + 1;
+  }
+  a.rest0[3] = o;  // W4 [512] and its bias
+  a.rest1[3] = o + 513;
+  adam_kernel<<<ctas + 1, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 cudaError_t to_bf16(const float *a, __nv_bfloat16 *b, int n, cudaStream_t s) {

@@ -8,17 +8,16 @@
 namespace ligate {
 namespace mlp {
 
-enum { EPI_BIAS_RELU = 0, EPI_RELU_MASK = 1, EPI_F32 = 2 };
-enum { GEMM_FWD = 0, GEMM_DGRAD = 1, GEMM_WGRAD = 2 };
+enum { EPI_BIAS_RELU = 0, EPI_RELU_MASK = 1 };
+enum { GEMM_FWD = 0, GEMM_DGRAD = 1 };
 
 struct GemmArgs {
   const __nv_bfloat16 *A, *B;
   int M, N, K;
-  long long sAm, sAk, sBk, sBn;  // element strides (the contiguous one is 1)
+  long long sAm, sBk, sBn;       // element strides (the contiguous ones are 1)
   const float *bias;             // EPI_BIAS_RELU
   const __nv_bfloat16 *mask;     // EPI_RELU_MASK: ReLU output of the forward layer
   __nv_bfloat16 *Cb;             // BF16 output
-  float *Cf;                     // FP32 output
   int ldc;
 };
 
@@ -29,10 +28,23 @@ cudaError_t gather_std(const float *desc, const int *idx, int rows, int row0, co
 cudaError_t head(const __nv_bfloat16 *h3, const __nv_bfloat16 *w4, const float *b4, int rows,
                  const float *t, float *y, float *dy, float inv_b2, double *sse, __nv_bfloat16 *dz3,
                  cudaStream_t s);
-cudaError_t head_grad(const __nv_bfloat16 *h3, const float *dy, int rows, float *gw4, float *gb4,
-                      cudaStream_t s);
-cudaError_t colsum(const __nv_bfloat16 *dz, int rows, int cols, float *out, cudaStream_t s);
-cudaError_t adam(float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb, int n, float lr,
+// Parameter gradients of a step: hidden layers l = 0..2 with inputs in[l]
+// [rows][fan_in[l]] and output gradients dz[l] [rows][512] -> dw[l]
+// [fan_in][512] and db[l][512]; head inputs h3 [rows][512] and dy [rows] ->
+// gw4[512], gb4[1].
+struct GradArgs {
+  const __nv_bfloat16 *in[3], *dz[3];
+  float *dw[3], *db[3];
+  int fan_in[3];
+  const __nv_bfloat16 *h3;
+  const float *dy;
+  float *gw4, *gb4;
+  int rows;
+};
+cudaError_t grads(const GradArgs &a, cudaStream_t s);
+// Adam over the flat parameter vector (LIGATE_SURROGATE_PARAMS); wt: the
+// transposed BF16 hidden weights, or NULL.
+cudaError_t adam(float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb, __nv_bfloat16 *wt, float lr,
                  float b1, float b2, float eps, float c1, float c2, cudaStream_t s);
 cudaError_t to_bf16(const float *a, __nv_bfloat16 *b, int n, cudaStream_t s);
 cudaError_t feature_stats(const float *desc, int n, float *mu, float *inv_sd, cudaStream_t s);

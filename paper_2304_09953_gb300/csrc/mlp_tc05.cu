@@ -6,13 +6,21 @@
 //     EPI_BIAS_RELU  forward layer   C = relu(acc + bias)   (B = W^T)
 //     EPI_RELU_MASK  data gradient   C = acc * (mask > 0)   (B = W)
 //
-// One CTA computes a 128 x 256 tile.  One elected thread streams 64-wide K
-// slices of X and Wt into shared memory with TMA (128-byte swizzle, three
-// stages, mbarrier transaction counts) and issues tcgen05.mma (kind::f16,
-// M = 128, N = 256, K = 16 per instruction) into a 256-column FP32
-// accumulator in tensor memory; tcgen05.commit signals each stage's release
-// and the final completion.  All four warps then read their 32 accumulator
-// rows with tcgen05.ld, add the bias, apply ReLU and store BF16.
+// One CTA computes a 128 x TN tile.  One elected thread streams 64-wide K
+// slices of X and Wt into shared memory with TMA (128-byte swizzle, mbarrier
+// transaction counts) and issues tcgen05.mma (kind::f16, M = 128, N = TN, K =
+// 16 per instruction) into a TN-column FP32 accumulator in tensor memory;
+// tcgen05.commit signals each stage's release and the final completion.  All
+// four warps then read their 32 accumulator rows with tcgen05.ld, add the
+// bias, apply ReLU and store BF16.
+//
+// TN and the stages follow the rows: a mini-batch of 1,024 rows has 8 row
+// tiles, so 256-column tiles would leave 136 of 152 SMs idle; narrow tiles (64
+// or 32 columns) fill them, and eight stages put the whole K = 512 in flight at
+// once, which makes the launch one memory latency, the MMAs and a short
+// epilogue.  Each output's sum runs over K in the same order for every TN.
+//
+// mlp_forward_kernel runs the whole network for inference: see there.
 //
 // Every mbarrier wait is bounded by the global timer: on a timeout the kernel
 // records an error, drains what it issued (bounded again), frees its tensor
@@ -31,9 +39,8 @@ namespace ligate {
 namespace mlp {
 namespace {
 
-constexpr int TM = 128, TN = 256, TK = 64, STAGES = 3;
-constexpr int A_BYTES = TM * TK * 2, B_BYTES = TN * TK * 2;  // 16 KB + 32 KB per stage
-constexpr int TMEM_COLS = 256;
+constexpr int TM = 128, TK = 64;
+constexpr int A_BYTES = TM * TK * 2;  // 16 KB per K slice
 constexpr unsigned long long WAIT_NS = 2000000000ull;  // 2 s per wait
 
 __device__ __forceinline__ uint32_t saddr(const void *p) {
@@ -85,14 +92,16 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
 // Instruction descriptor of kind::f16: FP32 accumulator (bits [4,6) = 1),
 // BF16 A and B ([7,10) = 1, [10,13) = 1), both K-major, N >> 3 in [17,23),
 // M >> 4 in [24,29).
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                           ((uint32_t)(TM >> 4) << 24);
+constexpr uint32_t idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+}
 
+template <int N>
 __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(tmem_d), "l"(a), "l"(b), "r"(IDESC), "r"(acc));
+      ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc(N)), "r"(acc));
 }
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -104,24 +113,26 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
 // nothing in normal operation sets it.
 __device__ int g_fault_skip_loads = 0;
 
+template <int TN, int STAGES>
 struct __align__(1024) Smem {
   uint8_t a[STAGES][A_BYTES];
-  uint8_t b[STAGES][B_BYTES];
+  uint8_t b[STAGES][TN * TK * 2];
   uint64_t full[STAGES];
   uint64_t empty[STAGES];
   uint64_t done;
   uint32_t tmem_base;
 };
 
-template <int EPI>
+template <int EPI, int TN, int STAGES>
 __global__ void __launch_bounds__(128, 1)
     gemm_tc05_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                      int M, int K, const float *__restrict__ bias,
                      const __nv_bfloat16 *__restrict__ mask, __nv_bfloat16 *__restrict__ out,
                      int ldc, int *__restrict__ err) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  Smem &s = *reinterpret_cast<Smem *>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  typedef Smem<TN, STAGES> S;
+  constexpr int B_BYTES = TN * TK * 2, TMEM_COLS = TN;
+  S &s = *reinterpret_cast<S *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
   const int nk = K / TK;
@@ -164,7 +175,7 @@ __global__ void __launch_bounds__(128, 1)
       const uint64_t da = sdesc(saddr(s.a[st])), db = sdesc(saddr(s.b[st]));
 #pragma unroll
       for (int kk = 0; kk < TK / 16; ++kk)  // 16 BF16 = 32 B per step: +2 in the address field
-        mma_f16(tmem, da + 2 * kk, db + 2 * kk, (kb > 0 || kk > 0) ? 1u : 0u);
+        mma_f16<TN>(tmem, da + 2 * kk, db + 2 * kk, (kb > 0 || kk > 0) ? 1u : 0u);
       mma_commit(&s.empty[st]);
       if (kb + STAGES < nk) {  // refill this stage once its MMAs are done
         if (!mbar_wait(&s.empty[st], ph)) { ok = false; break; }
@@ -271,8 +282,35 @@ bool make_map(CUtensorMap *m, const void *base, int rows, int cols, int box_rows
 }  // namespace
 
 bool tc05_supported(int M, int N, int K) {
-  return M > 0 && N % TN == 0 && K % TK == 0 && K >= TK && encode_fn() != nullptr;
+  return M > 0 && N % 256 == 0 && K % TK == 0 && K >= TK && encode_fn() != nullptr;
 }
+
+namespace {
+template <int EPI, int TN, int STAGES>
+cudaError_t gemm_tile(const __nv_bfloat16 *a, int M, int K, const __nv_bfloat16 *b, int N, const float *bias,
+                      const __nv_bfloat16 *mask, __nv_bfloat16 *out, int *err, cudaStream_t s) {
+  CUtensorMap ta, tb;
+  if (!make_map(&ta, a, M, K, TM) || !make_map(&tb, b, N, K, TN)) return cudaErrorInvalidValue;
+  const int smem = (int)sizeof(Smem<TN, STAGES>) + 1024;
+  // per-device attribute set-up is cheap; repeat it rather than cache per device
+  cudaError_t e = cudaFuncSetAttribute(gemm_tc05_kernel<EPI, TN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem);
+  if (e != cudaSuccess) return e;
+  gemm_tc05_kernel<EPI, TN, STAGES><<<dim3(N / TN, (M + TM - 1) / TM), 128, smem, s>>>(ta, tb, M, K, bias, mask, out,
+                                                                                     N, err);
+  return cudaGetLastError();
+}
+
+template <int EPI>
+cudaError_t gemm_rows(const __nv_bfloat16 *a, int M, int K, const __nv_bfloat16 *b, int N, const float *bias,
+                      const __nv_bfloat16 *mask, __nv_bfloat16 *out, int *err, cudaStream_t s) {
+  // widest tile that still gives about two thirds of the SMs a CTA
+  const int tiles = (M + TM - 1) / TM;
+  if (tiles * (N / 256) >= 96) return gemm_tile<EPI, 256, 3>(a, M, K, b, N, bias, mask, out, err, s);
+  if (tiles * (N / 64) >= 96) return gemm_tile<EPI, 64, 8>(a, M, K, b, N, bias, mask, out, err, s);
+  return gemm_tile<EPI, 32, 8>(a, M, K, b, N, bias, mask, out, err, s);
+}
+}  // namespace
 
 cudaError_t gemm_tc05(int epi, const __nv_bfloat16 *a, int M, int K, const __nv_bfloat16 *b, int N,
                       const float *bias, const __nv_bfloat16 *mask, __nv_bfloat16 *out, int *err,
@@ -280,22 +318,8 @@ cudaError_t gemm_tc05(int epi, const __nv_bfloat16 *a, int M, int K, const __nv_
   if (!tc05_supported(M, N, K) || (epi != EPI_BIAS_RELU && epi != EPI_RELU_MASK) ||
       (reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(out)) & 15)
     return cudaErrorInvalidValue;
-  CUtensorMap ta, tb;
-  if (!make_map(&ta, a, M, K, TM) || !make_map(&tb, b, N, K, TN)) return cudaErrorInvalidValue;
-  const int smem = (int)sizeof(Smem) + 1024;
-  // per-device attribute set-up is cheap; repeat it rather than cache per device
-  cudaError_t e = cudaFuncSetAttribute(gemm_tc05_kernel<EPI_BIAS_RELU>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(gemm_tc05_kernel<EPI_RELU_MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(N / TN, (M + TM - 1) / TM);
-  if (epi == EPI_BIAS_RELU)
-    gemm_tc05_kernel<EPI_BIAS_RELU><<<grid, 128, smem, s>>>(ta, tb, M, K, bias, nullptr, out, N, err);
-  else
-    gemm_tc05_kernel<EPI_RELU_MASK><<<grid, 128, smem, s>>>(ta, tb, M, K, nullptr, mask, out, N, err);
-  return cudaGetLastError();
+  return epi == EPI_BIAS_RELU ? gemm_rows<EPI_BIAS_RELU>(a, M, K, b, N, bias, nullptr, out, err, s)
+                              : gemm_rows<EPI_RELU_MASK>(a, M, K, b, N, nullptr, mask, out, err, s);
 }
 
 cudaError_t inject_skip_loads_once() {

@@ -184,7 +184,7 @@ mlp::GemmArgs fwd_args(const __nv_bfloat16 *in, int fan_in, const __nv_bfloat16 
                        __nv_bfloat16 *out, int rows) {
   mlp::GemmArgs a{};
   a.A = in; a.B = W; a.M = rows; a.N = F1; a.K = fan_in;
-  a.sAm = fan_in; a.sAk = 1; a.sBk = F1; a.sBn = 1;
+  a.sAm = fan_in; a.sBk = F1; a.sBn = 1;
   a.bias = b; a.Cb = out; a.ldc = F1;
   return a;
 }
@@ -206,35 +206,36 @@ cudaError_t forward_hidden(ligate_surrogate *s, int rows, cudaStream_t st) {
   return mlp::gemm(mlp::GEMM_FWD, fwd_args(s->h2, F1, s->wb + OW3, s->w + OB3, s->h3, rows), st);
 }
 
-// Backward from dz3 (set by the head kernel) into s->g.
+// Backward from dz3 (set by the head kernel) into s->g: the data gradients
+// down the layers, then every parameter gradient at once.
 cudaError_t backward(ligate_surrogate *s, int rows, cudaStream_t st) {
   cudaError_t e;
-  if ((e = mlp::head_grad(s->h3, s->dy, rows, s->g + OW4, s->g + OB4, st))) return e;
-  struct L { const __nv_bfloat16 *in; int fan_in; int ow, ob; __nv_bfloat16 *dz, *dz_prev; const __nv_bfloat16 *hin; };
-  const L layers[3] = {{s->h2, F1, OW3, OB3, s->dz3, s->dz2, s->h2},
-                       {s->h1, F1, OW2, OB2, s->dz2, s->dz1, s->h1},
-                       {s->x, F0, OW1, OB1, s->dz1, nullptr, nullptr}};
-  for (const L &l : layers) {
-    mlp::GemmArgs wg{};  // dW = in^T dZ
-    wg.A = l.in; wg.B = l.dz; wg.M = l.fan_in; wg.N = F1; wg.K = rows;
-    wg.sAm = 1; wg.sAk = l.fan_in; wg.sBk = F1; wg.sBn = 1;
-    wg.Cf = s->g + l.ow; wg.ldc = F1;
-    if ((e = mlp::gemm(mlp::GEMM_WGRAD, wg, st))) return e;
-    if ((e = mlp::colsum(l.dz, rows, F1, s->g + l.ob, st))) return e;
-    if (l.dz_prev) {  // dZ_prev = (dZ W^T) * (H_prev > 0)
+  struct L { int ow; const __nv_bfloat16 *dz; __nv_bfloat16 *dz_prev; const __nv_bfloat16 *hin; };
+  const L layers[2] = {{OW3, s->dz3, s->dz2, s->h2}, {OW2, s->dz2, s->dz1, s->h1}};
+  for (const L &l : layers) {  // dZ_prev = (dZ W^T) * (H_prev > 0)
+    if (s->tc05) {  // B[n][k] = W[n][k]: the row-major weights are already K-major here
+      e = mlp::gemm_tc05(mlp::EPI_RELU_MASK, l.dz, rows, F1, s->wb + l.ow, F1, nullptr, l.hin, l.dz_prev, s->err, st);
+    } else {
       mlp::GemmArgs dg{};
-      dg.A = l.dz; dg.B = s->wb + l.ow; dg.M = rows; dg.N = l.fan_in; dg.K = F1;
-      dg.sAm = F1; dg.sAk = 1; dg.sBk = 1; dg.sBn = F1;
-      dg.mask = l.hin; dg.Cb = l.dz_prev; dg.ldc = l.fan_in;
-      if (s->tc05)  // B[n][k] = W[n][k]: the row-major weights are already K-major here
-        e = mlp::gemm_tc05(mlp::EPI_RELU_MASK, l.dz, rows, F1, s->wb + l.ow, l.fan_in, nullptr, l.hin,
-                           l.dz_prev, s->err, st);
-      else
-        e = mlp::gemm(mlp::GEMM_DGRAD, dg, st);
-      if (e) return e;
+      dg.A = l.dz; dg.B = s->wb + l.ow; dg.M = rows; dg.N = F1; dg.K = F1;
+      dg.sAm = F1; dg.sBk = 1; dg.sBn = F1;
+      dg.mask = l.hin; dg.Cb = l.dz_prev; dg.ldc = F1;
+      e = mlp::gemm(mlp::GEMM_DGRAD, dg, st);
     }
+    if (e) return e;
   }
-  return cudaSuccess;
+  mlp::GradArgs a{};
+  const __nv_bfloat16 *in[3] = {s->x, s->h1, s->h2}, *dz[3] = {s->dz1, s->dz2, s->dz3};
+  const int ow[3] = {OW1, OW2, OW3}, ob[3] = {OB1, OB2, OB3};
+  for (int l = 0; l < 3; ++l) {
+    a.in[l] = in[l]; a.dz[l] = dz[l];
+    a.dw[l] = s->g + ow[l]; a.db[l] = s->g + ob[l];
+    a.fan_in[l] = l == 0 ? F0 : F1;
+  }
+  a.h3 = s->h3; a.dy = s->dy;
+  a.gw4 = s->g + OW4; a.gb4 = s->g + OB4;
+  a.rows = rows;
+  return mlp::grads(a, st);
 }
 
 }  // namespace
@@ -356,9 +357,8 @@ extern "C" ligate_status ligate_surrogate_train(ligate_surrogate *s, const float
           (e = mlp::head(s->h3, s->wb + OW4, s->w + OB4, batch, s->t, s->y, s->dy, 2.f / batch,
                          s->sse, s->dz3, st)) ||
           (e = backward(s, batch, st)) ||
-          (e = mlp::adam(s->w, s->g, s->m, s->v, s->wb, NPAR, lr, 0.9f, 0.999f, 1e-8f, (float)c1,
-                         (float)c2, st)) ||
-          (e = refresh_wt(s, st)))
+          (e = mlp::adam(s->w, s->g, s->m, s->v, s->wb, s->tc05 ? s->wt : nullptr, lr, 0.9f, 0.999f, 1e-8f, (float)c1,
+                         (float)c2, st)))
         return cuda_fail(e, "surrogate step");
     }
     double sse = 0.0;
