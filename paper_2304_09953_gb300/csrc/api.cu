@@ -967,7 +967,7 @@ struct ligate_plan {
   float *rot = nullptr, *anc = nullptr, *quat = nullptr;
   uint16_t *visit = nullptr;  // anchor visiting order (DockParams::visit)
   // scratch of ligate_plan_best_quantile (grown on demand): best scores,
-  // sort keys and sorted indices, q_cap entries each
+  // sort keys (two arrays) and sorted indices, q_cap entries each
   float *q_scores = nullptr;
   unsigned long long *q_keys = nullptr;
   int32_t *q_idx = nullptr;
@@ -1818,20 +1818,18 @@ extern "C" ligate_status ligate_plan_best_quantile(ligate_plan *pl, double frac,
   const int n = pl->rows;
   if (n == 0) { set_error("plan_best_quantile: the plan has no rows"); return LIGATE_ERR_INVALID; }
   const int k = std::min(n, std::max(1, (int)std::ceil(frac * n - 1e-9)));
-  int n2 = 2048;
-  while (n2 < n) n2 <<= 1;
   cudaError_t e = cudaSuccess;
-  if (pl->q_cap < n2) {  // grown once per size (allocates: not inside a capture)
+  if (pl->q_cap < n) {  // grown once per size (allocates: not inside a capture)
     cudaFree(pl->q_scores); cudaFree(pl->q_keys); cudaFree(pl->q_idx);
     pl->q_scores = nullptr; pl->q_keys = nullptr; pl->q_idx = nullptr; pl->q_cap = 0;
-    if ((e = dmalloc(&pl->q_scores, n2)) != cudaSuccess || (e = dmalloc(&pl->q_keys, n2)) != cudaSuccess ||
-        (e = dmalloc(&pl->q_idx, n2)) != cudaSuccess)
+    if ((e = dmalloc(&pl->q_scores, n)) != cudaSuccess || (e = dmalloc(&pl->q_keys, 2 * (size_t)n)) != cudaSuccess ||
+        (e = dmalloc(&pl->q_idx, n)) != cudaSuccess)
       return cuda_fail(e, "plan_best_quantile");
-    pl->q_cap = n2;
+    pl->q_cap = n;
   }
   cudaStream_t st = (cudaStream_t)stream;
   best_scores_kernel<<<(n + 255) / 256, 256, 0, st>>>(pl->out, n, pl->p.K, pl->q_scores, 1, 0);
-  if ((e = cudaGetLastError()) == cudaSuccess) e = mlp::sort_select(pl->q_scores, n, k, pl->q_keys, n2, pl->q_idx, st);
+  if ((e = cudaGetLastError()) == cudaSuccess) e = mlp::sort_select(pl->q_scores, n, k, pl->q_keys, pl->q_idx, st);
   if (e == cudaSuccess) {
     pick_value_kernel<<<1, 32, 0, st>>>(pl->q_scores, pl->q_idx, k, out);
     e = cudaGetLastError();

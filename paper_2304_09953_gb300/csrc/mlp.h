@@ -50,8 +50,9 @@ cudaError_t to_bf16(const float *a, __nv_bfloat16 *b, int n, cudaStream_t s);
 cudaError_t feature_stats(const float *desc, int n, float *mu, float *inv_sd, cudaStream_t s);
 cudaError_t label_stats(const float *y, int n, double *out, cudaStream_t s);
 cudaError_t unstd(float *y, int n, float mu, float sd, cudaStream_t s);
-cudaError_t sort_select(const float *pred, int n, int k, unsigned long long *keys, int n2,
-                        int32_t *idx, cudaStream_t s);
+// Indices of the k smallest of pred[n] in ascending (value, index) order (NaN
+// last) into idx; keys: scratch of 2 n entries.
+cudaError_t sort_select(const float *pred, int n, int k, unsigned long long *keys, int32_t *idx, cudaStream_t s);
 
 // tcgen05 path (mlp_tc05.cu) for K-major A [M][K] and B [N][K]:
 // C[M][N] = epi(A B^T), epi EPI_BIAS_RELU or EPI_RELU_MASK; needs N % 256 == 0,
@@ -61,6 +62,21 @@ bool tc05_supported(int M, int N, int K);
 cudaError_t gemm_tc05(int epi, const __nv_bfloat16 *a, int M, int K, const __nv_bfloat16 *b, int N,
                       const float *bias, const __nv_bfloat16 *mask, __nv_bfloat16 *out, int *err,
                       cudaStream_t s);
+// Inference of n_nets networks on desc [n][256] (FP32) in one launch per
+// FWD_NETS networks: predictions in label units into pred [n] of each.
+constexpr int FWD_NETS = 8;
+struct FwdSpec {
+  const __nv_bfloat16 *wt[3];  // transposed hidden weights, 16-byte aligned
+  const float *b[3];           // 16-byte aligned
+  const __nv_bfloat16 *w4;
+  const float *b4, *mu, *inv_sd;
+  float ly_mu, ly_sd;
+  float *pred;
+  int *err;
+};
+cudaError_t forward_tc05(const FwdSpec *nets, int n_nets, const float *desc, int n, cudaStream_t s);
+// mean[i] = sum_m (1 / n_nets) pred[m][i], accumulated in network order.
+cudaError_t mean_pred(const float *pred, int n_nets, int n, float *mean, cudaStream_t s);
 // Test hook: the next CTA of a tcgen05 contraction issues no loads, so its
 // bounded wait runs out (err set, LIGATE_ERR_TIMEOUT at the next check).
 cudaError_t inject_skip_loads_once();

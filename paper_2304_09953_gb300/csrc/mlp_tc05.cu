@@ -245,6 +245,251 @@ __global__ void __launch_bounds__(128, 1)
                  : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// The whole network on 128 rows per CTA: standardised inputs, three hidden
+// layers and the head, activations in shared memory, nothing but the rows'
+// descriptors read and 4 bytes per row written.
+//
+// What bounds it: the hidden weights (1.3 MB in BF16) pass through every CTA
+// once per 128 rows, from L2 (about 0.17 GFLOP of tcgen05 work per tile against
+// them); as layers of their own, each with a descriptor or activation pass
+// through memory, the same rows took gather + 3 GEMM + head + unscale launches
+// and 2 x 6 KB of activations per row: 100,000 rows 590 us (serialised), here
+// 240, 40 us per tile of which the weight tiles' way from L2 (8 TB/s over all
+// SMs) is about two thirds.
+//
+// A CTA keeps the layer input as eight 64-column K slices in the 128-byte
+// swizzle the tensor core reads (128 KB) and streams the transposed weights as
+// 256 x 64 tiles through a three-stage ring; the 128 x 512 FP32 accumulator is
+// the SM's whole tensor memory.  Warp 8 issues loads and MMAs; warps 0-7 write
+// the inputs, then per layer read their 32 rows x 256 columns of the
+// accumulator, add the bias, apply ReLU and write the next layer's slices in
+// place (the MMAs that read them are done).  Weight tiles of the next layer are
+// already in flight during an epilogue.  Every output is the same bits as the
+// layer-by-layer kernels': the same K order, rounding points, and head order
+// (column l of each group of 32 in one chain, then the butterfly's tree).
+constexpr int FW_THREADS = 288, FW_STAGES = 3, FW_B = 256 * TK * 2;
+
+struct FwdNet {
+  CUtensorMap w[3];  // transposed hidden weights [512][256], [512][512], [512][512]
+  const float *b[3];
+  const __nv_bfloat16 *w4;
+  const float *b4, *mu, *inv_sd;
+  float ly_mu, ly_sd;
+  float *pred;
+  int *err;
+};
+struct FwdArgs {
+  FwdNet net[FWD_NETS];
+  const float *desc;
+  int n, tiles, items, vec;  // rows, row tiles, tiles x networks, desc rows 16-byte aligned
+};
+struct __align__(1024) FwdSmem {
+  uint8_t h[8][A_BYTES];
+  uint8_t ring[FW_STAGES][FW_B];
+  __nv_bfloat16 w4[512];
+  uint64_t full[FW_STAGES], empty[FW_STAGES], done;
+  uint32_t tmem_base;
+};
+static_assert(sizeof(FwdSmem) + 1024 <= 227 * 1024, "one CTA's shared memory");
+
+__device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t addr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
+      "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t addr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+__global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid_constant__ FwdArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  FwdSmem &s = *reinterpret_cast<FwdSmem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool issuer = tid == 256;
+  if (tid == 0) {
+    for (int i = 0; i < FW_STAGES; ++i) { mbar_init(&s.full[i], 1); mbar_init(&s.empty[i], 1); }
+    mbar_init(&s.done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 8) {  // the whole tensor memory: 512 columns
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(saddr(&s.tmem_base))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = s.tmem_base;
+  const bool skip_loads = issuer && atomicExch(&g_fault_skip_loads, 0) != 0;  // test hook (see gemm_tc05_kernel)
+
+  bool ok = true;
+  int loaded = 0, used = 0;   // issuer: weight tiles loaded and consumed so far
+  unsigned done_phase = 0;
+  for (int item = blockIdx.x; item < a.items && ok; item += gridDim.x) {
+    const FwdNet &net = a.net[item / a.tiles];
+    const int row0 = item % a.tiles * TM;
+    const int first = used;  // this tile's weight tiles are first .. first + 39
+    // weight tile q of the row tile: layer, 64-wide K slice, 256-column half
+    auto load = [&](int q) {
+      const int l = q < 8 ? 0 : q < 24 ? 1 : 2, r = q - (l == 0 ? 0 : l == 1 ? 8 : 24), st = loaded % FW_STAGES;
+      if (loaded >= FW_STAGES && !mbar_wait(&s.empty[st], (loaded / FW_STAGES - 1) & 1u)) { ok = false; return; }
+      if (skip_loads) return;
+      mbar_expect_tx(&s.full[st], FW_B);
+      tma_load_2d(s.ring[st], &net.w[l], &s.full[st], (r >> 1) * TK, (r & 1) * 256);
+      ++loaded;
+    };
+    if (issuer)
+      while (ok && !skip_loads && loaded < first + FW_STAGES) load(loaded - first);
+    if (warp < 8) {  // standardised inputs into slices 0-3: a warp per row, eight columns per lane
+      float mu[8], sd[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) { mu[q] = __ldg(net.mu + 8 * lane + q); sd[q] = __ldg(net.inv_sd + 8 * lane + q); }
+      uint8_t *const slice = s.h[lane >> 3];
+#pragma unroll 4
+      for (int i = 0; i < TM / 8; ++i) {
+        const int r = warp + 8 * i;
+        float v[8];
+        if (row0 + r < a.n) {
+          const float *src = a.desc + (size_t)(row0 + r) * 256 + 8 * lane;
+          if (a.vec) {
+            const float4 x = __ldg(reinterpret_cast<const float4 *>(src)), y = __ldg(reinterpret_cast<const float4 *>(src) + 1);
+            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+          } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = __ldg(src + q);
+          }
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = (v[q] - mu[q]) * sd[q];
+        } else {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = 0.f;
+        }
+        *reinterpret_cast<uint4 *>(slice + r * 128 + (((lane & 7) ^ (r & 7)) << 4)) =
+            make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+      }
+      s.w4[tid] = net.w4[tid];
+      s.w4[256 + tid] = net.w4[256 + tid];
+      if (item + (int)gridDim.x < a.items) {  // the next tile's rows towards L2
+        const int nrow = (item + (int)gridDim.x) % a.tiles * TM;
+        for (int q = tid; q < TM * 8; q += 256)
+          if (nrow + (q >> 3) < a.n)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(a.desc + (size_t)(nrow + (q >> 3)) * 256 + (q & 7) * 32));
+      }
+    }
+    for (int l = 0; l < 3; ++l) {
+      // the layer's input is written (and the accumulator read): visible to
+      // the tensor core's proxy, then one thread issues the layer
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      if (!__syncthreads_and(ok)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (issuer) {
+        const int slices = l == 0 ? 4 : 8;
+        for (int kb = 0; kb < slices && ok; ++kb)
+          for (int nh = 0; nh < 2 && ok; ++nh) {
+            const int st = used % FW_STAGES;
+            if (!mbar_wait(&s.full[st], (used / FW_STAGES) & 1u)) { ok = false; break; }
+            ++used;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t da = sdesc(saddr(s.h[kb])), db = sdesc(saddr(s.ring[st]));
+#pragma unroll
+            for (int kk = 0; kk < TK / 16; ++kk)
+              mma_f16<256>(tmem + nh * 256, da + 2 * kk, db + 2 * kk, (kb > 0 || kk > 0) ? 1u : 0u);
+            mma_commit(&s.empty[st]);
+            // two tiles ahead: the stage of the previous step, whose MMAs run before this one's
+            while (ok && loaded < first + 40 && loaded < used + FW_STAGES - 1) load(loaded - first);
+          }
+        mma_commit(&s.done);  // arrives once every MMA issued so far has completed
+      }
+      if (warp < 8) {
+        const int row = (warp & 3) * 32 + lane, half = warp >> 2;
+        const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        ok = __all_sync(0xffffffffu, mbar_wait(&s.done, done_phase)) && ok;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (l < 2) {
+          const float *bias = net.b[l] + half * 256;
+#pragma unroll 1
+          for (int c0 = 0; c0 < 256 && ok; c0 += 32) {
+            uint32_t r[32];
+            tmem_ld32(r, trow + half * 256 + c0);
+            uint8_t *const slice = s.h[half * 4 + (c0 >> 6)] + row * 128;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float4 b0 = __ldg(reinterpret_cast<const float4 *>(bias + c0 + 8 * q)),
+                           b1 = __ldg(reinterpret_cast<const float4 *>(bias + c0 + 8 * q) + 1);
+              const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+              float v[8];
+#pragma unroll
+              for (int k = 0; k < 8; ++k) v[k] = fmaxf(__uint_as_float(r[8 * q + k]) + bb[k], 0.f);
+              *reinterpret_cast<uint4 *>(slice + (((((c0 & 32) >> 3) + q) ^ (row & 7)) << 4)) =
+                  make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+            }
+          }
+        } else {
+          // head: chain c of 32 sums the columns c, c + 32, ...; this warp has
+          // chains 16 half .. 16 half + 15 of its rows
+          float acc[16];
+#pragma unroll
+          for (int c = 0; c < 16; ++c) acc[c] = 0.f;
+          const float *bias = net.b[2] + 16 * half;
+          const __nv_bfloat16 *w4 = s.w4 + 16 * half;
+#pragma unroll 1
+          for (int j = 0; j < 512 && ok; j += 32) {
+            uint32_t r[16];
+            tmem_ld16(r, trow + j + 16 * half);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+              const float h = __bfloat162float(__float2bfloat16_rn(fmaxf(__uint_as_float(r[c]) + __ldg(bias + j + c), 0.f)));
+              acc[c] = fmaf(h, __bfloat162float(w4[j + c]), acc[c]);
+            }
+          }
+          // the butterfly's tree: lanes 16 apart first, which are the two
+          // warps' chains (through slices 4-7, which no one reads any more)
+          float *const xch = reinterpret_cast<float *>(s.h[4]) + row;
+          if (half == 1)
+#pragma unroll
+            for (int c = 0; c < 16; ++c) xch[c * TM] = acc[c];
+          asm volatile("bar.sync 1, 256;" ::: "memory");
+          if (half == 0) {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) acc[c] += xch[c * TM];
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+              for (int c = 0; c < o; ++c) acc[c] += acc[c + o];
+            if (row0 + row < a.n && ok) net.pred[row0 + row] = fmaf(acc[0] + __ldg(net.b4), net.ly_sd, net.ly_mu);
+          }
+        }
+      }
+      done_phase ^= 1u;
+    }
+    ok = __syncthreads_and(ok);  // the same decision in every thread; the tile's shared memory is free
+    if (!ok && tid == 0) atomicExch(net.err, 1);
+  }
+  if (issuer && !ok)  // drain loads still in flight (bounded) before the shared memory goes
+    for (int q = used; q < loaded; ++q) (void)mbar_wait(&s.full[q % FW_STAGES], (q / FW_STAGES) & 1u);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 8)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link
 // against the driver library).
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
@@ -320,6 +565,41 @@ cudaError_t gemm_tc05(int epi, const __nv_bfloat16 *a, int M, int K, const __nv_
     return cudaErrorInvalidValue;
   return epi == EPI_BIAS_RELU ? gemm_rows<EPI_BIAS_RELU>(a, M, K, b, N, bias, nullptr, out, err, s)
                               : gemm_rows<EPI_RELU_MASK>(a, M, K, b, N, nullptr, mask, out, err, s);
+}
+
+cudaError_t forward_tc05(const FwdSpec *nets, int n_nets, const float *desc, int n, cudaStream_t s) {
+  if (n <= 0 || n_nets <= 0) return cudaSuccess;
+  int dev = 0, sms = 0;
+  cudaError_t e;
+  const int smem = (int)sizeof(FwdSmem) + 1024;
+  if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
+      (e = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
+    return e;
+  for (int m0 = 0; m0 < n_nets; m0 += FWD_NETS) {
+    const int m = n_nets - m0 < FWD_NETS ? n_nets - m0 : FWD_NETS;
+    FwdArgs a;
+    for (int q = 0; q < m; ++q) {
+      const FwdSpec &f = nets[m0 + q];
+      FwdNet &t = a.net[q];
+      const int K[3] = {256, 512, 512};
+      for (int l = 0; l < 3; ++l) {
+        if (!make_map(&t.w[l], f.wt[l], 512, K[l], 256)) return cudaErrorInvalidValue;
+        t.b[l] = f.b[l];
+      }
+      t.w4 = f.w4; t.b4 = f.b4; t.mu = f.mu; t.inv_sd = f.inv_sd;
+      t.ly_mu = f.ly_mu; t.ly_sd = f.ly_sd;
+      t.pred = f.pred; t.err = f.err;
+    }
+    for (int q = m; q < FWD_NETS; ++q) a.net[q] = a.net[0];
+    a.desc = desc;
+    a.n = n;
+    a.tiles = (n + TM - 1) / TM;
+    a.items = a.tiles * m;
+    a.vec = (reinterpret_cast<uintptr_t>(desc) & 15) == 0;
+    mlp_forward_kernel<<<a.items < sms ? a.items : sms, FW_THREADS, smem, s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t inject_skip_loads_once() {

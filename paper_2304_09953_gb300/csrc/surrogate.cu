@@ -19,27 +19,45 @@ namespace ligate {
 // (8 bins, edges (1.5 k) A, k = 1..7; the bin is decided on d^2 computed in
 // FP32 as (dx*dx + dy*dy) + dz*dz without contraction, against the exactly
 // representable squared edges), rotatable-bond count; log1p of every count.
-__global__ void descriptor_kernel(const LigDesc *__restrict__ lig, const float4 *__restrict__ atoms,
-                                  int n_ligands, float *__restrict__ out) {
+//
+// What bounds it: 1 KB written per ligand (15 us per 100,000 at the copy rate)
+// against 700 pair tests and shared-memory increments of a 38-atom ligand.
+// The pairs are enumerated with a running (row, column) over folded rows (row r
+// and row n - 2 - r of the triangle together have n pairs) instead of decoding
+// every pair index from the start, atoms come from shared memory, and log1p of
+// the small counts comes from a table made by the same function: 100,000
+// ligands 409 -> 218 us (serialised), bound by instruction issue.
+constexpr int DESC_LOGS = 64;
+__global__ void __launch_bounds__(256) descriptor_kernel(const LigDesc *__restrict__ lig,
+                                                         const float4 *__restrict__ atoms, int n_ligands,
+                                                         float *__restrict__ out) {
   __shared__ unsigned int hist[8][28 * 8 + 8];
+  __shared__ float4 xyz[8][LIGATE_MAX_ATOMS];
+  __shared__ float logs[DESC_LOGS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int li = blockIdx.x * (blockDim.x >> 5) + warp;
   unsigned int *h = hist[warp];
+  float4 *a = xyz[warp];
+  if (threadIdx.x < DESC_LOGS) logs[threadIdx.x] = log1pf((float)threadIdx.x);
   for (int q = lane; q < 28 * 8 + 8; q += 32) h[q] = 0;
+  __syncthreads();
+  if (li >= n_ligands) return;
+  const int base = lig[li].atom_base, n = lig[li].n_atoms, nrot = lig[li].n_rot;
+  for (int i = lane; i < n; i += 32) {
+    const float4 v = __ldg(atoms + base + i);
+    a[i] = v;
+    atomicAdd(&h[224 + __float_as_int(v.w)], 1u);
+  }
   __syncwarp();
-  if (li < n_ligands) {
-    const LigDesc d = lig[li];
-    const float4 *a = atoms + d.atom_base;
-    for (int i = lane; i < d.n_atoms; i += 32) atomicAdd(&h[224 + __float_as_int(a[i].w)], 1u);
-    const int npairs = d.n_atoms * (d.n_atoms - 1) / 2;
-    for (int q = lane; q < npairs; q += 32) {
-      // pair index q -> (i, j), i < j, row-major over the upper triangle
-      int i = 0, rem = q, row = d.n_atoms - 1;
-      while (rem >= row) { rem -= row; ++i; --row; }
-      const int j = i + 1 + rem;
-      const float4 x = a[i], y = a[j];
-      int ta = __float_as_int(x.w), tb = __float_as_int(y.w);
-      if (ta == tb) continue;
+  const int npairs = n * (n - 1) / 2;
+  int r = 0, c = lane;
+  while (c >= n) { c -= n; ++r; }
+  for (int q = lane; q < npairs; q += 32) {
+    const int up = n - 1 - r;  // pairs of row r; the rest of the folded row is row n - 2 - r
+    const int i = c < up ? r : n - 2 - r, j = c < up ? r + 1 + c : n - 1 - r + c - up;
+    const float4 x = a[i], y = a[j];
+    int ta = __float_as_int(x.w), tb = __float_as_int(y.w);
+    if (ta != tb) {
       if (ta > tb) { const int t = ta; ta = tb; tb = t; }
       const int p = ta * 8 - ta * (ta + 1) / 2 + (tb - ta - 1);
       const float dx = __fsub_rn(x.x, y.x), dy = __fsub_rn(x.y, y.y), dz = __fsub_rn(x.z, y.z);
@@ -49,18 +67,14 @@ __global__ void descriptor_kernel(const LigDesc *__restrict__ lig, const float4 
       bin += d2 >= 56.25f; bin += d2 >= 81.0f; bin += d2 >= 110.25f;
       atomicAdd(&h[p * 8 + bin], 1u);
     }
+    c += 32;
+    while (c >= n) { c -= n; ++r; }
   }
   __syncwarp();
-  if (li < n_ligands) {
-    float *o = out + (size_t)li * 256;
-    const int nrot = lig[li].n_rot;
-    for (int q = lane; q < 256; q += 32) {
-      float v = 0.f;
-      if (q < 8) v = log1pf((float)h[224 + q]);
-      else if (q < 232) v = log1pf((float)h[q - 8]);
-      else if (q == 232) v = log1pf((float)nrot);
-      o[q] = v;
-    }
+  float *o = out + (size_t)li * 256;
+  for (int q = lane; q < 256; q += 32) {
+    const unsigned cnt = q < 8 ? h[224 + q] : q < 232 ? h[q - 8] : q == 232 ? (unsigned)nrot : 0u;
+    o[q] = cnt < DESC_LOGS ? logs[cnt] : log1pf((float)cnt);
   }
 }
 
@@ -122,6 +136,8 @@ struct ligate_surrogate {
   bool tc05 = false;
   __nv_bfloat16 *wt = nullptr;
   int *err = nullptr;
+  unsigned char *rank_ws = nullptr;  // scratch of rankings (ensure_rank)
+  size_t rank_cap = 0;
 };
 
 namespace {
@@ -204,6 +220,33 @@ cudaError_t forward_hidden(ligate_surrogate *s, int rows, cudaStream_t st) {
   if ((e = mlp::gemm(mlp::GEMM_FWD, fwd_args(s->x, F0, s->wb + OW1, s->w + OB1, s->h1, rows), st))) return e;
   if ((e = mlp::gemm(mlp::GEMM_FWD, fwd_args(s->h1, F1, s->wb + OW2, s->w + OB2, s->h2, rows), st))) return e;
   return mlp::gemm(mlp::GEMM_FWD, fwd_args(s->h2, F1, s->wb + OW3, s->w + OB3, s->h3, rows), st);
+}
+
+mlp::FwdSpec fwd_spec(const ligate_surrogate *s, float *pred) {
+  mlp::FwdSpec f{};
+  f.wt[0] = s->wt + TW1; f.wt[1] = s->wt + TW2; f.wt[2] = s->wt + TW3;
+  f.b[0] = s->w + OB1; f.b[1] = s->w + OB2; f.b[2] = s->w + OB3;
+  f.w4 = s->wb + OW4; f.b4 = s->w + OB4;
+  f.mu = s->mu; f.inv_sd = s->inv_sd;
+  f.ly_mu = (float)s->label_mu; f.ly_sd = (float)s->label_sd;
+  f.pred = pred; f.err = s->err;
+  return f;
+}
+
+// Scratch of a ranking: n_nets + 1 prediction arrays of n, then the sort's
+// keys; kept with the network and grown on demand.
+cudaError_t ensure_rank(ligate_surrogate *s, int n, int n_nets, float **pred, unsigned long long **keys) {
+  const size_t pb = ((size_t)n * (n_nets + 1) * 4 + 15) / 16 * 16, need = pb + (size_t)n * 16;
+  if (need > s->rank_cap) {
+    cudaFree(s->rank_ws);
+    s->rank_ws = nullptr;
+    s->rank_cap = 0;
+    if (cudaError_t e = cudaMalloc(&s->rank_ws, need)) return e;
+    s->rank_cap = need;
+  }
+  *pred = reinterpret_cast<float *>(s->rank_ws);
+  *keys = reinterpret_cast<unsigned long long *>(s->rank_ws + pb);
+  return cudaSuccess;
 }
 
 // Backward from dz3 (set by the head kernel) into s->g: the data gradients
@@ -300,7 +343,7 @@ extern "C" void ligate_surrogate_destroy(ligate_surrogate *s) {
   free_work(s);
   cudaFree(s->w); cudaFree(s->m); cudaFree(s->v); cudaFree(s->g); cudaFree(s->wb);
   cudaFree(s->mu); cudaFree(s->inv_sd); cudaFree(s->lstat); cudaFree(s->sse); cudaFree(s->idx);
-  cudaFree(s->wt); cudaFree(s->err);
+  cudaFree(s->wt); cudaFree(s->err); cudaFree(s->rank_ws);
   delete s;
 }
 
@@ -393,15 +436,15 @@ extern "C" ligate_status ligate_surrogate_grad(const ligate_surrogate *cs, const
   return LIGATE_OK;
 }
 
-extern "C" ligate_status ligate_surrogate_predict(const ligate_surrogate *cs, const float *desc, int n,
-                                                  float *pred, void *stream) {
-  NvtxRange nvtx_("ligate:surrogate_predict");
-  ligate_surrogate *s = const_cast<ligate_surrogate *>(cs);
-  if (!s || (n > 0 && (!desc || !pred)) || n < 0) { set_error("surrogate_predict: bad argument"); return LIGATE_ERR_INVALID; }
-  cudaStream_t st = (cudaStream_t)stream;
+// Predictions of the network on desc [n][256] into pred [n] (enqueues).
+static cudaError_t predict_enqueue(ligate_surrogate *s, const float *desc, int n, float *pred, cudaStream_t st) {
+  if (s->tc05) {
+    const mlp::FwdSpec f = fwd_spec(s, pred);
+    return mlp::forward_tc05(&f, 1, desc, n, st);
+  }
   const int chunk = 32768;
   cudaError_t e;
-  if ((e = ensure_work(s, n < chunk ? (n > 0 ? n : 1) : chunk))) return cuda_fail(e, "surrogate workspace");
+  if ((e = ensure_work(s, n < chunk ? (n > 0 ? n : 1) : chunk))) return e;
   for (int r0 = 0; r0 < n; r0 += chunk) {
     const int rows = n - r0 < chunk ? n - r0 : chunk;
     if ((e = mlp::gather_std(desc, nullptr, rows, r0, s->mu, s->inv_sd, nullptr, 0.f, 0.f, s->x, nullptr, st)) ||
@@ -409,9 +452,54 @@ extern "C" ligate_status ligate_surrogate_predict(const ligate_surrogate *cs, co
         (e = mlp::head(s->h3, s->wb + OW4, s->w + OB4, rows, nullptr, pred + r0, nullptr, 0.f, nullptr,
                        nullptr, st)) ||
         (e = mlp::unstd(pred + r0, rows, (float)s->label_mu, (float)s->label_sd, st)))
-      return cuda_fail(e, "surrogate_predict");
+      return e;
   }
+  return cudaSuccess;
+}
+
+extern "C" ligate_status ligate_surrogate_predict(const ligate_surrogate *cs, const float *desc, int n,
+                                                  float *pred, void *stream) {
+  NvtxRange nvtx_("ligate:surrogate_predict");
+  ligate_surrogate *s = const_cast<ligate_surrogate *>(cs);
+  if (!s || (n > 0 && (!desc || !pred)) || n < 0) { set_error("surrogate_predict: bad argument"); return LIGATE_ERR_INVALID; }
+  cudaStream_t st = (cudaStream_t)stream;
+  if (n == 0) return LIGATE_OK;
+  if (cudaError_t e = predict_enqueue(s, desc, n, pred, st)) return cuda_fail(e, "surrogate_predict");
   return check_err(s, st, "surrogate_predict");
+}
+
+// Ranking by the mean prediction of the networks (a single network: its own):
+// all tcgen05 networks run in one launch, the scratch is the first network's.
+static ligate_status rank_nets(const ligate_surrogate *const *nets, int n_nets, const float *desc, int n,
+                               double keep_frac, int32_t *idx_out, float *pred_out, void *stream, const char *what) {
+  cudaStream_t st = (cudaStream_t)stream;
+  const int k = (int)ceil((double)n * keep_frac - 1e-9);
+  float *each = nullptr;
+  unsigned long long *keys = nullptr;
+  cudaError_t e = ensure_rank(const_cast<ligate_surrogate *>(nets[0]), n, n_nets, &each, &keys);
+  if (e) return cuda_fail(e, what);
+  float *const mean = pred_out ? pred_out : each + (size_t)n_nets * n;
+  bool all_tc05 = true;
+  for (int m = 0; m < n_nets; ++m) all_tc05 &= nets[m]->tc05;
+  std::vector<mlp::FwdSpec> spec;
+  for (int m = 0; m < n_nets && !e; ++m) {
+    float *const p = n_nets == 1 ? mean : each + (size_t)m * n;
+    if (all_tc05) {
+      spec.push_back(fwd_spec(nets[m], p));
+      spec.back().err = nets[0]->err;  // one launch, one flag to read
+    }
+    else {
+      e = predict_enqueue(const_cast<ligate_surrogate *>(nets[m]), desc, n, p, st);
+    }
+  }
+  if (!e && all_tc05) e = mlp::forward_tc05(spec.data(), n_nets, desc, n, st);
+  if (!e && n_nets > 1) e = mlp::mean_pred(each, n_nets, n, mean, st);
+  if (!e) e = mlp::sort_select(mean, n, k, keys, idx_out, st);
+  if (e) return cuda_fail(e, what);
+  for (int m = 0; m < (all_tc05 ? 1 : n_nets); ++m)
+    if (ligate_status r = check_err(const_cast<ligate_surrogate *>(nets[m]), st, what)) return r;
+  if ((e = cudaStreamSynchronize(st))) return cuda_fail(e, what);
+  return LIGATE_OK;
 }
 
 extern "C" ligate_status ligate_surrogate_rank(const ligate_surrogate *s, const float *desc, int n,
@@ -423,35 +511,8 @@ extern "C" ligate_status ligate_surrogate_rank(const ligate_surrogate *s, const 
     return LIGATE_ERR_INVALID;
   }
   if (n == 0) return LIGATE_OK;
-  cudaStream_t st = (cudaStream_t)stream;
-  const int k = (int)ceil((double)n * keep_frac - 1e-9);
-  int n2 = 2048;
-  while (n2 < n) n2 <<= 1;
-  float *pred = pred_out;
-  unsigned long long *keys = nullptr;
-  cudaError_t e = cudaSuccess;
-  if (!pred && (e = cudaMalloc(&pred, (size_t)n * 4))) return cuda_fail(e, "surrogate_rank");
-  if ((e = cudaMalloc(&keys, (size_t)n2 * 8))) {
-    if (!pred_out) cudaFree(pred);
-    return cuda_fail(e, "surrogate_rank");
-  }
-  ligate_status r = ligate_surrogate_predict(s, desc, n, pred, stream);
-  if (r == LIGATE_OK) {
-    e = mlp::sort_select(pred, n, k, keys, n2, idx_out, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) r = cuda_fail(e, "surrogate_rank");
-  }
-  cudaFree(keys);
-  if (!pred_out) cudaFree(pred);
-  return r;
+  return rank_nets(&s, 1, desc, n, keep_frac, idx_out, pred_out, stream, "surrogate_rank");
 }
-
-namespace {
-__global__ void axpy_kernel(float *__restrict__ acc, const float *__restrict__ x, int n, float a, int first) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) acc[i] = first ? a * x[i] : fmaf(a, x[i], acc[i]);
-}
-}  // namespace
 
 extern "C" ligate_status ligate_surrogate_rank_ensemble(const ligate_surrogate *const *nets, int n_nets,
                                                         const float *desc, int n, double keep_frac,
@@ -464,34 +525,7 @@ extern "C" ligate_status ligate_surrogate_rank_ensemble(const ligate_surrogate *
   for (int m = 0; m < n_nets; ++m)
     if (!nets[m]) { set_error("surrogate_rank_ensemble: network %d is NULL", m); return LIGATE_ERR_INVALID; }
   if (n == 0) return LIGATE_OK;
-  cudaStream_t st = (cudaStream_t)stream;
-  const int k = (int)ceil((double)n * keep_frac - 1e-9);
-  int n2 = 2048;
-  while (n2 < n) n2 <<= 1;
-  float *mean = pred_out, *one = nullptr;
-  unsigned long long *keys = nullptr;
-  cudaError_t e = cudaSuccess;
-  ligate_status r = LIGATE_OK;
-  if ((!pred_out && (e = cudaMalloc(&mean, (size_t)n * 4))) || (e = cudaMalloc(&one, (size_t)n * 4)) ||
-      (e = cudaMalloc(&keys, (size_t)n2 * 8))) {
-    r = cuda_fail(e, "surrogate_rank_ensemble");
-  }
-  // mean = sum_m (1 / n_nets) pred_m, accumulated in network order
-  for (int m = 0; m < n_nets && r == LIGATE_OK; ++m) {
-    r = ligate_surrogate_predict(nets[m], desc, n, one, stream);
-    if (r != LIGATE_OK) break;
-    axpy_kernel<<<(n + 255) / 256, 256, 0, st>>>(mean, one, n, 1.f / (float)n_nets, m == 0);
-    if ((e = cudaGetLastError()) != cudaSuccess) r = cuda_fail(e, "surrogate_rank_ensemble");
-  }
-  if (r == LIGATE_OK) {
-    e = mlp::sort_select(mean, n, k, keys, n2, idx_out, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) r = cuda_fail(e, "surrogate_rank_ensemble");
-  }
-  cudaFree(keys);
-  cudaFree(one);
-  if (!pred_out) cudaFree(mean);
-  return r;
+  return rank_nets(nets, n_nets, desc, n, keep_frac, idx_out, pred_out, stream, "surrogate_rank_ensemble");
 }
 
 extern "C" ligate_status ligate_surrogate_get_weights(const ligate_surrogate *s, float *out) {
