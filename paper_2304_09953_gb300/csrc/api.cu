@@ -906,6 +906,7 @@ ligate_status base_params(const ligate_pocket *P, const ligate_batch *B, const l
   p.n_ligands = B->d.n_ligands;
   p.maps = mode_maps(d, mode);
   p.maps_f32 = d.map_f32;
+  p.maps_f32c = reinterpret_cast<const float4 *>(d.map_f32c);
   p.g.nx = d.nx; p.g.ny = d.ny; p.g.nz = d.nz;
   p.g.fx1 = (float)(d.nx - 1); p.g.fy1 = (float)(d.ny - 1); p.g.fz1 = (float)(d.nz - 1);
   p.g.penalty = s->penalty;

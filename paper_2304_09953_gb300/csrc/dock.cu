@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(256) score_poses_kernel(const DockParams p, in
     if (lane == 0) out[pi] = __int_as_float(0x7fc00000);
     return;
   }
-  LigDesc d;
-  (void)load_ligand(p, w, li, d, lane);
+  const LigDesc d = p.lig[li];
+  load_coords(p, w, d, lane);
   uint32_t tt[4];
   for (int q = 0; q < 4; ++q) {
     const uint8_t *t = tors + (size_t)pi * LIGATE_MAX_ROT + 4 * q;
@@ -109,8 +109,8 @@ __global__ void __launch_bounds__(256) pose_coords_kernel(const DockParams p, co
     for (int q = lane; q < LIGATE_MAX_ATOMS * 3; q += 32) o[q] = __int_as_float(0x7fc00000);
     return;
   }
-  LigDesc d;
-  (void)load_ligand(p, w, li, d, lane);
+  const LigDesc d = p.lig[li];
+  load_coords(p, w, d, lane);
   uint32_t tt[4];
   for (int q = 0; q < 4; ++q) {
     const uint8_t *t = tors + (size_t)pi * LIGATE_MAX_ROT + 4 * q;

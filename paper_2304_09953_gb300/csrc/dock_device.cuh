@@ -368,6 +368,37 @@ __device__ __forceinline__ void load_coords(const DockParams &p, const WarpSmem 
   __syncwarp();
 }
 
+// This lane's part of the clash sum (without the weight) of coordinates x of
+// the loaded ligand: the pairs of its own atoms lane, lane + 32, ... with
+// later atoms, at least 4 bonds apart.  The lanes step through the partners
+// together (a broadcast read, the lane's own eligibility bit) instead of each
+// through its own bit list: the same terms in the same order (a pair that does
+// not touch adds an exact zero), 11 instructions per partner for 32 pairs.
+__device__ __forceinline__ float clash_pairs(const DockParams &p, const float4 *x, const LigDesc &d, float inv_dc2,
+                                             int lane) {
+  float cl = 0.f;
+  for (int h0 = 0; h0 < d.n_atoms; h0 += 32) {
+    const int i = h0 + lane;
+    const bool own = i < d.n_atoms;
+    const float4 xi = own ? x[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int wd = h0 >> 5; wd < d.n_words; ++wd) {
+      uint32_t m = own ? __ldg(p.elig + d.elig_base + i * d.n_words + wd) : 0u;
+      const int lo = i + 1 - 32 * wd;  // keep only j > i
+      if (lo >= 32) m = 0; else if (lo > 0) m &= ~0u << lo;
+      if (!__any_sync(FULL, m != 0u)) continue;
+      const int jn = min(32, d.n_atoms - 32 * wd);
+      for (int b = 0; b < jn; ++b) {
+        const float4 xj = x[32 * wd + b];
+        const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
+        const float t = fmaxf(0.f, fmaf(-fmaf(dx, dx, fmaf(dy, dy, dz * dz)), inv_dc2, 1.f));
+        const float te = m >> b & 1u ? t : 0.f;
+        cl = fmaf(te, te, cl);
+      }
+    }
+  }
+  return cl;
+}
+
 // Load ligand `li` into the warp's slot: load_coords and the clash sum
 // (without the weight) of the input conformation, which every pose shares up
 // to the torsion-dependent part.
@@ -375,23 +406,7 @@ __device__ inline float load_ligand(const DockParams &p, const WarpSmem &w, int 
                              int lane) {
   d = p.lig[li];
   load_coords(p, w, d, lane);
-  float cl = 0.f;
-  for (int i = lane; i < d.n_atoms; i += 32) {
-    const float4 xi = w.ref[i];
-    for (int wd = 0; wd < d.n_words; ++wd) {
-      uint32_t m = __ldg(p.elig + d.elig_base + i * d.n_words + wd);
-      const int lo = i + 1 - 32 * wd;  // keep only j > i
-      if (lo >= 32) m = 0; else if (lo > 0) m &= ~0u << lo;
-      while (m) {
-        const int j = 32 * wd + __ffs(m) - 1;
-        m &= m - 1;
-        const float4 xj = w.ref[j];
-        const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
-        const float t = fmaxf(0.f, fmaf(-fmaf(dx, dx, fmaf(dy, dy, dz * dz)), p.inv_dc2_ang, 1.f));
-        cl = fmaf(t, t, cl);
-      }
-    }
-  }
+  const float cl = clash_pairs(p, w.ref, d, p.inv_dc2_ang, lane);
   return warp_sum(cl);
 }
 
@@ -485,16 +500,19 @@ __device__ void build_pose(const DockParams &p, const WarpSmem &w, float4 *buf, 
 __device__ inline void build_state(const float4 *ref, float4 *buf, const BondRec *bonds, const LigDesc &d,
                                    const float *R, const float *T, const float *phi, int lane) {
   for (int i = lane; i < d.n_atoms; i += 32) buf[i] = ref[i];
+  // the bonds' sines and cosines side by side, a lane per bond
+  const float ang_l = lane < d.n_rot ? phi[lane] : 0.f;
+  float sn_l, cs_l;
+  sincosf(ang_l, &sn_l, &cs_l);
+  const unsigned turned = __ballot_sync(FULL, ang_l != 0.f);
   __syncwarp();
   for (int b = 0; b < d.n_rot; ++b) {
-    const float ang = phi[b];
-    if (ang == 0.f) continue;
+    if (!(turned >> b & 1u)) continue;
     const BondRec br = bonds[b];
     float nx, ny, nz;
     const float4 pv = buf[br.v];
     bond_axis(buf[br.u], pv, nx, ny, nz);
-    float sn, cs;
-    sincosf(ang, &sn, &cs);
+    const float sn = __shfl_sync(FULL, sn_l, b), cs = __shfl_sync(FULL, cs_l, b);
     Rot rot;
     rot.make(cs, sn, nx, ny, nz, pv.x, pv.y, pv.z);
     __syncwarp();
@@ -523,24 +541,12 @@ template <int MODE>
 __device__ float full_score(const DockParams &p, const void *maps, const WarpSmem &w, float4 *buf,
                             const LigDesc &d, int sid, const uint32_t (&tors)[4], int lane) {
   build_pose<MODE>(p, w, buf, d, sid, tors, lane);
-  float e = 0.f, cl = 0.f;
+  float e = 0.f;
   for (int i = lane; i < d.n_atoms; i += 32) {
     const float4 xi = buf[i];
     e += grid_eval<MODE>(maps, __float_as_int(xi.w), xi.x, xi.y, xi.z, p.g);
-    for (int wd = 0; wd < d.n_words; ++wd) {
-      uint32_t m = __ldg(p.elig + d.elig_base + i * d.n_words + wd);
-      const int lo = i + 1 - 32 * wd;
-      if (lo >= 32) m = 0; else if (lo > 0) m &= ~0u << lo;
-      while (m) {
-        const int j = 32 * wd + __ffs(m) - 1;
-        m &= m - 1;
-        const float4 xj = buf[j];
-        const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
-        const float t = fmaxf(0.f, fmaf(-fmaf(dx, dx, fmaf(dy, dy, dz * dz)), p.inv_dc2_grid, 1.f));
-        cl = fmaf(t, t, cl);
-      }
-    }
   }
+  float cl = clash_pairs(p, buf, d, p.inv_dc2_grid, lane);
   e = warp_sum(e);
   cl = warp_sum(cl);
   __syncwarp();

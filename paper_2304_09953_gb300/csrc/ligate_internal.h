@@ -171,6 +171,7 @@ struct DockParams {
   // pocket
   const void *maps;        // map read by the sweep (mode)
   const float *maps_f32;   // FP32 map for rescoring (plain)
+  const float4 *maps_f32c; // its corner copy, or null: the same values
   GridConst g;
   // start frames
   const float *rot;        // [n_orient][9] rotation / h (grid units)
