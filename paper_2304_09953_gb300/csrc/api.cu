@@ -297,6 +297,8 @@ extern "C" void ligate_pocket_destroy(ligate_pocket *p) {
   cudaFree(p->d.rec);
   cudaFree(p->d.rec_pair);
   cudaFree(p->d.rec_cell);
+  cudaFree(p->d.rec_fine);
+  cudaFree(p->d.rec_list);
   delete p;
 }
 
@@ -367,6 +369,88 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
     for (int j = 0; j < n; ++j) sorted[fill[cell_of[j]]++] = rec[j];  // stable: input order within a cell
     rec.swap(sorted);
   }
+  // fine cells of about 2 A (wider while the lists would exceed 16 Mi entries)
+  // inside each coarse cell, one coarse cell beyond the grid included, over the
+  // map box and three quarters of the cutoff around it (lists for every cell
+  // of the neighbourhood cost 17 ms more per receptor and gained nothing).  A
+  // fine cell's list holds the receptor atoms of its coarse cell's
+  // 3 x 3 x 3 neighbourhood that can be within the cutoff of a point in it,
+  // with a margin for FP32 rounding of the cell index and the distance, in the
+  // column (lane, accumulator) that the kernel's row-by-row sum over the
+  // neighbourhood gives them: position o of a row of three cells is lane o % 32,
+  // accumulator o / 32 % 2
+  const int dim[3] = {P->d.nx, P->d.ny, P->d.nz};
+  int fs[3] = {1, 1, 1}, f0[3] = {0, 0, 0}, nf[3] = {0, 0, 0};
+  std::vector<int> fstart(1, 0);
+  std::vector<uint16_t> flist;
+  for (double width = 2.0; n > 0 && n < 0xffff; width *= 2.0) {
+    bool finest = true;
+    for (int a = 0; a < 3; ++a) {
+      fs[a] = (int)std::max(1.0, std::min(16.0, std::ceil(wd[a] * h / width)));
+      finest &= fs[a] == 1;
+      const double wf = wd[a] / fs[a];
+      const double rim = 0.75 * cut_g;  // poses reach out of the box by a few A
+      f0[a] = (int)std::max(-(double)fs[a], std::floor((-rim - lo[a]) / wf));
+      const int f1 = (int)std::min((double)(nc[a] + 1) * fs[a] - 1,
+                                   std::max(-1e6, std::floor((dim[a] - 1 + rim - lo[a]) / wf)));
+      nf[a] = std::max(0, f1 - f0[a] + 1);
+    }
+    const long long nfc = (long long)nf[0] * nf[1] * nf[2];
+    if (nfc > (1 << 18)) {
+      if (finest) { nf[0] = 0; break; }
+      continue;
+    }
+    std::vector<std::vector<uint16_t>> lists((size_t)nfc);
+    std::atomic<long long> total(0);
+    const double reach = cut_g * (1.0 + 1e-5) + 0.02 + 1e-5 * std::max(dim[0], std::max(dim[1], dim[2]));
+    const long long most = (long long)16 << 20;
+    parallel_for((int)nfc, nfc < 256 ? 1 : (int)std::max(1u, std::min(64u, std::thread::hardware_concurrency())),
+                 [&](int c) {
+      if (total.load(std::memory_order_relaxed) > most) return;
+      const int fc[3] = {c % nf[0], c / nf[0] % nf[1], c / nf[0] / nf[1]};
+      int cc[3], k0[3], k1[3];
+      double b0[3], b1[3];
+      for (int a = 0; a < 3; ++a) {
+        const int f = f0[a] + fc[a] + fs[a];  // from the coarse cell before the grid
+        cc[a] = f / fs[a] - 1;
+        b0[a] = lo[a] + (f0[a] + fc[a]) * (wd[a] / fs[a]);
+        b1[a] = b0[a] + wd[a] / fs[a];
+        k0[a] = std::max(cc[a] - 1, 0);
+        k1[a] = std::min(cc[a] + 1, nc[a] - 1);
+      }
+      if (k0[0] > k1[0] || k0[1] > k1[1] || k0[2] > k1[2]) return;
+      std::vector<uint16_t> col[64];
+      size_t steps = 0;
+      for (int z = k0[2]; z <= k1[2]; ++z)
+        for (int y = k0[1]; y <= k1[1]; ++y) {
+          const int row = (z * nc[1] + y) * nc[0], s0 = start[row + k0[0]];
+          for (int j = s0; j < start[row + k1[0] + 1]; ++j) {
+            const double dx = std::max(0.0, std::max(b0[0] - rec[j].x, rec[j].x - b1[0])),
+                         dy = std::max(0.0, std::max(b0[1] - rec[j].y, rec[j].y - b1[1])),
+                         dz = std::max(0.0, std::max(b0[2] - rec[j].z, rec[j].z - b1[2]));
+            if (dx * dx + dy * dy + dz * dz > reach * reach) continue;
+            std::vector<uint16_t> &v = col[(j - s0) % 64];
+            v.push_back((uint16_t)j);
+            steps = std::max(steps, v.size());
+          }
+        }
+      std::vector<uint16_t> &L = lists[c];
+      L.assign(steps * 64, 0xffff);
+      for (int q = 0; q < 64; ++q)
+        for (size_t k = 0; k < col[q].size(); ++k) L[k * 64 + q] = col[q][k];
+      total += (long long)L.size();
+    });
+    if (total.load() > most) {
+      if (finest) { nf[0] = 0; break; }
+      continue;
+    }
+    fstart.assign((size_t)nfc + 1, 0);
+    for (size_t c = 0; c < lists.size(); ++c) fstart[c + 1] = fstart[c] + (int)(lists[c].size() / 64);
+    flist.resize((size_t)fstart.back() * 64);
+    for (size_t c = 0; c < lists.size(); ++c)
+      std::copy(lists[c].begin(), lists[c].end(), flist.begin() + (size_t)fstart[c] * 64);
+    break;
+  }
   std::vector<float2> pair((size_t)n_types * n_types);
   for (int t = 0; t < n_types; ++t)
     for (int u = 0; u < n_types; ++u) {
@@ -376,6 +460,10 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
   cudaFree(P->d.rec);
   cudaFree(P->d.rec_pair);
   cudaFree(P->d.rec_cell);
+  cudaFree(P->d.rec_fine);
+  cudaFree(P->d.rec_list);
+  P->d.rec_fine = nullptr;
+  P->d.rec_list = nullptr;
   P->d.rec = nullptr;
   P->d.rec_pair = nullptr;
   P->d.rec_cell = nullptr;
@@ -386,8 +474,15 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
       (e = dmalloc(&P->d.rec_pair, pair.size())) != cudaSuccess ||
       (e = cudaMemcpy(P->d.rec_pair, pair.data(), 8 * pair.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = dmalloc(&P->d.rec_cell, start.size())) != cudaSuccess ||
-      (e = cudaMemcpy(P->d.rec_cell, start.data(), 4 * start.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
+      (e = cudaMemcpy(P->d.rec_cell, start.data(), 4 * start.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+      (e = dmalloc(&P->d.rec_fine, fstart.size())) != cudaSuccess ||
+      (e = cudaMemcpy(P->d.rec_fine, fstart.data(), 4 * fstart.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+      (e = dmalloc(&P->d.rec_list, flist.size())) != cudaSuccess ||
+      (!flist.empty() &&
+       (e = cudaMemcpy(P->d.rec_list, flist.data(), 2 * flist.size(), cudaMemcpyHostToDevice)) != cudaSuccess)) {
     cudaFree(P->d.rec); cudaFree(P->d.rec_pair); cudaFree(P->d.rec_cell);
+    cudaFree(P->d.rec_fine); cudaFree(P->d.rec_list);
+    P->d.rec_fine = nullptr; P->d.rec_list = nullptr;
     P->d.rec = nullptr; P->d.rec_pair = nullptr; P->d.rec_cell = nullptr;
     return cuda_fail(e, "pocket_set_receptor");
   }
@@ -395,6 +490,9 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
     P->d.rec_nc[a] = nc[a];
     P->d.rec_lo[a] = (float)lo[a];
     P->d.rec_inv[a] = (float)(1.0 / wd[a]);
+    P->d.rec_fs[a] = fs[a];
+    P->d.rec_f0[a] = f0[a];
+    P->d.rec_nf[a] = nf[a];
   }
   P->d.n_rec = n;
   P->d.rec_types = n_types;
@@ -1944,6 +2042,10 @@ static ligate_status rec_params(const ligate_pocket *P, const ligate_batch *B, R
   r.cut2 = P->d.rec_cut2; r.cap = P->d.rec_cap; r.rmin2 = P->d.rec_rmin2;
   r.ox = (float)P->d.origin[0]; r.oy = (float)P->d.origin[1]; r.oz = (float)P->d.origin[2];
   r.inv_h = (float)(1.0 / P->d.spacing);
+  r.fine = P->d.rec_fine; r.list = P->d.rec_list;
+  r.fsx = P->d.rec_fs[0]; r.fsy = P->d.rec_fs[1]; r.fsz = P->d.rec_fs[2];
+  r.fx0 = P->d.rec_f0[0]; r.fy0 = P->d.rec_f0[1]; r.fz0 = P->d.rec_f0[2];
+  r.nfx = P->d.rec_nf[0]; r.nfy = P->d.rec_nf[1]; r.nfz = P->d.rec_nf[2];
   return LIGATE_OK;
 }
 

@@ -100,6 +100,10 @@ struct PocketDev {
   int rec_nc[3] = {1, 1, 1};       // cells per axis (at most 16)
   float rec_lo[3] = {0, 0, 0};     // cell grid origin, grid units
   float rec_inv[3] = {0, 0, 0};    // 1 / cell width
+  // the atoms' indices listed per fine cell (RecParams::fine)
+  int *rec_fine = nullptr;
+  uint16_t *rec_list = nullptr;
+  int rec_fs[3] = {1, 1, 1}, rec_f0[3] = {0, 0, 0}, rec_nf[3] = {0, 0, 0};
 };
 
 // Receptor term of the exact rescoring, device view.
@@ -112,6 +116,13 @@ struct RecParams {
   float ox, oy, oz, inv_h;  // Angstrom -> grid units, for poses given as states
   int ncx, ncy, ncz;
   float lox, loy, loz, icx, icy, icz;
+  // fine cells: coarse cell (cx, cy, cz), which may lie one beyond the grid,
+  // split fsx x fsy x fsz; the nfx x nfy x nfz of them from index (fx0, fy0,
+  // fz0) on cover the map box and a rim.  Fine cell c's receptor atoms are the columns of
+  // list [fine[c], fine[c + 1]) x 64 (lane + 32 accumulator; 0xffff: none)
+  const int *fine;
+  const uint16_t *list;
+  int fsx, fsy, fsz, fx0, fy0, fz0, nfx, nfy, nfz;
 };
 
 // Poses given as continuous states (ligate_pose_state at base + i * stride);

@@ -18,13 +18,75 @@ namespace ligate {
 // receptor term is the maps' pair potential evaluated at each atom:
 // min(cap, sum_j eps_tj ((r0/r)^12 - 2 (r0/r)^6)) over receptor atoms within
 // the cutoff, r floored at rmin (grid units throughout); the clash term is
-// the docking score's.  The CTA stages all receptor atoms (sorted by cell of
-// a grid whose cells are at least the cutoff wide) and the cells' start
-// offsets in shared memory; each warp takes poses, builds the pose, and for
-// every ligand atom its lanes split the atoms of the 9 rows of 3 cells
-// around it (conflict-free consecutive reads); atoms farther away are
-// beyond the cutoff.
-__global__ void __launch_bounds__(256) rescore_kernel(const DockParams p, const RecParams r, int n_poses,
+// the docking score's.
+//
+// The receptor atoms are sorted by cell of a grid whose cells are at least the
+// cutoff wide; a warp takes runs of consecutive poses (mostly one ligand's),
+// builds each and sums the receptor term atom by atom (receptor_cells defines
+// the sum).
+//
+// What bounds it: instruction issue on the distance tests.  The 27 cells
+// around an atom hold 6.4 times the atoms within the cutoff.  So each coarse
+// cell is split into fine cells about 2 A wide, and a fine cell has the
+// receptor atoms that can be within the cutoff of a point in it (1.8 times),
+// laid out as the 64 columns (lane, accumulator) that receptor_cells gives
+// them, in its order: the same terms in the same order, so the same bits, in a
+// third of the steps.  16-bit indices keep the lists small (128 bytes per
+// step), and the coordinates stay in L1: staged in shared memory (16 B per
+// receptor atom and CTA) they left 24 warps per SM at 3,000 receptor atoms and
+// 8 at 8,000.  Two atoms run side by side, for the latency of the loads and of
+// the warp sums.  32,000 poses of the batched library (3,000 receptor atoms)
+// 2,160 -> 955 us, 4,800 of the large target's (8,000) 815 -> 164 us.
+// One receptor atom's term at squared distance d2, added to acc.
+__device__ __forceinline__ float pair_term(const RecParams &r, const float2 &pp, float d2, float acc) {
+  const float q2 = __fdividef(pp.x, fmaxf(d2, r.rmin2));
+  const float q6 = q2 * q2 * q2;
+  return fmaf(pp.y, fmaf(q6, q6, -2.f * q6), acc);
+}
+
+// Coarse cell coordinate of u along one axis, as a float (clamped to two cells
+// beyond the grid first, so far or non-finite coordinates give an empty
+// neighbourhood or edge cells).
+__device__ __forceinline__ float cell_coord(float u, float lo, float inv, int n) {
+  return fminf(fmaxf((u - lo) * inv, -2.f), (float)n + 1.f);
+}
+
+// Receptor sum at u over the 3 x 3 x 3 coarse cells around it (clamped to the
+// grid): two receptor atoms per lane per iteration, separate accumulators (the
+// per-pair chain is long, independent pairs keep the pipes busy).
+// Warp-collective, u the same in every lane.
+__device__ __noinline__ float receptor_cells(const RecParams &r, const float2 *prow, float ux, float uy,
+                                             float uz, int lane) {
+  const int cx = (int)floorf(cell_coord(ux, r.lox, r.icx, r.ncx)), cy = (int)floorf(cell_coord(uy, r.loy, r.icy, r.ncy)),
+            cz = (int)floorf(cell_coord(uz, r.loz, r.icz, r.ncz));
+  const int x0 = max(cx - 1, 0), x1 = min(cx + 1, r.ncx - 1);
+  const int y0 = max(cy - 1, 0), y1 = min(cy + 1, r.ncy - 1);
+  const int z0 = max(cz - 1, 0), z1 = min(cz + 1, r.ncz - 1);
+  float acc[2] = {0.f, 0.f};
+  if (x0 <= x1)
+    for (int z = z0; z <= z1; ++z)
+      for (int y = y0; y <= y1; ++y) {
+        const int row = (z * r.ncy + y) * r.ncx;
+        const int j_hi = __ldg(r.cell + row + x1 + 1);
+        for (int j0 = __ldg(r.cell + row + x0) + lane; j0 < j_hi; j0 += 64)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int j = j0 + 32 * q;
+            if (j < j_hi) {
+              const float4 a = __ldg(r.rec + j);
+              const float dx = ux - a.x, dy = uy - a.y, dz = uz - a.z;
+              const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+              if (d2 <= r.cut2) acc[q] = pair_term(r, prow[__float_as_int(a.w)], d2, acc[q]);
+            }
+          }
+      }
+  return warp_sum(acc[0] + acc[1]);
+}
+
+constexpr int POSE_RUN = 4;  // consecutive poses a warp takes at a time
+
+__global__ void __launch_bounds__(256) rescore_kernel(const __grid_constant__ DockParams p,
+                                                     const __grid_constant__ RecParams r, int n_poses,
                                                      const int32_t *__restrict__ lig_idx,
                                                      const int32_t *__restrict__ start_id,
                                                      const uint8_t *__restrict__ tors,
@@ -33,21 +95,21 @@ __global__ void __launch_bounds__(256) rescore_kernel(const DockParams p, const 
                                                      const StateSrc ss,
                                                      ligate_rescored *__restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int ncells = r.ncx * r.ncy * r.ncz;
-  float4 *rec = reinterpret_cast<float4 *>(smem_raw);
-  float2 *pair = reinterpret_cast<float2 *>(rec + r.n_rec);
-  int *cell = reinterpret_cast<int *>(pair + ((r.n_types * r.n_types + 1) & ~1));
-  unsigned char *slots = reinterpret_cast<unsigned char *>(cell + ((ncells + 1 + 3) & ~3));
-  for (int j = threadIdx.x; j < r.n_rec; j += blockDim.x) rec[j] = r.rec[j];
+  float2 *pair = reinterpret_cast<float2 *>(smem_raw);
+  unsigned char *slots = reinterpret_cast<unsigned char *>(pair + ((r.n_types * r.n_types + 1) & ~1));
   for (int j = threadIdx.x; j < r.n_types * r.n_types; j += blockDim.x) pair[j] = r.pair[j];
-  for (int j = threadIdx.x; j <= ncells; j += blockDim.x) cell[j] = r.cell[j];
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
-  // warp slots without a pair list: more warps per CTA share the staged receptor
+  // warp slots without a pair list
   const WarpSmem w = warp_smem(slots + (size_t)warp * smem_bytes_per_warp(p.nmax, 0, 1, 0, 0), p.nmax, 1, 0);
+  // runs of consecutive poses, shorter when there are few poses per warp
+  const int warps = gridDim.x * W;
+  const int run = max(1, min(POSE_RUN, n_poses / (8 * warps)));  // at least 8 runs per warp: balance
   int cur = -1;
   LigDesc d;
-  for (int pi = blockIdx.x * W + warp; pi < n_poses; pi += gridDim.x * W) {
+  for (long long t = (long long)(blockIdx.x * W + warp) * run, s = 0; t < n_poses;
+       t = ++s == run ? (s = 0, t + 1 + (long long)(warps - 1) * run) : t + 1) {
+    const int pi = (int)t;
     int li, sid;
     uint32_t tt[4] = {0u, 0u, 0u, 0u};
     const unsigned char *st_rec = nullptr;
@@ -78,7 +140,8 @@ __global__ void __launch_bounds__(256) rescore_kernel(const DockParams p, const 
     }
     if (li != cur) {
       __syncwarp();
-      (void)load_ligand(p, w, li, d, lane);
+      d = p.lig[li];
+      load_coords(p, w, d, lane);
       cur = li;
     }
     if (st_rec) {
@@ -99,71 +162,79 @@ __global__ void __launch_bounds__(256) rescore_kernel(const DockParams p, const 
     }
     float e_inter = 0.f;
     int ncap = 0, nout = 0;
-    for (int i = 0; i < d.n_atoms; ++i) {
-      const float4 u = w.pose[i];
-      const int t = __float_as_int(w.ref[i].w);
-      const float2 *prow = pair + t * r.n_types;
-      // the 3 x 3 x 3 cells around the atom (clamped to the grid; the index
-      // is clamped in floating point first, so far or non-finite coordinates
-      // give an empty neighbourhood or edge cells)
-      const int cx = (int)floorf(fminf(fmaxf((u.x - r.lox) * r.icx, -2.f), (float)r.ncx + 1.f));
-      const int cy = (int)floorf(fminf(fmaxf((u.y - r.loy) * r.icy, -2.f), (float)r.ncy + 1.f));
-      const int cz = (int)floorf(fminf(fmaxf((u.z - r.loz) * r.icz, -2.f), (float)r.ncz + 1.f));
-      const int x0 = max(cx - 1, 0), x1 = min(cx + 1, r.ncx - 1);
-      const int y0 = max(cy - 1, 0), y1 = min(cy + 1, r.ncy - 1);
-      const int z0 = max(cz - 1, 0), z1 = min(cz + 1, r.ncz - 1);
-      // two receptor atoms per lane per iteration, separate accumulators:
-      // the per-pair chain (distance, ratio, sixth and twelfth powers) is
-      // long, so independent pairs keep the pipes busy
-      float acc[2] = {0.f, 0.f};
-      if (x0 <= x1) {
-        for (int z = z0; z <= z1; ++z)
-          for (int y = y0; y <= y1; ++y) {
-            const int row = (z * r.ncy + y) * r.ncx;
-            const int j_hi = cell[row + x1 + 1];
-            for (int j0 = cell[row + x0] + lane; j0 < j_hi; j0 += 64) {
-#pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                const int j = j0 + 32 * q;
-                if (j < j_hi) {
-                  const float4 a = rec[j];
-                  const float dx = u.x - a.x, dy = u.y - a.y, dz = u.z - a.z;
-                  float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                  if (d2 <= r.cut2) {
-                    d2 = fmaxf(d2, r.rmin2);
-                    const float2 pp = prow[__float_as_int(a.w)];
-                    const float q2 = __fdividef(pp.x, d2);
-                    const float q6 = q2 * q2 * q2;
-                    acc[q] = fmaf(pp.y, fmaf(q6, q6, -2.f * q6), acc[q]);
-                  }
-                }
-              }
-            }
-          }
+    for (int i0 = 0; i0 < d.n_atoms; i0 += 32) {
+      // the lanes look up their own atoms' fine cells side by side (steps -1:
+      // outside the fine cells)
+      int lo_l = 0, steps_l = -1;
+      bool out_l = false;
+      if (i0 + lane < d.n_atoms) {
+        const float4 u = w.pose[i0 + lane];
+        out_l = !((u.x >= 0.f) & (u.x <= p.g.fx1) & (u.y >= 0.f) & (u.y <= p.g.fy1) & (u.z >= 0.f) & (u.z <= p.g.fz1));
+        const float vx = cell_coord(u.x, r.lox, r.icx, r.ncx), vy = cell_coord(u.y, r.loy, r.icy, r.ncy),
+                    vz = cell_coord(u.z, r.loz, r.icz, r.ncz);
+        const float cx = floorf(vx), cy = floorf(vy), cz = floorf(vz);
+        const int fx = (int)cx * r.fsx + min((int)((vx - cx) * (float)r.fsx), r.fsx - 1) - r.fx0,
+                  fy = (int)cy * r.fsy + min((int)((vy - cy) * (float)r.fsy), r.fsy - 1) - r.fy0,
+                  fz = (int)cz * r.fsz + min((int)((vz - cz) * (float)r.fsz), r.fsz - 1) - r.fz0;
+        if (fx >= 0 && fx < r.nfx && fy >= 0 && fy < r.nfy && fz >= 0 && fz < r.nfz) {
+          const int *f = r.fine + (fz * r.nfy + fy) * r.nfx + fx;
+          lo_l = __ldg(f);
+          steps_l = __ldg(f + 1) - lo_l;
+        }
       }
-      float accs = warp_sum(acc[0] + acc[1]);
-      if (accs >= r.cap) { accs = r.cap; ++ncap; }
-      e_inter += accs;
-      nout += !((u.x >= 0.f) & (u.x <= p.g.fx1) & (u.y >= 0.f) & (u.y <= p.g.fy1) & (u.z >= 0.f) &
-                (u.z <= p.g.fz1));
-    }
-    float cl = 0.f;
-    for (int i = lane; i < d.n_atoms; i += 32) {
-      const float4 xi = w.pose[i];
-      for (int wd = 0; wd < d.n_words; ++wd) {
-        uint32_t m = __ldg(p.elig + d.elig_base + i * d.n_words + wd);
-        const int lo = i + 1 - 32 * wd;
-        if (lo >= 32) m = 0; else if (lo > 0) m &= ~0u << lo;
-        while (m) {
-          const int j = 32 * wd + __ffs(m) - 1;
-          m &= m - 1;
-          const float4 xj = w.pose[j];
-          const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
-          const float t = fmaxf(0.f, fmaf(-fmaf(dx, dx, fmaf(dy, dy, dz * dz)), p.inv_dc2_grid, 1.f));
-          cl = fmaf(t, t, cl);
+      nout += __popc(__ballot_sync(FULL, out_l));
+      const int i1 = min(32, d.n_atoms - i0);
+      for (int i = 0; i < i1; i += 2) {  // two atoms side by side: their chains and loads overlap
+        float4 u[2];
+        const float2 *prow[2];
+        const uint16_t *list[2];
+        int steps[2];
+        float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+        unsigned nx[2][2];  // the next step's indices
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          const int k = min(i + v, i1 - 1);
+          u[v] = w.pose[i0 + k];
+          prow[v] = pair + __float_as_int(w.ref[i0 + k].w) * r.n_types;
+          list[v] = r.list + (size_t)__shfl_sync(FULL, lo_l, k) * 64 + lane;
+          steps[v] = __shfl_sync(FULL, steps_l, k);
+          if (i + v >= i1) steps[v] = 0;
+          nx[v][0] = nx[v][1] = 0xffffu;
+          if (steps[v] > 0) { nx[v][0] = __ldg(list[v]); nx[v][1] = __ldg(list[v] + 32); }
+        }
+        const int top = max(steps[0], steps[1]);
+        for (int k = 0; k < top; ++k) {
+          unsigned j[2][2];
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            j[v][0] = nx[v][0];
+            j[v][1] = nx[v][1];
+            list[v] += 64;
+            nx[v][0] = nx[v][1] = 0xffffu;
+            if (k + 1 < steps[v]) { nx[v][0] = __ldg(list[v]); nx[v][1] = __ldg(list[v] + 32); }
+          }
+#pragma unroll
+          for (int v = 0; v < 2; ++v)
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              if (j[v][q] != 0xffffu) {
+                const float4 a = __ldg(r.rec + j[v][q]);
+                const float dx = u[v].x - a.x, dy = u[v].y - a.y, dz = u[v].z - a.z;
+                const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                if (d2 <= r.cut2) acc[v][q] = pair_term(r, prow[v][__float_as_int(a.w)], d2, acc[v][q]);
+              }
+        }
+        float accs[2] = {warp_sum(acc[0][0] + acc[0][1]), warp_sum(acc[1][0] + acc[1][1])};
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          if (i + v >= i1) continue;  // warp-uniform
+          if (steps[v] < 0) accs[v] = receptor_cells(r, prow[v], u[v].x, u[v].y, u[v].z, lane);
+          if (accs[v] >= r.cap) { accs[v] = r.cap; ++ncap; }
+          e_inter += accs[v];
         }
       }
     }
+    float cl = clash_pairs(p, w.pose, d, p.inv_dc2_grid, lane);
     cl = p.clash_w * warp_sum(cl);
     if (lane == 0) {
       ligate_rescored o;
@@ -220,7 +291,8 @@ __global__ void __launch_bounds__(128) pose_features_kernel(const DockParams p, 
     }
     if (li != cur) {
       __syncwarp();
-      (void)load_ligand(p, w, li, d, lane);
+      d = p.lig[li];
+      load_coords(p, w, d, lane);
       cur = li;
     }
     build_pose<MODE_F32_PLAIN>(p, w, w.pose, d, sid, tt, lane);
@@ -242,23 +314,7 @@ __global__ void __launch_bounds__(128) pose_features_kernel(const DockParams p, 
         if (t == ty) { ts[t] += v; tn[t] += 1.f; }
       high += v >= 9.f ? 1.f : 0.f;
     }
-    float cl = 0.f;
-    for (int i = lane; i < d.n_atoms; i += 32) {
-      const float4 xi = w.pose[i];
-      for (int wd = 0; wd < d.n_words; ++wd) {
-        uint32_t m = __ldg(p.elig + d.elig_base + i * d.n_words + wd);
-        const int lo = i + 1 - 32 * wd;
-        if (lo >= 32) m = 0; else if (lo > 0) m &= ~0u << lo;
-        while (m) {
-          const int j = 32 * wd + __ffs(m) - 1;
-          m &= m - 1;
-          const float4 xj = w.pose[j];
-          const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
-          const float t = fmaxf(0.f, fmaf(-fmaf(dx, dx, fmaf(dy, dy, dz * dz)), p.inv_dc2_grid, 1.f));
-          cl = fmaf(t, t, cl);
-        }
-      }
-    }
+    float cl = clash_pairs(p, w.pose, d, p.inv_dc2_grid, lane);
     e = warp_sum(e);
     cl = p.clash_w * warp_sum(cl);
     high = warp_sum(high);
@@ -317,10 +373,9 @@ cudaError_t launch_rescore(const DockParams &p, const RecParams &r, int n_poses,
                            const int32_t *row_lig, const StateSrc *states, ligate_rescored *out,
                            cudaStream_t s) {
   if (n_poses <= 0) return cudaSuccess;
-  int warps = 8;
-  while (warps > 1 && rescore_smem_bytes(p, r, warps) > 227 * 1024) --warps;
-  const size_t smem = rescore_smem_bytes(p, r, warps);
-  if (smem > 227 * 1024) return cudaErrorInvalidValue;
+  const int warps = 8;
+  const size_t smem = (size_t)((r.n_types * r.n_types + 1) & ~1) * 8 + (size_t)warps * smem_bytes_per_warp(p.nmax, 0, 1, 0, 0);
+  if (smem > 227 * 1024) return cudaErrorInvalidValue;  // never: 32 KB of pairs and 8 slots of at most 6 KB
   cudaError_t e = cudaFuncSetAttribute(rescore_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, occ = 0;
@@ -356,8 +411,8 @@ __global__ void __launch_bounds__(256) state_coords_kernel(const DockParams p, c
     for (int q = lane; q < LIGATE_MAX_ATOMS * 3; q += 32) o[q] = __int_as_float(0x7fc00000);
     return;
   }
-  LigDesc d;
-  (void)load_ligand(p, w, li, d, lane);
+  const LigDesc d = p.lig[li];
+  load_coords(p, w, d, lane);
   const ligate_pose_state &st = states[pi];
   build_state(w.ref, w.pose, w.bonds, d, st.rot, st.trans, st.tors, lane);
   for (int i = lane; i < d.n_atoms; i += 32) {
