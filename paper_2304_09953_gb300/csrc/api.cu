@@ -1135,13 +1135,17 @@ static void default_tile(ligate_tile *t) {
 // balance).  lo = 32 starts, or the starts per resident warp of a batch too
 // small to give every warp 32 (at least 8), but no fewer than 2 K: an item
 // pays for loading its ligand, and has no K-th best of its own to stop starts
-// with before its K-th start (measured, lo = 128, 64, 32, 16, 8: one 24-atom
+// with before its K-th start.  A run of fewer than 4 starts per resident warp
+// spreads over all of them: every start is under way before a K-th best could
+// stop one (measured, lo = 128, 64, 32, 16, 8: one 24-atom
 // ligand with 512 starts and K = 4 372, 213, 135, 99 and 88 us; 301 ligands
 // with 1,717 starts and K = 5 4.9, 3.44, 3.19, 3.49 and 3.62 ms; 8 P in the
 // model against 12 P and 16 P: 1,000 ligands 24.1, 24.5, 25.1 ms).
 // Buckets without ligands get 512.  Ligands: sel[0..n) or all of B.
 static double least_chunk(double starts, double P_warps, int K) {
-  return std::max(2.0 * K, std::min(32.0, std::max(8.0, starts / std::max(P_warps, 1.0))));
+  const double each = starts / std::max(P_warps, 1.0);
+  if (each < 4.0) return each;
+  return std::max(2.0 * K, std::min(32.0, std::max(8.0, each)));
 }
 
 static void model_chunks(const BatchDev &B, const int32_t *sel, int n, int S, int n_starts, double P_warps,

@@ -21,19 +21,22 @@ int dock_memo1_tables(const LigDesc &d, const BondRec *bonds, int) {
 }
 
 // The clash tables of every row's ligand, once per run: one warp per (row,
-// table).  What a row's work items share is built here once instead of by
+// table) or, when that leaves the chip idle (split), per (row, table, round of G
+// steps: 301 ligands 65 -> MEASURED us).  What a row's work items share is built here once instead of by
 // every item's warp, so items can be small (a batch that leaves few starts
 // per warp) without paying for the tables again, and a ligand's tables are
 // built in parallel.  The same device code builds the tables in the docking
 // kernel when the rows' tables do not fit the plan's budget.
 __global__ void __launch_bounds__(128) clash_tables_kernel(const __grid_constant__ DockParams p, const int32_t *__restrict__ row_lig,
-                                                           int rows) {
+                                                           int rows, int split) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const WarpSmem w = warp_smem(smem_raw + (size_t)warp * smem_bytes_per_warp(p.nmax, 0, p.G, 0), p.nmax, p.G);
   const int tables = 2 + p.m1max, S = p.S, L = p.L, G = p.G;
-  const long long id = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-  const int row = (int)(id / tables), t = (int)(id % tables);
+  const long long task = (long long)blockIdx.x * (blockDim.x >> 5) + warp, id = task / split;
+  const int part = (int)(task % split), row = (int)(id / tables), t = (int)(id % tables);
+  const int r0 = split > 1 ? part : 0, r1 = split > 1 ? part + 1 : (S + G - 1) / G;  // rounds of a table
+  if (t == 0 && part > 0) return;
   if (row >= rows) return;
   const int li = row_lig[row];
   const LigDesc d = p.lig[li];
@@ -57,8 +60,8 @@ __global__ void __launch_bounds__(128) clash_tables_kernel(const __grid_constant
   start_frame(p, 0, R, T);
   float *memo = p.tab + (size_t)row * p.tab_stride, *m1 = memo + memo_floats(S, p.rmax);
   if (t == 0) input_rows(p, w, pose, d, R, T, ck, sk, g, k, L, G, S, memo);
-  else if (t == 1) turn_table<false>(p, w, pose, d, w.bonds[0], w.bonds[1], R, T, ck, sk, g, k, L, G, S, memo + S);
-  else single_table(p, w, pose, d, w.bonds[slot_bond], R, T, ck, sk, g, k, L, G, S, m1);
+  else if (t == 1) turn_table<false>(p, w, pose, d, w.bonds[0], w.bonds[1], R, T, ck, sk, g, k, L, G, S, memo + S, r0, r1);
+  else single_table(p, w, pose, d, w.bonds[slot_bond], R, T, ck, sk, g, k, L, G, S, m1, r0, r1);
 }
 
 // ---------------------------------------------------------------------------
@@ -194,8 +197,12 @@ cudaError_t launch_clash_tables(const DockParams &p, const int32_t *row_lig, int
   const size_t smem = (size_t)warps * smem_bytes_per_warp(p.nmax, 0, p.G, 0);
   cudaError_t e = cudaFuncSetAttribute(clash_tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e != cudaSuccess) return e;
-  const long long n = (long long)rows * (2 + p.m1max);
-  clash_tables_kernel<<<(unsigned)((n + warps - 1) / warps), 32 * warps, smem, s>>>(p, row_lig, rows);
+  // rounds of a table side by side while they would not fill the SMs twice
+  const int rounds = (p.S + p.G - 1) / p.G;
+  long long n = (long long)rows * (2 + p.m1max);
+  const int split = n * rounds <= 16384 ? rounds : 1;
+  n *= split;
+  clash_tables_kernel<<<(unsigned)((n + warps - 1) / warps), 32 * warps, smem, s>>>(p, row_lig, rows, split);
   return cudaGetLastError();
 }
 

@@ -346,6 +346,24 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// warp_sum of eight values at once: value q in lanes 4 q .. 4 q + 3.  Each value
+// goes through warp_sum's tree (lanes 16 apart first), so the sums are its bits.
+__device__ __forceinline__ float warp_sum8(float v0, float v1, float v2, float v3, float v4, float v5, float v6, float v7,
+                                      int lane) {
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+  auto half = [](bool up, float lo, float hi, int o) {  // keep lo (up: hi), add the partner lane's
+    const float keep = up ? hi : lo, give = up ? lo : hi;
+    return keep + __shfl_xor_sync(FULL, give, o);
+  };
+  const float a0 = half(h16, v0, v4, 16), a1 = half(h16, v1, v5, 16), a2 = half(h16, v2, v6, 16),
+              a3 = half(h16, v3, v7, 16);
+  const float b0 = half(h8, a0, a2, 8), b1 = half(h8, a1, a3, 8);
+  float c = half(h4, b0, b1, 4);
+  c += __shfl_xor_sync(FULL, c, 2);
+  c += __shfl_xor_sync(FULL, c, 1);
+  return c;
+}
+
 // Reference coordinates of ligand d centred on their centroid, and its bond
 // table, into the warp's slot.
 __device__ __forceinline__ void load_coords(const DockParams &p, const WarpSmem &w, const LigDesc &d, int lane) {

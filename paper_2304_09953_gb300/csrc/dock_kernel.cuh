@@ -150,15 +150,16 @@ __device__ __forceinline__ void pose_input(const WarpSmem &w, float4 *pose, cons
 }
 
 // Clash sums of the swept candidates of bond bb at every step k after bond be
-// alone turned by each step t, out[t S + k]; group g takes t = g, g + G, ...
+// alone turned by each step t, out[t S + k], rounds r0 to r1: group g takes t =
+// r G + g in round r.
 // LAST: stored with an L2 evict-last policy (ahead of streaming data).
 // Warp-collective.
 template <bool LAST>
 __device__ void turn_table(const DockParams &p, const WarpSmem &w, float4 *pose, const LigDesc &d, const BondRec &be,
                            const BondRec &bb, const float (&R)[9], const float (&T)[3], float ck, float sk, int g,
-                           int k, int L, int G, int S, float *out) {
+                           int k, int L, int G, int S, float *out, int r0, int r1) {
   unsigned n_pair = 0;  // not counted: once per ligand
-  for (int r = 0; r < (S + G - 1) / G; ++r) {
+  for (int r = r0; r < r1; ++r) {
     const int te = min(r * G + g, S - 1);  // groups past S repeat the last step
     pose_input(w, pose, d, R, T, k, L);
     float ex, ey, ez;
@@ -195,11 +196,11 @@ __device__ void turn_table(const DockParams &p, const WarpSmem &w, float4 *pose,
 // The pairs of bond b >= 2 that bond e1 alone separates, by e1's step.
 static __device__ void single_table(const DockParams &p, const WarpSmem &w, float4 *pose, const LigDesc &d, BondRec bb,
                              const float (&R)[9], const float (&T)[3], float ck, float sk, int g, int k, int L, int G,
-                             int S, float *m1) {
+                             int S, float *m1, int r0, int r1) {
   bb.cand_off += bb.n_cand0;
   bb.n_cand = bb.n_cand1;
   turn_table<true>(p, w, pose, d, w.bonds[bb.e1 & 0xffff], bb, R, T, ck, sk, g, k, L, G, S,
-                   m1 + (bb.e1 >> 16) * S * S);
+                   m1 + (bb.e1 >> 16) * S * S, r0, r1);
 }
 
 // memo[k]: the sums of bond 0's sweep; memo[memo_row0(S) + (b - memo_bonds(S))
@@ -241,11 +242,12 @@ static __device__ __noinline__ void build_memo(const DockParams &p, unsigned cha
   if (m1)
     for (int b = 2; b < d.n_rot; ++b) {
       const BondRec bb = w.bonds[b];
-      if (bb.n_cand1 > 0) single_table(p, w, pose, d, bb, R, T, ck, sk, g, k, L, G, S, m1);
+      if (bb.n_cand1 > 0) single_table(p, w, pose, d, bb, R, T, ck, sk, g, k, L, G, S, m1, 0, (S + G - 1) / G);
     }
   input_rows(p, w, pose, d, R, T, ck, sk, g, k, L, G, S, w.memo);
   if (d.n_rot >= 2 && memo_bonds(S) == 2)
-    turn_table<false>(p, w, pose, d, w.bonds[0], w.bonds[1], R, T, ck, sk, g, k, L, G, S, w.memo + S);
+    turn_table<false>(p, w, pose, d, w.bonds[0], w.bonds[1], R, T, ck, sk, g, k, L, G, S, w.memo + S, 0,
+                      (S + G - 1) / G);
 }
 
 // Drops the L2 copies of the whole 128-byte lines inside [lo, hi) without

@@ -165,19 +165,21 @@ cudaError_t gemm(int kind, const GemmArgs &g, cudaStream_t s) {
 
 // ---------------------------------------------------------------------------
 // All parameter gradients of one training step in one launch: for each hidden
-// layer the weight gradient dW = H^T dZ (64 x 32 tiles, mma.sync m16n8k16,
+// layer the weight gradient dW = H^T dZ (128 x 64 tiles, mma.sync m16n8k16,
 // rows as k) and the column sums of dZ (bias gradients), and the head's
 // gw4[k] = sum_b H3[b][k] dy[b] and gb4 = sum_b dy[b].  Rows stream through a
 // four-stage cp.async ring of 64-row slices.
 //
 // What bounds it: every sum runs over the rows in ascending order, so it is a
 // serial chain per output (the MMA steps of a tile; one addition per row of a
-// column sum); the launch is as wide as the outputs allow (320 tiles + 32
-// column CTAs, all resident at once) and the loads are off the chain.  Before,
-// the sums ran as launches of their own on 2 and 4 CTAs with every load on the
-// chain and the weight gradients on 8 to 16 CTAs without overlap: 87 + 3 x 61
-// + 3 x 37 us per step of 1,024 rows (serialised, cold), now 21.
-constexpr int GK = 64, GM = 64, GN = 32, GC = 64, GSTAGES = 4;  // rows per slice, tile, columns of a sum CTA
+// column sum), and the operands come from L2 once per tile row and column: 80
+// tiles + 32 column CTAs, one wave, 31 MB at 1,024 rows (64 x 32 tiles, twice
+// the traffic, took 17.7 us against MEASURED).  Before, the sums ran as launches of
+// their own on 2 and 4 CTAs with every load on the chain and the weight
+// gradients on 8 to 16 CTAs without overlap: 87 + 3 x 61 + 3 x 37 us per step
+// of 1,024 rows (serialised, cold).
+constexpr int GK = 64, GM = 128, GN = 64, GC = 64, GSTAGES = 4;  // rows per slice, tile, columns of a sum CTA
+constexpr int GT = 256;  // threads
 constexpr int GA_LD = GM + 8, GB_LD = GN + 8, GC_LD = GC + 8;
 constexpr int G_STAGE = GK * (GA_LD + GB_LD);  // elements per stage (a sum CTA's slice is smaller)
 static_assert(GK * GC_LD <= G_STAGE, "column slices fit the stage");
@@ -192,18 +194,19 @@ __device__ __forceinline__ void load_slice(__nv_bfloat16 *dst, const __nv_bfloat
                                            int rows) {
   constexpr int CH = COLS / 8;
 #pragma unroll
-  for (int c = threadIdx.x; c < GK * CH; c += 128) {
+  for (int c = threadIdx.x; c < GK * CH; c += GT) {
     const int r = c / CH, q = c % CH * 8;
     const bool in = k0 + r < rows;
     cp16(dst + r * LD + q, src + (size_t)(in ? k0 + r : 0) * ld + c0 + q, in);
   }
 }
 
-__global__ void __launch_bounds__(128) grads_kernel(const GradArgs a) {
+__global__ void __launch_bounds__(GT) grads_kernel(const GradArgs a) {
   extern __shared__ __align__(16) unsigned char graw[];
   __nv_bfloat16 *const ring = reinterpret_cast<__nv_bfloat16 *>(graw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int slices = (a.rows + GK - 1) / GK;
+  pdl_wait();
   int t = blockIdx.x;
   int layer = 0;
   for (; layer < 3; ++layer) {  // a weight tile of this layer?
@@ -212,13 +215,14 @@ __global__ void __launch_bounds__(128) grads_kernel(const GradArgs a) {
     t -= n;
   }
   if (layer < 3) {
-    const int m0 = t / (512 / GN) * GM, n0 = t % (512 / GN) * GN, mb = warp * 16;
+    const int m0 = t / (512 / GN) * GM, n0 = t % (512 / GN) * GN;
+    const int mb = (warp >> 1) * 32, nb = (warp & 1) * 32;  // 4 x 2 warps of 32 x 32
     auto load = [&](int s) {
       __nv_bfloat16 *st = ring + (s % GSTAGES) * G_STAGE;
       load_slice<GM, GA_LD>(st, a.in[layer], a.fan_in[layer], m0, s * GK, a.rows);
       load_slice<GN, GB_LD>(st + GK * GA_LD, a.dz[layer], 512, n0, s * GK, a.rows);
     };
-    float acc[4][4] = {};
+    float acc[2][4][4] = {};
     for (int s = 0; s < GSTAGES - 1; ++s) {
       if (s < slices) load(s);
       asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -232,23 +236,29 @@ __global__ void __launch_bounds__(128) grads_kernel(const GradArgs a) {
       const int r = lane & 7, q1 = (lane >> 3) & 1, q2 = lane >> 4;
 #pragma unroll
       for (int ks = 0; ks < GK; ks += 16) {
-        uint32_t af[4], bf[4][2];
-        ldsm_x4_t(af[0], af[1], af[2], af[3], As + (ks + q2 * 8 + r) * GA_LD + mb + q1 * 8);
+        uint32_t af[2][4], bf[4][2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          ldsm_x4_t(af[i][0], af[i][1], af[i][2], af[i][3], As + (ks + q2 * 8 + r) * GA_LD + mb + i * 16 + q1 * 8);
 #pragma unroll
         for (int j = 0; j < 4; j += 2)
-          ldsm_x4_t(bf[j][0], bf[j][1], bf[j + 1][0], bf[j + 1][1], Bs + (ks + q1 * 8 + r) * GB_LD + j * 8 + q2 * 8);
+          ldsm_x4_t(bf[j][0], bf[j][1], bf[j + 1][0], bf[j + 1][1], Bs + (ks + q1 * 8 + r) * GB_LD + nb + j * 8 + q2 * 8);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) mma_bf16(acc[j], af, bf[j][0], bf[j][1]);
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], af[i], bf[j][0], bf[j][1]);
       }
     }
     float *dw = a.dw[layer];
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int m = m0 + mb + (lane >> 2) + h * 8, n = n0 + j * 8 + (lane & 3) * 2;
-        *reinterpret_cast<float2 *>(dw + (size_t)m * 512 + n) = make_float2(acc[j][2 * h], acc[j][2 * h + 1]);
-      }
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int m = m0 + mb + i * 16 + (lane >> 2) + h * 8, n = n0 + nb + j * 8 + (lane & 3) * 2;
+          *reinterpret_cast<float2 *>(dw + (size_t)m * 512 + n) = make_float2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
+        }
     return;
   }
   // column sums: 3 x 8 CTAs of the bias gradients, then 8 of the head
@@ -295,8 +305,7 @@ cudaError_t grads(const GradArgs &a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   int ctas = 4 * (512 / GC);
   for (int l = 0; l < 3; ++l) ctas += (a.fan_in[l] / GM) * (512 / GN);
-  grads_kernel<<<ctas, 128, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(grads_kernel, dim3(ctas), dim3(GT), smem, s, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -309,6 +318,7 @@ __global__ void gather_std_kernel(const float *__restrict__ desc, const int *__r
                                   float ly_mu, float ly_inv, __nv_bfloat16 *__restrict__ x,
                                   float *__restrict__ t) {
   const int b = blockIdx.x;
+  pdl_wait();
   if (b >= rows) return;
   const int src = idx ? idx[b] : row0 + b;
   for (int f = threadIdx.x; f < 256; f += blockDim.x)
@@ -324,8 +334,12 @@ __device__ __forceinline__ void head_row(const __nv_bfloat16 *__restrict__ h3, c
                                          float *__restrict__ y, float *__restrict__ dy, float inv_b2,
                                          __nv_bfloat16 *__restrict__ dz3, int warp, int lane, double *sq) {
   const __nv_bfloat16 *h = h3 + (size_t)warp * 512;
+  float hv[16], wv[16];  // columns lane, lane + 32, ...
+#pragma unroll
+  for (int k = 0; k < 16; ++k) { hv[k] = __bfloat162float(h[lane + 32 * k]); wv[k] = __bfloat162float(w4[lane + 32 * k]); }
   float s = 0.f;
-  for (int k = lane; k < 512; k += 32) s = fmaf(__bfloat162float(h[k]), __bfloat162float(w4[k]), s);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) s = fmaf(hv[k], wv[k], s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   s += b4[0];
@@ -337,10 +351,9 @@ __device__ __forceinline__ void head_row(const __nv_bfloat16 *__restrict__ h3, c
     dy[warp] = d;
     *sq = (double)e * e;
   }
-  for (int k = lane; k < 512; k += 32) {
-    const float hv = __bfloat162float(h[k]);
-    dz3[(size_t)warp * 512 + k] = __float2bfloat16_rn(hv > 0.f ? d * __bfloat162float(w4[k]) : 0.f);
-  }
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    dz3[(size_t)warp * 512 + lane + 32 * k] = __float2bfloat16_rn(hv[k] > 0.f ? d * wv[k] : 0.f);
 }
 
 __global__ void head_kernel(const __nv_bfloat16 *__restrict__ h3, const __nv_bfloat16 *__restrict__ w4,
@@ -351,6 +364,7 @@ __global__ void head_kernel(const __nv_bfloat16 *__restrict__ h3, const __nv_bfl
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x < 8) sq[threadIdx.x] = 0.0;
   __syncthreads();
+  pdl_wait();
   if (warp < rows) head_row(h3, w4, b4, t, y, dy, inv_b2, dz3, warp, lane, &sq[threadIdx.x >> 5]);
   if (!t) return;
   __syncthreads();
@@ -394,6 +408,7 @@ __device__ __forceinline__ __nv_bfloat16 adam_one(const AdamArgs &a, int i) {
 __global__ void __launch_bounds__(256) adam_kernel(const AdamArgs a) {
   __shared__ __nv_bfloat16 tile[32][34];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  pdl_wait();
   int t = blockIdx.x;
   for (int l = 0; l < 3; ++l) {
     const int n = a.K[l] / 32 * 16;
@@ -603,14 +618,14 @@ cudaError_t gather_std(const float *desc, const int *idx, int rows, int row0, co
                        const float *inv_sd, const float *labels, float ly_mu, float ly_inv,
                        __nv_bfloat16 *x, float *t, cudaStream_t s) {
   if (rows <= 0) return cudaSuccess;
-  gather_std_kernel<<<rows, 128, 0, s>>>(desc, idx, rows, row0, mu, inv_sd, labels, ly_mu, ly_inv, x, t);
-  return cudaGetLastError();
+  return launch_pdl(gather_std_kernel, dim3(rows), dim3(128), 0, s, desc, idx, rows, row0, mu, inv_sd, labels, ly_mu,
+                    ly_inv, x, t);
 }
 cudaError_t head(const __nv_bfloat16 *h3, const __nv_bfloat16 *w4, const float *b4, int rows,
                  const float *t, float *y, float *dy, float inv_b2, double *sse, __nv_bfloat16 *dz3,
                  cudaStream_t s) {
-  head_kernel<<<(rows * 32 + 255) / 256, 256, 0, s>>>(h3, w4, b4, rows, t, y, dy, inv_b2, sse, dz3);
-  return cudaGetLastError();
+  return launch_pdl(head_kernel, dim3((rows * 32 + 255) / 256), dim3(256), 0, s, h3, w4, b4, rows, t, y, dy, inv_b2,
+                    sse, dz3);
 }
 cudaError_t adam(float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb, __nv_bfloat16 *wt, float lr,
                  float b1, float b2, float eps, float c1, float c2, cudaStream_t s) {
@@ -630,8 +645,7 @@ cudaError_t adam(float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb
   }
   a.rest0[3] = o;  // W4 [512] and its bias
   a.rest1[3] = o + 513;
-  adam_kernel<<<ctas + 1, 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(adam_kernel, dim3(ctas + 1), dim3(256), 0, s, a);
 }
 cudaError_t to_bf16(const float *a, __nv_bfloat16 *b, int n, cudaStream_t s) {
   to_bf16_kernel<<<(n + 255) / 256 < 2048 ? (n + 255) / 256 : 2048, 256, 0, s>>>(a, b, n);

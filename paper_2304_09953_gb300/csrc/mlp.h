@@ -8,6 +8,32 @@
 namespace ligate {
 namespace mlp {
 
+// The kernels of a training step follow one another on one stream, each a few
+// microseconds long, so a launch's own latency counts: they are launched with
+// programmatic stream serialisation.  A kernel's CTAs may start while the one
+// before it drains, and pdl_wait (before the first access to memory that
+// another kernel writes or reads) holds them until it has finished.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+#endif
+
 enum { EPI_BIAS_RELU = 0, EPI_RELU_MASK = 1 };
 enum { GEMM_FWD = 0, GEMM_DGRAD = 1 };
 

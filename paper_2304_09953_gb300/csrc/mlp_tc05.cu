@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(128, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s.tmem_base;
+  pdl_wait();
 
   __shared__ int ok_shared;
   if (threadIdx.x == 0) {
@@ -541,9 +542,8 @@ cudaError_t gemm_tile(const __nv_bfloat16 *a, int M, int K, const __nv_bfloat16 
   cudaError_t e = cudaFuncSetAttribute(gemm_tc05_kernel<EPI, TN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        smem);
   if (e != cudaSuccess) return e;
-  gemm_tc05_kernel<EPI, TN, STAGES><<<dim3(N / TN, (M + TM - 1) / TM), 128, smem, s>>>(ta, tb, M, K, bias, mask, out,
-                                                                                     N, err);
-  return cudaGetLastError();
+  return launch_pdl(gemm_tc05_kernel<EPI, TN, STAGES>, dim3(N / TN, (M + TM - 1) / TM), dim3(128), smem, s, ta, tb, M, K,
+                    bias, mask, out, N, err);
 }
 
 template <int EPI>

@@ -94,24 +94,6 @@ __device__ __forceinline__ float wsum(float v) {
   return v;
 }
 
-// wsum of eight values at once: value q in lanes 4 q .. 4 q + 3.  Each value
-// goes through wsum's tree (lanes 16 apart first), so the sums are its bits.
-__device__ __forceinline__ float sum8(float v0, float v1, float v2, float v3, float v4, float v5, float v6, float v7,
-                                      int lane) {
-  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
-  auto half = [](bool up, float lo, float hi, int o) {  // keep lo (up: hi), add the partner lane's
-    const float keep = up ? hi : lo, give = up ? lo : hi;
-    return keep + __shfl_xor_sync(FULLM, give, o);
-  };
-  const float a0 = half(h16, v0, v4, 16), a1 = half(h16, v1, v5, 16), a2 = half(h16, v2, v6, 16),
-              a3 = half(h16, v3, v7, 16);
-  const float b0 = half(h8, a0, a2, 8), b1 = half(h8, a1, a3, 8);
-  float c = half(h4, b0, b1, 4);
-  c += __shfl_xor_sync(FULLM, c, 2);
-  c += __shfl_xor_sync(FULLM, c, 1);
-  return c;
-}
-
 __device__ __forceinline__ void unit_axis(const float4 &a, const float4 &b, float &nx, float &ny,
                                           float &nz) {
   nx = b.x - a.x; ny = b.y - a.y; nz = b.z - a.z;
@@ -247,7 +229,7 @@ __device__ float eval_state(const RefineArgs &a, const RSmem &w, const LigDesc &
     T0 += ry * gz - rz * gy; T1 += rz * gx - rx * gz; T2 += rx * gy - ry * gx;
     IR += rx * rx + ry * ry + rz * rz;
   }
-  const float s8 = sum8(fmaf(p.clash_w, cl, e), F0, F1, F2, T0, T1, T2, IR, lane);  // value lane >> 2 of the eight
+  const float s8 = warp_sum8(fmaf(p.clash_w, cl, e), F0, F1, F2, T0, T1, T2, IR, lane);  // value lane >> 2 of the eight
   const float E = __shfl_sync(FULLM, s8, 0);
   float *G = w.G + s * NG, *I = w.I + s * NI;
   __syncwarp();

@@ -27,11 +27,13 @@ namespace ligate {
 // every pair index from the start, atoms come from shared memory, and log1p of
 // the small counts comes from a table made by the same function: 100,000
 // ligands 409 -> 218 us (serialised), bound by instruction issue.
-constexpr int DESC_LOGS = 64;
+constexpr int DESC_LOGS = 64, DESC_SAME = 28 * 8;
 __global__ void __launch_bounds__(256) descriptor_kernel(const LigDesc *__restrict__ lig,
                                                          const float4 *__restrict__ atoms, int n_ligands,
                                                          float *__restrict__ out) {
-  __shared__ unsigned int hist[8][28 * 8 + 8];
+  // per warp: 28 x 8 pair bins, a bin group for pairs of equal type, 8 type counts
+  __shared__ unsigned int hist[8][DESC_SAME + 8 + 8];
+  __shared__ uint16_t first_bin[64];  // pair bins of types (ta, tb), either order
   __shared__ float4 xyz[8][LIGATE_MAX_ATOMS];
   __shared__ float logs[DESC_LOGS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -39,14 +41,18 @@ __global__ void __launch_bounds__(256) descriptor_kernel(const LigDesc *__restri
   unsigned int *h = hist[warp];
   float4 *a = xyz[warp];
   if (threadIdx.x < DESC_LOGS) logs[threadIdx.x] = log1pf((float)threadIdx.x);
-  for (int q = lane; q < 28 * 8 + 8; q += 32) h[q] = 0;
+  else if (threadIdx.x < DESC_LOGS + 64) {
+    const int q = threadIdx.x - DESC_LOGS, ta = min(q >> 3, q & 7), tb = max(q >> 3, q & 7);
+    first_bin[q] = ta == tb ? DESC_SAME : (ta * 8 - ta * (ta + 1) / 2 + (tb - ta - 1)) * 8;
+  }
+  for (int q = lane; q < DESC_SAME + 16; q += 32) h[q] = 0;
   __syncthreads();
   if (li >= n_ligands) return;
   const int base = lig[li].atom_base, n = lig[li].n_atoms, nrot = lig[li].n_rot;
   for (int i = lane; i < n; i += 32) {
     const float4 v = __ldg(atoms + base + i);
     a[i] = v;
-    atomicAdd(&h[224 + __float_as_int(v.w)], 1u);
+    atomicAdd(&h[DESC_SAME + 8 + __float_as_int(v.w)], 1u);
   }
   __syncwarp();
   const int npairs = n * (n - 1) / 2;
@@ -56,24 +62,21 @@ __global__ void __launch_bounds__(256) descriptor_kernel(const LigDesc *__restri
     const int up = n - 1 - r;  // pairs of row r; the rest of the folded row is row n - 2 - r
     const int i = c < up ? r : n - 2 - r, j = c < up ? r + 1 + c : n - 1 - r + c - up;
     const float4 x = a[i], y = a[j];
-    int ta = __float_as_int(x.w), tb = __float_as_int(y.w);
-    if (ta != tb) {
-      if (ta > tb) { const int t = ta; ta = tb; tb = t; }
-      const int p = ta * 8 - ta * (ta + 1) / 2 + (tb - ta - 1);
-      const float dx = __fsub_rn(x.x, y.x), dy = __fsub_rn(x.y, y.y), dz = __fsub_rn(x.z, y.z);
-      const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-      int bin = 0;
-      bin += d2 >= 2.25f; bin += d2 >= 9.0f; bin += d2 >= 20.25f; bin += d2 >= 36.0f;
-      bin += d2 >= 56.25f; bin += d2 >= 81.0f; bin += d2 >= 110.25f;
-      atomicAdd(&h[p * 8 + bin], 1u);
-    }
+    const float dx = __fsub_rn(x.x, y.x), dy = __fsub_rn(x.y, y.y), dz = __fsub_rn(x.z, y.z);
+    const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+    // bin: the squared edges (1.5 k)^2 not above d2, by bisection
+    const bool b4 = d2 >= 36.0f;
+    const bool b2 = d2 >= (b4 ? 81.0f : 9.0f);
+    const bool b1 = d2 >= (b4 ? (b2 ? 110.25f : 56.25f) : (b2 ? 20.25f : 2.25f));
+    const int bin = (b4 ? 4 : 0) + (b2 ? 2 : 0) + (b1 ? 1 : 0);
+    atomicAdd(&h[first_bin[__float_as_int(x.w) * 8 + __float_as_int(y.w)] + bin], 1u);
     c += 32;
     while (c >= n) { c -= n; ++r; }
   }
   __syncwarp();
   float *o = out + (size_t)li * 256;
   for (int q = lane; q < 256; q += 32) {
-    const unsigned cnt = q < 8 ? h[224 + q] : q < 232 ? h[q - 8] : q == 232 ? (unsigned)nrot : 0u;
+    const unsigned cnt = q < 8 ? h[DESC_SAME + 8 + q] : q < 232 ? h[q - 8] : q == 232 ? (unsigned)nrot : 0u;
     o[q] = cnt < DESC_LOGS ? logs[cnt] : log1pf((float)cnt);
   }
 }
