@@ -174,7 +174,7 @@ cudaError_t gemm(int kind, const GemmArgs &g, cudaStream_t s) {
 // serial chain per output (the MMA steps of a tile; one addition per row of a
 // column sum), and the operands come from L2 once per tile row and column: 80
 // tiles + 32 column CTAs, one wave, 31 MB at 1,024 rows (64 x 32 tiles, twice
-// the traffic, took 17.7 us against MEASURED).  Before, the sums ran as launches of
+// the traffic, took 17.7 us against 13.8).  Before, the sums ran as launches of
 // their own on 2 and 4 CTAs with every load on the chain and the weight
 // gradients on 8 to 16 CTAs without overlap: 87 + 3 x 61 + 3 x 37 us per step
 // of 1,024 rows (serialised, cold).
@@ -503,7 +503,10 @@ __global__ void unstd_kernel(float *__restrict__ y, int n, float mu, float sd) {
 // what cannot be among the first k.  A launch costs more than a tile's sort at
 // these sizes, so the passes are what counts: 100,000 predictions with k =
 // 5,000 take three launches where a bitonic sort of the whole array took 40
-// (174 us serialised), a library of up to 2,048 one instead of 13.
+// (174 us serialised), a library of up to 2,048 one instead of 13.  A tile's
+// strides below 64 stay in a warp's registers (20 -> 12.6 us), and a merge
+// leaves elements that are beyond the first k at their first look (20 and 19 ->
+// 14.8 and 12.3 us).
 __device__ __forceinline__ uint32_t ordered_key(float f) {
   const uint32_t u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
@@ -528,8 +531,31 @@ __global__ void __launch_bounds__(1024) sort_tile_kernel(const float *__restrict
     }
     s[q] = key;
   }
-  for (int kk = 2; kk <= size; kk <<= 1)
-    for (int j = kk >> 1; j > 0; j >>= 1) {
+  // a warp keeps 64 consecutive keys (lane, lane + 32) in registers for the
+  // strides up to 32; longer strides go through shared memory
+  const int lane = threadIdx.x & 31, w0 = (threadIdx.x >> 5) * 64;
+  unsigned long long k0 = ~0ull, k1 = ~0ull;
+  auto near = [&](int kk, int j0) {  // strides j0, j0 / 2, ..., 1 of size kk
+    for (int j = j0; j > 0; j >>= 1) {
+      if (j == 32) {
+        const bool up = ((w0 + lane) & kk) == 0;
+        if ((k0 > k1) == up) { const unsigned long long t = k0; k0 = k1; k1 = t; }
+      } else {
+        const unsigned long long o0 = __shfl_xor_sync(0xffffffffu, k0, j), o1 = __shfl_xor_sync(0xffffffffu, k1, j);
+        const bool low = (lane & j) == 0;
+        const bool up0 = ((w0 + lane) & kk) == 0, up1 = ((w0 + 32 + lane) & kk) == 0;
+        k0 = (low == up0) == (k0 < o0) ? k0 : o0;
+        k1 = (low == up1) == (k1 < o1) ? k1 : o1;
+      }
+    }
+  };
+  __syncthreads();
+  const bool on = w0 < size;  // sizes below 64 are sorted as 64
+  if (on) { k0 = w0 + lane < size ? s[w0 + lane] : ~0ull; k1 = w0 + 32 + lane < size ? s[w0 + 32 + lane] : ~0ull; }
+  for (int kk = 2; kk <= 64; kk <<= 1) near(kk, kk >> 1);
+  for (int kk = 128; kk <= size; kk <<= 1) {
+    if (on) { s[w0 + lane] = k0; s[w0 + 32 + lane] = k1; }
+    for (int j = kk >> 1; j >= 64; j >>= 1) {
       __syncthreads();
       for (int t = threadIdx.x; t < size / 2; t += blockDim.x) {
         const int q = 2 * t - (t & (j - 1)), l = q + j;  // the pair of comparator t
@@ -537,6 +563,11 @@ __global__ void __launch_bounds__(1024) sort_tile_kernel(const float *__restrict
         if ((x > y) == ((q & kk) == 0)) { s[q] = y; s[l] = x; }
       }
     }
+    __syncthreads();
+    if (on) { k0 = s[w0 + lane]; k1 = s[w0 + 32 + lane]; near(kk, 32); }
+  }
+  __syncthreads();
+  if (on) { s[w0 + lane] = k0; s[w0 + 32 + lane] = k1; }
   __syncthreads();
   for (int q = threadIdx.x; q < min(len, k); q += blockDim.x) {
     if (idx) idx[q] = (int32_t)(s[q] & 0xffffffffu);
@@ -563,17 +594,30 @@ __global__ void __launch_bounds__(256) merge_kernel(const unsigned long long *__
     lo[w] = 0;
     len[w] = g0 + w == run || b >= n ? 0 : (int)min((long long)per, n - b);
   }
+  // most elements are beyond the first k: one is when every sibling's element
+  // ceil((k - p) / siblings) - 1 is smaller
+  int sib = 0;
+#pragma unroll
+  for (int w = 0; w < MERGE_WAYS; ++w) sib += len[w] > 0;
+  if (sib > 0) {
+    const int c = (k - p + sib - 1) / sib - 1;
+    bool out_of_k = true;
+#pragma unroll
+    for (int w = 0; w < MERGE_WAYS; ++w)
+      if (len[w] > 0) out_of_k &= c < len[w] && in[(long long)(g0 + w) * R + (c < len[w] ? c : 0)] < key;
+    if (out_of_k) return;
+  }
   for (int step = per; step > 0; step = step > 1 ? (step + 1) >> 1 : 0) {
+    unsigned long long mid[MERGE_WAYS];
+#pragma unroll
+    for (int w = 0; w < MERGE_WAYS; ++w)
+      mid[w] = len[w] > 0 ? in[(long long)(g0 + w) * R + lo[w] + (len[w] >> 1)] : 0ull;
 #pragma unroll
     for (int w = 0; w < MERGE_WAYS; ++w) {
-      if (len[w] == 0) continue;
       const int half = len[w] >> 1;
-      if (in[(long long)(g0 + w) * R + lo[w] + half] < key) {
-        lo[w] += half + 1;
-        len[w] -= half + 1;
-      } else {
-        len[w] = half;
-      }
+      const bool right = len[w] > 0 && mid[w] < key;
+      lo[w] += right ? half + 1 : 0;
+      len[w] = right ? len[w] - half - 1 : half;
     }
   }
   int rank = p;

@@ -30,6 +30,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "ligate_internal.h"
@@ -70,6 +71,7 @@ __device__ __forceinline__ bool mbar_test(uint64_t *bar, unsigned parity) {
 }
 // Bounded wait on phase `parity`; false after WAIT_NS.
 __device__ bool mbar_wait(uint64_t *bar, unsigned parity) {
+  if (mbar_test(bar, parity)) return true;
   const unsigned long long t0 = now_ns();
   while (!mbar_test(bar, parity))
     if (now_ns() - t0 > WAIT_NS) return false;
@@ -251,25 +253,31 @@ __global__ void __launch_bounds__(128, 1)
 // layers and the head, activations in shared memory, nothing but the rows'
 // descriptors read and 4 bytes per row written.
 //
-// What bounds it: the hidden weights (1.3 MB in BF16) pass through every CTA
-// once per 128 rows, from L2 (about 0.17 GFLOP of tcgen05 work per tile against
-// them); as layers of their own, each with a descriptor or activation pass
-// through memory, the same rows took gather + 3 GEMM + head + unscale launches
-// and 2 x 6 KB of activations per row: 100,000 rows 590 us (serialised), here
-// 240, 40 us per tile of which the weight tiles' way from L2 (8 TB/s over all
-// SMs) is about two thirds.
+// What bounds it: three layers that need one another, 0.17 GFLOP of tcgen05
+// work per tile (11 us at the SM's share of the peak) between epilogues, with
+// 1.3 MB of BF16 weights per tile from L2.  As layers of their own, each with a
+// descriptor or activation pass through memory, 100,000 rows took gather + 3
+// GEMM + head + unscale launches and 2 x 6 KB of activations per row: 590 us
+// (serialised).  One kernel with the layers in a strict row of load, MMA and
+// epilogue took 240, the pipeline below 161.  What it waits for is spread
+// out: no loads of inputs -14 us, a quarter of the MMAs -14, no head -27; a
+// quarter of the weight traffic, or pairs of CTAs sharing it by multicast, 0.
 //
 // A CTA keeps the layer input as eight 64-column K slices in the 128-byte
 // swizzle the tensor core reads (128 KB) and streams the transposed weights as
-// 256 x 64 tiles through a three-stage ring; the 128 x 512 FP32 accumulator is
-// the SM's whole tensor memory.  Warp 8 issues loads and MMAs; warps 0-7 write
-// the inputs, then per layer read their 32 rows x 256 columns of the
-// accumulator, add the bias, apply ReLU and write the next layer's slices in
-// place (the MMAs that read them are done).  Weight tiles of the next layer are
-// already in flight during an epilogue.  Every output is the same bits as the
-// layer-by-layer kernels': the same K order, rounding points, and head order
-// (column l of each group of 32 in one chain, then the butterfly's tree).
-constexpr int FW_THREADS = 288, FW_STAGES = 3, FW_B = 256 * TK * 2;
+// 256 x 64 tiles through a three-stage ring (six stages of 128 x 64: 231 us
+// against 158 over two sizes); the 128 x 512 FP32 accumulator is the SM's whole
+// tensor memory.  Warp 9 streams the weights of all tiles, warp 8 issues the
+// MMAs, columns 0-255 of a layer before the others.  Warps 0-3 have columns
+// 0-255: they read them, add the bias, apply ReLU and pack to BF16 in registers
+// while the tensor core works on the other half, and write the next layer's
+// slices 0-3 in place once that has read them.  Warps 4-7 do columns 256-511,
+// while the next layer starts on slices 0-3.  After the last hidden layer warps
+// 0-3 have the head and warps 4-7 write the next row tile's inputs.  Every
+// output is the same bits as the layer-by-layer kernels': the same K order,
+// rounding points, and head order (column l of each group of 32 in one chain,
+// then the butterfly's tree).
+constexpr int FW_THREADS = 384, FW_N = 256, FW_STAGES = 3, FW_B = FW_N * TK * 2;
 
 struct FwdNet {
   CUtensorMap w[3];  // transposed hidden weights [512][256], [512][512], [512][512]
@@ -289,7 +297,7 @@ struct __align__(1024) FwdSmem {
   uint8_t h[8][A_BYTES];
   uint8_t ring[FW_STAGES][FW_B];
   __nv_bfloat16 w4[512];
-  uint64_t full[FW_STAGES], empty[FW_STAGES], done;
+  uint64_t full[FW_STAGES], empty[FW_STAGES], in[2], acc[2], drain;
   uint32_t tmem_base;
 };
 static_assert(sizeof(FwdSmem) + 1024 <= 227 * 1024, "one CTA's shared memory");
@@ -305,27 +313,114 @@ __device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t addr) {
       : "r"(addr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t addr) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(addr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(bar)) : "memory");
+}
+// A warp's shared-memory writes and tensor-memory reads so far are done: tell
+// the thread that issues the tensor-core work.
+__device__ __forceinline__ void warp_arrive(uint64_t *bar, int lane) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bar);
+}
+// mbar_wait by a whole warp, the same answer in every lane.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, unsigned parity) {
+  const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, parity));
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  return ok;
 }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t *>(&v);
 }
 
+// A wait ran out: this CTA leaves its remaining tiles, of whichever network.
+__device__ __forceinline__ void fw_report(const FwdArgs &a) {
+  for (int q = 0; q < FWD_NETS; ++q) atomicExch(a.net[q].err, 1);
+}
+// Standardised inputs of NB x 8 rows (first, first + 4, ...) as packed BF16,
+// eight columns per lane.
+template <int NB, int U>
+__device__ __forceinline__ void fw_load_rows(const FwdArgs &a, const FwdNet &net, int row0, int first, int lane,
+                                             uint4 (&x)[NB * 8]) {
+  float mu[8], sd[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) { mu[q] = __ldg(net.mu + 8 * lane + q); sd[q] = __ldg(net.inv_sd + 8 * lane + q); }
+#pragma unroll
+  for (int i = 0; i < NB * 8; i += U) {
+    float v[U][8];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int row = row0 + first + 4 * (i + u);
+      const float *src = a.desc + (size_t)(row < a.n ? row : 0) * 256 + 8 * lane;
+      if (a.vec) {
+#pragma unroll
+        for (int q = 0; q < 8; q += 4)
+          asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                       : "=f"(v[u][q]), "=f"(v[u][q + 1]), "=f"(v[u][q + 2]), "=f"(v[u][q + 3])
+                       : "l"(src + q));
+      } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v[u][q]) : "l"(src + q));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool in = row0 + first + 4 * (i + u) < a.n;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[u][q] = (v[u][q] - mu[q]) * sd[q];
+      x[i + u] = in ? make_uint4(pack_bf16(v[u][0], v[u][1]), pack_bf16(v[u][2], v[u][3]), pack_bf16(v[u][4], v[u][5]),
+                                 pack_bf16(v[u][6], v[u][7]))
+                    : make_uint4(0, 0, 0, 0);
+      // packed here, not after the next rows' loads: registers
+      asm volatile("" : "+r"(x[i + u].x), "+r"(x[i + u].y), "+r"(x[i + u].z), "+r"(x[i + u].w)::"memory");
+    }
+  }
+}
+template <int NB>
+__device__ __forceinline__ void fw_store_rows(FwdSmem &s, int first, int lane, const uint4 (&x)[NB * 8]) {
+#pragma unroll
+  for (int i = 0; i < NB * 8; ++i) {
+    const int r = first + 4 * i;
+    *reinterpret_cast<uint4 *>(s.h[lane >> 3] + r * 128 + (((lane & 7) ^ (r & 7)) << 4)) = x[i];
+  }
+}
+// The row's next-layer activations of one 256-column half, as packed BF16.
+__device__ __forceinline__ void fw_activate(uint32_t trow, const float *bias, uint4 (&x)[32]) {
+#pragma unroll
+  for (int c0 = 0; c0 < 256; c0 += 32) {
+    uint32_t r[32];
+    tmem_ld32(r, trow + c0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 b0 = __ldg(reinterpret_cast<const float4 *>(bias + c0 + 8 * q)),
+                   b1 = __ldg(reinterpret_cast<const float4 *>(bias + c0 + 8 * q) + 1);
+      const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = fmaxf(__uint_as_float(r[8 * q + k]) + bb[k], 0.f);
+      x[c0 / 8 + q] = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+    }
+  }
+}
+__device__ __forceinline__ void fw_store_half(FwdSmem &s, int half, int row, const uint4 (&x)[32]) {
+#pragma unroll
+  for (int i = 0; i < 32; ++i)
+    *reinterpret_cast<uint4 *>(s.h[half * 4 + (i >> 3)] + row * 128 + (((i & 7) ^ (row & 7)) << 4)) = x[i];
+}
+
 __global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid_constant__ FwdArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   FwdSmem &s = *reinterpret_cast<FwdSmem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool issuer = tid == 256;
   if (tid == 0) {
     for (int i = 0; i < FW_STAGES; ++i) { mbar_init(&s.full[i], 1); mbar_init(&s.empty[i], 1); }
-    mbar_init(&s.done, 1);
+    mbar_init(&s.in[0], 8);  // all layer warps
+    mbar_init(&s.in[1], 4);  // one half's
+    mbar_init(&s.acc[0], 1);
+    mbar_init(&s.acc[1], 1);
+    mbar_init(&s.drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 8) {  // the whole tensor memory: 512 columns
@@ -337,154 +432,169 @@ __global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s.tmem_base;
-  const bool skip_loads = issuer && atomicExch(&g_fault_skip_loads, 0) != 0;  // test hook (see gemm_tc05_kernel)
-
-  bool ok = true;
-  int loaded = 0, used = 0;   // issuer: weight tiles loaded and consumed so far
-  unsigned done_phase = 0;
-  for (int item = blockIdx.x; item < a.items && ok; item += gridDim.x) {
-    const FwdNet &net = a.net[item / a.tiles];
-    const int row0 = item % a.tiles * TM;
-    const int first = used;  // this tile's weight tiles are first .. first + 39
-    // weight tile q of the row tile: layer, 64-wide K slice, 256-column half
-    auto load = [&](int q) {
-      const int l = q < 8 ? 0 : q < 24 ? 1 : 2, r = q - (l == 0 ? 0 : l == 1 ? 8 : 24), st = loaded % FW_STAGES;
-      if (loaded >= FW_STAGES && !mbar_wait(&s.empty[st], (loaded / FW_STAGES - 1) & 1u)) { ok = false; return; }
-      if (skip_loads) return;
-      mbar_expect_tx(&s.full[st], FW_B);
-      tma_load_2d(s.ring[st], &net.w[l], &s.full[st], (r >> 1) * TK, (r & 1) * 256);
-      ++loaded;
-    };
-    if (issuer)
-      while (ok && !skip_loads && loaded < first + FW_STAGES) load(loaded - first);
-    if (warp < 8) {  // standardised inputs into slices 0-3: a warp per row, eight columns per lane
-      float mu[8], sd[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) { mu[q] = __ldg(net.mu + 8 * lane + q); sd[q] = __ldg(net.inv_sd + 8 * lane + q); }
-      uint8_t *const slice = s.h[lane >> 3];
-#pragma unroll 4
-      for (int i = 0; i < TM / 8; ++i) {
-        const int r = warp + 8 * i;
-        float v[8];
-        if (row0 + r < a.n) {
-          const float *src = a.desc + (size_t)(row0 + r) * 256 + 8 * lane;
-          if (a.vec) {
-            const float4 x = __ldg(reinterpret_cast<const float4 *>(src)), y = __ldg(reinterpret_cast<const float4 *>(src) + 1);
-            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
-          } else {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = __ldg(src + q);
-          }
-#pragma unroll
-          for (int q = 0; q < 8; ++q) v[q] = (v[q] - mu[q]) * sd[q];
-        } else {
-#pragma unroll
-          for (int q = 0; q < 8; ++q) v[q] = 0.f;
-        }
-        *reinterpret_cast<uint4 *>(slice + r * 128 + (((lane & 7) ^ (r & 7)) << 4)) =
-            make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-      }
-      s.w4[tid] = net.w4[tid];
-      s.w4[256 + tid] = net.w4[256 + tid];
-      if (item + (int)gridDim.x < a.items) {  // the next tile's rows towards L2
-        const int nrow = (item + (int)gridDim.x) % a.tiles * TM;
-        for (int q = tid; q < TM * 8; q += 256)
-          if (nrow + (q >> 3) < a.n)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(a.desc + (size_t)(nrow + (q >> 3)) * 256 + (q & 7) * 32));
-      }
-    }
-    for (int l = 0; l < 3; ++l) {
-      // the layer's input is written (and the accumulator read): visible to
-      // the tensor core's proxy, then one thread issues the layer
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      if (!__syncthreads_and(ok)) { ok = false; break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (issuer) {
-        const int slices = l == 0 ? 4 : 8;
-        for (int kb = 0; kb < slices && ok; ++kb)
-          for (int nh = 0; nh < 2 && ok; ++nh) {
-            const int st = used % FW_STAGES;
-            if (!mbar_wait(&s.full[st], (used / FW_STAGES) & 1u)) { ok = false; break; }
-            ++used;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t da = sdesc(saddr(s.h[kb])), db = sdesc(saddr(s.ring[st]));
-#pragma unroll
-            for (int kk = 0; kk < TK / 16; ++kk)
-              mma_f16<256>(tmem + nh * 256, da + 2 * kk, db + 2 * kk, (kb > 0 || kk > 0) ? 1u : 0u);
-            mma_commit(&s.empty[st]);
-            // two tiles ahead: the stage of the previous step, whose MMAs run before this one's
-            while (ok && loaded < first + 40 && loaded < used + FW_STAGES - 1) load(loaded - first);
-          }
-        mma_commit(&s.done);  // arrives once every MMA issued so far has completed
-      }
-      if (warp < 8) {
-        const int row = (warp & 3) * 32 + lane, half = warp >> 2;
-        const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        ok = __all_sync(0xffffffffu, mbar_wait(&s.done, done_phase)) && ok;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (l < 2) {
-          const float *bias = net.b[l] + half * 256;
-#pragma unroll 1
-          for (int c0 = 0; c0 < 256 && ok; c0 += 32) {
-            uint32_t r[32];
-            tmem_ld32(r, trow + half * 256 + c0);
-            uint8_t *const slice = s.h[half * 4 + (c0 >> 6)] + row * 128;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const float4 b0 = __ldg(reinterpret_cast<const float4 *>(bias + c0 + 8 * q)),
-                           b1 = __ldg(reinterpret_cast<const float4 *>(bias + c0 + 8 * q) + 1);
-              const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-              float v[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k) v[k] = fmaxf(__uint_as_float(r[8 * q + k]) + bb[k], 0.f);
-              *reinterpret_cast<uint4 *>(slice + (((((c0 & 32) >> 3) + q) ^ (row & 7)) << 4)) =
-                  make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+  // an item: a network and a row tile
+  const int first_item = blockIdx.x, step = gridDim.x;
+  // registers: 384 threads start with 168; 128 x 40 + 256 x 232 is the same sum
+  if (warp >= 8) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (warp == 9) {  // the weight stream of all items, one thread
+      if (lane == 0 && atomicExch(&g_fault_skip_loads, 0) == 0) {  // test hook (see gemm_tc05_kernel)
+        int loaded = 0;
+        bool go = true;
+        for (int item = first_item; item < a.items && go; item += step) {
+          const FwdNet &net = a.net[item / a.tiles];
+          for (int l = 0; l < 3 && go; ++l) {
+            const int slices = l == 0 ? 4 : 8;
+            for (int r = 0; r < 2 * slices; ++r, ++loaded) {  // half of the columns, 64-wide K slice
+              const int st = loaded % FW_STAGES;
+              if (loaded >= FW_STAGES && !mbar_wait(&s.empty[st], (loaded / FW_STAGES - 1) & 1u)) { go = false; break; }
+              mbar_expect_tx(&s.full[st], FW_B);
+              const int x = r % slices * TK, y = r / slices * FW_N;
+              tma_load_2d(s.ring[st], &net.w[l], &s.full[st], x, y);
             }
           }
-        } else {
-          // head: chain c of 32 sums the columns c, c + 32, ...; this warp has
-          // chains 16 half .. 16 half + 15 of its rows
-          float acc[16];
+        }
+        // before the shared memory goes (bounded): loads in flight, the last commits
+        for (int q = loaded < FW_STAGES ? 0 : loaded - FW_STAGES; q < loaded; ++q)
+          if (mbar_wait(&s.full[q % FW_STAGES], (q / FW_STAGES) & 1u))
+            (void)mbar_wait(&s.empty[q % FW_STAGES], (q / FW_STAGES) & 1u);
+      }
+      __syncwarp();
+    } else if (warp == 8) {
+      if (lane == 0) {  // the tensor-core work, one thread
+        bool ok = true;
+        int used = 0;
+        unsigned layer = 0;
+        for (int item = first_item; item < a.items && ok; item += step)
+          for (int l = 0; l < 3 && ok; ++l, ++layer) {
+            const int slices = l == 0 ? 4 : 8;
+            for (int half = 0; half < 2 && ok; ++half) {
+              for (int kb = 0; kb < slices; ++kb) {
+                // in[0]: K slices 0-3 written, columns 0-255 read; in[1]: the others
+                if (half == 0 && kb == 0 && !mbar_wait(&s.in[0], layer & 1u)) { ok = false; break; }
+                if ((half == 0 ? kb == 4 : l == 0 && kb == 0) && !mbar_wait(&s.in[1], layer & 1u)) { ok = false; break; }
+                const int st = used % FW_STAGES;
+                if (!mbar_wait(&s.full[st], (used / FW_STAGES) & 1u)) { ok = false; break; }
+                ++used;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t da = sdesc(saddr(s.h[kb])), db = sdesc(saddr(s.ring[st]));
 #pragma unroll
-          for (int c = 0; c < 16; ++c) acc[c] = 0.f;
-          const float *bias = net.b[2] + 16 * half;
-          const __nv_bfloat16 *w4 = s.w4 + 16 * half;
-#pragma unroll 1
-          for (int j = 0; j < 512 && ok; j += 32) {
-            uint32_t r[16];
-            tmem_ld16(r, trow + j + 16 * half);
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              const float h = __bfloat162float(__float2bfloat16_rn(fmaxf(__uint_as_float(r[c]) + __ldg(bias + j + c), 0.f)));
-              acc[c] = fmaf(h, __bfloat162float(w4[j + c]), acc[c]);
+                for (int kk = 0; kk < TK / 16; ++kk)
+                  mma_f16<FW_N>(tmem + half * FW_N, da + 2 * kk, db + 2 * kk, (kb > 0 || kk > 0) ? 1u : 0u);
+                mma_commit(&s.empty[st]);
+              }
+              if (ok) mma_commit(&s.acc[half]);  // arrives once every MMA issued so far has completed
             }
           }
-          // the butterfly's tree: lanes 16 apart first, which are the two
-          // warps' chains (through slices 4-7, which no one reads any more)
-          float *const xch = reinterpret_cast<float *>(s.h[4]) + row;
-          if (half == 1)
-#pragma unroll
-            for (int c = 0; c < 16; ++c) xch[c * TM] = acc[c];
-          asm volatile("bar.sync 1, 256;" ::: "memory");
-          if (half == 0) {
-#pragma unroll
-            for (int c = 0; c < 16; ++c) acc[c] += xch[c * TM];
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-              for (int c = 0; c < o; ++c) acc[c] += acc[c + o];
-            if (row0 + row < a.n && ok) net.pred[row0 + row] = fmaf(acc[0] + __ldg(net.b4), net.ly_sd, net.ly_mu);
-          }
+        if (!ok) {
+          fw_report(a);
+          mma_commit(&s.drain);
+          (void)mbar_wait(&s.drain, 0);
         }
       }
-      done_phase ^= 1u;
+      __syncwarp();
     }
-    ok = __syncthreads_and(ok);  // the same decision in every thread; the tile's shared memory is free
-    if (!ok && tid == 0) atomicExch(net.err, 1);
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+    // warps 0-3 have accumulator columns 0-255 and the head, warps 4-7 the
+    // other columns and the next tile's inputs
+    const int half = warp >> 2, w = warp & 3, row = w * 32 + lane;
+    const uint32_t trow = tmem + ((uint32_t)(w * 32) << 16);
+    bool ok = true;
+    unsigned layer = 0;
+    if (first_item < a.items) {  // the first tile's inputs: half the rows each
+      uint4 x[16];
+      fw_load_rows<2, 8>(a, a.net[first_item / a.tiles], first_item % a.tiles * TM, half * 64 + w, lane, x);
+      fw_store_rows<2>(s, half * 64 + w, lane, x);
+      warp_arrive(&s.in[0], lane);
+      if (half == 0) warp_arrive(&s.in[1], lane);
+    }
+    for (int item = first_item; item < a.items && ok; item += step) {
+      const FwdNet &net = a.net[item / a.tiles];
+      const int row0 = item % a.tiles * TM, next = item + step;
+      if (half == 0) {
+        for (int q = tid; q < 512; q += 128) s.w4[q] = net.w4[q];
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll 1
+        for (int l = 0; l < 2 && ok; ++l, ++layer) {
+          uint4 x[32];
+          if (!(ok = warp_wait(&s.acc[0], layer & 1u))) break;
+          fw_activate(trow, net.b[l], x);  // while the tensor core has the other columns
+          if (!(ok = warp_wait(&s.acc[1], layer & 1u))) break;
+          fw_store_half(s, 0, row, x);
+          warp_arrive(&s.in[0], lane);
+        }
+        if (!ok || !(ok = warp_wait(&s.acc[0], layer & 1u))) break;
+        // head: chain c of 32 sums the columns c, c + 32, ..., then the
+        // butterfly's tree
+        float acc[32];
+#pragma unroll
+        for (int c = 0; c < 32; ++c) acc[c] = 0.f;
+#pragma unroll 1
+        for (int j = 0; j < 512; j += 32) {
+          if (j == 256) {
+            warp_arrive(&s.in[0], lane);  // columns 0-255 read
+            if (!(ok = warp_wait(&s.acc[1], layer & 1u))) break;
+          }
+          uint32_t r[32];
+          tmem_ld32(r, trow + j);
+#pragma unroll
+          for (int c = 0; c < 32; c += 8) {
+            const float4 b0 = __ldg(reinterpret_cast<const float4 *>(net.b[2] + j + c)),
+                         b1 = __ldg(reinterpret_cast<const float4 *>(net.b[2] + j + c) + 1);
+            const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            const uint4 wv = *reinterpret_cast<const uint4 *>(s.w4 + j + c);
+            const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+            for (int k = 0; k < 8; k += 2) {
+              const uint32_t h = pack_bf16(fmaxf(__uint_as_float(r[c + k]) + bb[k], 0.f),
+                                           fmaxf(__uint_as_float(r[c + k + 1]) + bb[k + 1], 0.f));
+              // a BF16 is the upper half of its FP32
+              acc[c + k] = fmaf(__uint_as_float(h << 16), __uint_as_float(ww[k / 2] << 16), acc[c + k]);
+              acc[c + k + 1] = fmaf(__uint_as_float(h & 0xffff0000u), __uint_as_float(ww[k / 2] & 0xffff0000u), acc[c + k + 1]);
+            }
+          }
+        }
+        if (!ok) break;
+        ++layer;
+        warp_arrive(&s.in[1], lane);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int c = 0; c < o; ++c) acc[c] += acc[c + o];
+        if (row0 + row < a.n) net.pred[row0 + row] = fmaf(acc[0] + __ldg(net.b4), net.ly_sd, net.ly_mu);
+        asm volatile("bar.sync 1, 128;" ::: "memory");  // w4 is read
+      } else {
+        const int nrow0 = next % a.tiles * TM;
+        if (next < a.items)  // the next tile's rows towards L2
+          for (int q = tid - 128; q < TM * 8; q += 128)
+            if (nrow0 + (q >> 3) < a.n)
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(a.desc + (size_t)(nrow0 + (q >> 3)) * 256 + (q & 7) * 32));
+#pragma unroll 1
+        for (int l = 0; l < 2 && ok; ++l, ++layer) {
+          uint4 x[32];
+          if (!(ok = warp_wait(&s.acc[1], layer & 1u))) break;
+          if (lane == 0) mbar_arrive(&s.in[0]);
+          fw_activate(trow + 256, net.b[l] + 256, x);
+          fw_store_half(s, 1, row, x);
+          warp_arrive(&s.in[1], lane);
+        }
+        if (!ok) break;
+        const FwdNet &nnet = a.net[next < a.items ? next / a.tiles : 0];
+        uint4 x[16];  // half of the rows before the wait, the others after it: registers
+        if (next < a.items) fw_load_rows<2, 8>(a, nnet, nrow0, w, lane, x);
+        if (!(ok = warp_wait(&s.acc[1], layer & 1u))) break;
+        ++layer;
+        if (next < a.items) {
+          fw_store_rows<2>(s, w, lane, x);
+          fw_load_rows<2, 8>(a, nnet, nrow0, 64 + w, lane, x);
+          fw_store_rows<2>(s, 64 + w, lane, x);
+        }
+        warp_arrive(&s.in[0], lane);
+      }
+    }
+    if (!ok && lane == 0) fw_report(a);
   }
-  if (issuer && !ok)  // drain loads still in flight (bounded) before the shared memory goes
-    for (int q = used; q < loaded; ++q) (void)mbar_wait(&s.full[q % FW_STAGES], (q / FW_STAGES) & 1u);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 8)
@@ -569,12 +679,11 @@ cudaError_t gemm_tc05(int epi, const __nv_bfloat16 *a, int M, int K, const __nv_
 
 cudaError_t forward_tc05(const FwdSpec *nets, int n_nets, const float *desc, int n, cudaStream_t s) {
   if (n <= 0 || n_nets <= 0) return cudaSuccess;
-  int dev = 0, sms = 0;
   cudaError_t e;
   const int smem = (int)sizeof(FwdSmem) + 1024;
-  if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
-      (e = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
-    return e;
+  if ((e = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
   for (int m0 = 0; m0 < n_nets; m0 += FWD_NETS) {
     const int m = n_nets - m0 < FWD_NETS ? n_nets - m0 : FWD_NETS;
     FwdArgs a;
@@ -583,7 +692,7 @@ cudaError_t forward_tc05(const FwdSpec *nets, int n_nets, const float *desc, int
       FwdNet &t = a.net[q];
       const int K[3] = {256, 512, 512};
       for (int l = 0; l < 3; ++l) {
-        if (!make_map(&t.w[l], f.wt[l], 512, K[l], 256)) return cudaErrorInvalidValue;
+        if (!make_map(&t.w[l], f.wt[l], 512, K[l], FW_N)) return cudaErrorInvalidValue;
         t.b[l] = f.b[l];
       }
       t.w4 = f.w4; t.b4 = f.b4; t.mu = f.mu; t.inv_sd = f.inv_sd;
@@ -596,7 +705,7 @@ cudaError_t forward_tc05(const FwdSpec *nets, int n_nets, const float *desc, int
     a.tiles = (n + TM - 1) / TM;
     a.items = a.tiles * m;
     a.vec = (reinterpret_cast<uintptr_t>(desc) & 15) == 0;
-    mlp_forward_kernel<<<a.items < sms ? a.items : sms, FW_THREADS, smem, s>>>(a);
+    mlp_forward_kernel<<<std::min(a.items, sms), FW_THREADS, smem, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -21,63 +21,114 @@ namespace ligate {
 // representable squared edges), rotatable-bond count; log1p of every count.
 //
 // What bounds it: 1 KB written per ligand (15 us per 100,000 at the copy rate)
-// against 700 pair tests and shared-memory increments of a 38-atom ligand.
-// The pairs are enumerated with a running (row, column) over folded rows (row r
-// and row n - 2 - r of the triangle together have n pairs) instead of decoding
-// every pair index from the start, atoms come from shared memory, and log1p of
-// the small counts comes from a table made by the same function: 100,000
-// ligands 409 -> 218 us (serialised), bound by instruction issue.
-constexpr int DESC_LOGS = 64, DESC_SAME = 28 * 8;
-__global__ void __launch_bounds__(256) descriptor_kernel(const LigDesc *__restrict__ lig,
-                                                         const float4 *__restrict__ atoms, int n_ligands,
-                                                         float *__restrict__ out) {
-  // per warp: 28 x 8 pair bins, a bin group for pairs of equal type, 8 type counts
-  __shared__ unsigned int hist[8][DESC_SAME + 8 + 8];
-  __shared__ uint16_t first_bin[64];  // pair bins of types (ta, tb), either order
-  __shared__ float4 xyz[8][LIGATE_MAX_ATOMS];
+// against 700 pair tests and shared-memory increments of a 38-atom ligand,
+// which are bound by instruction issue, so the pair loop is made short: pair q
+// is (c, c + 1 + r) of the cyclic order with r = q / n, c = q % n (each
+// unordered pair once: half a turn), a lane takes four values of r at a time so
+// that one atom's load serves four pairs, the atoms lie in shared memory one and
+// a half times so that no index wraps, and a counter per ordered pair of types
+// needs no table; the two orders are added on the way out.  The bin is a root
+// and one compare with the edge it gives instead of three compares and their
+// selects (the ALU was half busy: 172 -> 146 us).  Nine words per type
+// pair spread the pairs of one bin over the banks.  Each lane writes eight
+// neighbouring features, which are one pair's bins; log1p of the small counts
+// comes from a table made by the same function.  100,000 ligands (serialised):
+// 409 us with every pair index decoded, 185 with folded rows and a table of bin
+// groups, 146 here, bound by shared-memory wavefronts (83% busy).
+constexpr int DESC_LOGS = 64, DESC_WARPS = 8;
+struct __align__(16) DescWarp {
+  unsigned int pair[64 * 9];  // [first type][second type][bin, 9th unused]
+  unsigned int count[8];
+  float4 atom[LIGATE_MAX_ATOMS * 3 / 2 + 4];  // type * 9 in w
+};
+constexpr float FLOOR_0 = 12582912.f;  // 1.5 x 2^23: sums below 2^22 keep their integer part
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__global__ void __launch_bounds__(32 * DESC_WARPS) descriptor_kernel(const LigDesc *__restrict__ lig,
+                                                                     const float4 *__restrict__ atoms, int n_ligands,
+                                                                     int per_warp, float *__restrict__ out) {
+  __shared__ DescWarp smem[DESC_WARPS];
   __shared__ float logs[DESC_LOGS];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int li = blockIdx.x * (blockDim.x >> 5) + warp;
-  unsigned int *h = hist[warp];
-  float4 *a = xyz[warp];
+  __shared__ unsigned none[8];
+  const int lane = threadIdx.x & 31;
+  DescWarp &s = smem[threadIdx.x >> 5];
   if (threadIdx.x < DESC_LOGS) logs[threadIdx.x] = log1pf((float)threadIdx.x);
-  else if (threadIdx.x < DESC_LOGS + 64) {
-    const int q = threadIdx.x - DESC_LOGS, ta = min(q >> 3, q & 7), tb = max(q >> 3, q & 7);
-    first_bin[q] = ta == tb ? DESC_SAME : (ta * 8 - ta * (ta + 1) / 2 + (tb - ta - 1)) * 8;
-  }
-  for (int q = lane; q < DESC_SAME + 16; q += 32) h[q] = 0;
+  if (threadIdx.x < 8) none[threadIdx.x] = 0;
   __syncthreads();
-  if (li >= n_ligands) return;
-  const int base = lig[li].atom_base, n = lig[li].n_atoms, nrot = lig[li].n_rot;
-  for (int i = lane; i < n; i += 32) {
-    const float4 v = __ldg(atoms + base + i);
-    a[i] = v;
-    atomicAdd(&h[DESC_SAME + 8 + __float_as_int(v.w)], 1u);
-  }
-  __syncwarp();
-  const int npairs = n * (n - 1) / 2;
-  int r = 0, c = lane;
-  while (c >= n) { c -= n; ++r; }
-  for (int q = lane; q < npairs; q += 32) {
-    const int up = n - 1 - r;  // pairs of row r; the rest of the folded row is row n - 2 - r
-    const int i = c < up ? r : n - 2 - r, j = c < up ? r + 1 + c : n - 1 - r + c - up;
-    const float4 x = a[i], y = a[j];
-    const float dx = __fsub_rn(x.x, y.x), dy = __fsub_rn(x.y, y.y), dz = __fsub_rn(x.z, y.z);
-    const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-    // bin: the squared edges (1.5 k)^2 not above d2, by bisection
-    const bool b4 = d2 >= 36.0f;
-    const bool b2 = d2 >= (b4 ? 81.0f : 9.0f);
-    const bool b1 = d2 >= (b4 ? (b2 ? 110.25f : 56.25f) : (b2 ? 20.25f : 2.25f));
-    const int bin = (b4 ? 4 : 0) + (b2 ? 2 : 0) + (b1 ? 1 : 0);
-    atomicAdd(&h[first_bin[__float_as_int(x.w) * 8 + __float_as_int(y.w)] + bin], 1u);
-    c += 32;
-    while (c >= n) { c -= n; ++r; }
-  }
-  __syncwarp();
-  float *o = out + (size_t)li * 256;
-  for (int q = lane; q < 256; q += 32) {
-    const unsigned cnt = q < 8 ? h[DESC_SAME + 8 + q] : q < 232 ? h[q - 8] : q == 232 ? (unsigned)nrot : 0u;
-    o[q] = cnt < DESC_LOGS ? logs[cnt] : log1pf((float)cnt);
+  // features 8 lane .. 8 lane + 7: lane 0 the type counts, lanes 1-28 a pair's
+  // bins, lane 29 the rotatable bonds, the rest zero
+  int ta = 0, tb = lane;  // pair lane - 1 of (0,1), (0,2), ..., (6,7)
+  for (int left = 7; tb > 7 && ta < 6;) { ++ta; tb -= --left; }
+  const unsigned *fwd = lane == 0 ? s.count : none, *rev = none;
+  if (lane >= 1 && lane <= 28) { fwd = s.pair + ta * 72 + tb * 9; rev = s.pair + tb * 72 + ta * 9; }
+  const bool aligned = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  const int first = blockIdx.x * (DESC_WARPS * per_warp) + (threadIdx.x >> 5);
+  for (int li = first; li < min(first + DESC_WARPS * per_warp, n_ligands); li += DESC_WARPS) {
+    const int base = lig[li].atom_base, n = lig[li].n_atoms, nrot = lig[li].n_rot;
+#pragma unroll
+    for (int q = 0; q < 5; ++q)  // pair and count
+      if (lane + 32 * q < (64 * 9 + 8) / 4) reinterpret_cast<uint4 *>(s.pair)[lane + 32 * q] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) {
+      float4 v = __ldg(atoms + base + i);
+      const int type = __float_as_int(v.w);
+      atomicAdd(&s.count[type], 1u);
+      v.w = __int_as_float(type * 9);
+      s.atom[i] = v;
+      if (i < n / 2) s.atom[n + i] = v;
+    }
+    __syncwarp();
+    // an item: atom c with the four atoms r, r + 1, r + 2, r + 3 places on; a
+    // step of 32 items moves c by dc and wraps `dr` times, or once more
+    const int pairs = n * (n - 1) / 2, turn3 = 3 * n;
+    int c = lane, r = 1, q = lane, dc = 32, dr = 0;
+    if (n <= 32 && n > 0) { c = lane % n; r = 1 + 4 * (lane / n); q = (r - 1) * n + c; dc = 32 % n; dr = 32 / n; }
+    while (q < pairs) {
+      const float4 x = s.atom[c];
+      const int row = __float_as_int(x.w) * 8 - __float_as_int(FLOOR_0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 y = s.atom[c + r + u];
+        const float dx = __fsub_rn(x.x, y.x), dy = __fsub_rn(x.y, y.y), dz = __fsub_rn(x.z, y.z);
+        const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+        // bin: the squared edges (1.5 k)^2, k = 1..7, not above d2.  The root
+        // in units of 1.5, a little high, gives that or one more; the square of
+        // the edge (exact) decides.  FLOOR_0 + k is k in the low bits.
+        const float t = fminf(__fmaf_rd(sqrt_approx(d2), 0.666668f, FLOOR_0), FLOOR_0 + 7.f), k = t - FLOOR_0;
+        int at = row + __float_as_int(y.w) + __float_as_int(t);
+        if (d2 < 2.25f * k * k) --at;
+        if (q + u * n < pairs) atomicAdd(&s.pair[at], 1u);
+      }
+      c += dc;
+      r += 4 * dr;
+      q += 32 + turn3 * dr;
+      if (c >= n) { c -= n; r += 4; q += turn3; }
+    }
+    __syncwarp();
+    float o[8];
+    unsigned cnt[8], most = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      cnt[q] = fwd[q] + rev[q] + (q == 0 && lane == 29 ? (unsigned)nrot : 0u);
+      most = max(most, cnt[q]);
+      o[q] = logs[min(cnt[q], (unsigned)DESC_LOGS - 1)];
+    }
+    if (most >= DESC_LOGS)
+#pragma unroll 1
+      for (int q = 0; q < 8; ++q)
+        if (cnt[q] >= DESC_LOGS) o[q] = log1pf((float)cnt[q]);
+    float *const dst = out + (size_t)li * 256 + 8 * lane;
+    if (aligned) {
+      reinterpret_cast<float4 *>(dst)[0] = make_float4(o[0], o[1], o[2], o[3]);
+      reinterpret_cast<float4 *>(dst)[1] = make_float4(o[4], o[5], o[6], o[7]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) dst[q] = o[q];
+    }
+    __syncwarp();  // the next ligand overwrites the counters
   }
 }
 
@@ -90,9 +141,11 @@ extern "C" ligate_status ligate_descriptors(const ligate_batch *b, float *out, v
   if (!b || (!out && b->d.n_ligands)) { set_error("descriptors: NULL argument"); return LIGATE_ERR_INVALID; }
   if (b->d.n_ligands == 0) return LIGATE_OK;
   if (b->max_type >= 8) { set_error("descriptors: need atom types < 8"); return LIGATE_ERR_UNSUPPORTED; }
-  const int wpb = 8;
-  descriptor_kernel<<<(b->d.n_ligands + wpb - 1) / wpb, 32 * wpb, 0, (cudaStream_t)stream>>>(
-      b->d.lig, b->d.atoms, b->d.n_ligands, out);
+  // four ligands per warp (they share the table of logarithms) once that still
+  // gives every SM several blocks
+  const int per_warp = b->d.n_ligands >= 32768 ? 4 : 1, per_block = DESC_WARPS * per_warp;
+  descriptor_kernel<<<(b->d.n_ligands + per_block - 1) / per_block, 32 * DESC_WARPS, 0, (cudaStream_t)stream>>>(
+      b->d.lig, b->d.atoms, b->d.n_ligands, per_warp, out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "descriptor kernel");
   return LIGATE_OK;
