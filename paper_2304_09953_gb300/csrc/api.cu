@@ -1136,15 +1136,16 @@ static void default_tile(ligate_tile *t) {
 // small to give every warp 32 (at least 8), but no fewer than 2 K: an item
 // pays for loading its ligand, and has no K-th best of its own to stop starts
 // with before its K-th start.  A run of fewer than 4 starts per resident warp
-// spreads over all of them: every start is under way before a K-th best could
-// stop one (measured, lo = 128, 64, 32, 16, 8: one 24-atom
+// spreads over all of them, in at most 512 items per ligand (their lists are
+// merged by one warp): every start is under way before a K-th best could stop
+// one (measured, lo = 128, 64, 32, 16, 8: one 24-atom
 // ligand with 512 starts and K = 4 372, 213, 135, 99 and 88 us; 301 ligands
 // with 1,717 starts and K = 5 4.9, 3.44, 3.19, 3.49 and 3.62 ms; 8 P in the
 // model against 12 P and 16 P: 1,000 ligands 24.1, 24.5, 25.1 ms).
 // Buckets without ligands get 512.  Ligands: sel[0..n) or all of B.
-static double least_chunk(double starts, double P_warps, int K) {
-  const double each = starts / std::max(P_warps, 1.0);
-  if (each < 4.0) return each;
+static double least_chunk(double n, int n_starts, double P_warps, int K) {
+  const double each = n * n_starts / std::max(P_warps, 1.0);
+  if (each < 4.0) return std::max(each, n_starts / 512.0);
   return std::max(2.0 * K, std::min(32.0, std::max(8.0, each)));
 }
 
@@ -1164,7 +1165,7 @@ static void model_chunks(const BatchDev &B, const int32_t *sel, int n, int S, in
   for (int b = 0; b < LIGATE_N_BUCKETS; ++b) {
     double chunk = 512.0;
     if (nb[b] > 0) chunk = W / (8.0 * std::max(P_warps, 1.0) * (cb[b] / nb[b]));
-    chunk = std::min(2048.0, std::max(least_chunk((double)n * n_starts, P_warps, K), chunk));
+    chunk = std::min(2048.0, std::max(least_chunk(n, n_starts, P_warps, K), chunk));
     chunks[b] = std::max(G, (int)chunk / G * G);
   }
 }
@@ -1617,7 +1618,7 @@ extern "C" ligate_status ligate_plan_run_subset(ligate_plan *pl, const int32_t *
     for (int b = 0; b < LIGATE_N_BUCKETS; ++b) {
       double chunk = 512.0;
       if (pl->model_cb[b] > 0) chunk = pl->model_W * ((double)m / std::max(n, 1)) / (8.0 * P_warps * pl->model_cb[b]);
-      chunk = std::min(2048.0, std::max(least_chunk((double)m * p.n_starts, P_warps, p.K), chunk));
+      chunk = std::min(2048.0, std::max(least_chunk(m, p.n_starts, P_warps, p.K), chunk));
       ch.c[b] = std::max(p.G, (int)chunk / p.G * p.G);
       cmin = std::min(cmin, ch.c[b]);
     }

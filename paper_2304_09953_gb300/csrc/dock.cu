@@ -22,7 +22,7 @@ int dock_memo1_tables(const LigDesc &d, const BondRec *bonds, int) {
 
 // The clash tables of every row's ligand, once per run: one warp per (row,
 // table) or, when that leaves the chip idle (split), per (row, table, round of G
-// steps: 301 ligands 65 -> MEASURED us).  What a row's work items share is built here once instead of by
+// steps): 301 ligands 68 -> 39 us.  What a row's work items share is built here once instead of by
 // every item's warp, so items can be small (a batch that leaves few starts
 // per warp) without paying for the tables again, and a ligand's tables are
 // built in parallel.  The same device code builds the tables in the docking
@@ -197,10 +197,10 @@ cudaError_t launch_clash_tables(const DockParams &p, const int32_t *row_lig, int
   const size_t smem = (size_t)warps * smem_bytes_per_warp(p.nmax, 0, p.G, 0);
   cudaError_t e = cudaFuncSetAttribute(clash_tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e != cudaSuccess) return e;
-  // rounds of a table side by side while they would not fill the SMs twice
+  // rounds of a table side by side while that makes few warps per SM
   const int rounds = (p.S + p.G - 1) / p.G;
   long long n = (long long)rows * (2 + p.m1max);
-  const int split = n * rounds <= 16384 ? rounds : 1;
+  const int split = n * rounds <= 65536 ? rounds : 1;
   n *= split;
   clash_tables_kernel<<<(unsigned)((n + warps - 1) / warps), 32 * warps, smem, s>>>(p, row_lig, rows, split);
   return cudaGetLastError();

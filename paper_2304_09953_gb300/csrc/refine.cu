@@ -464,7 +464,7 @@ cudaError_t launch_refine(int mode, const DockParams &p, const double origin[3],
   a.grad = grad;
   const int warps = 4;
   const size_t smem = refine_smem_per_warp(p.nmax) * warps;
-  const int hw = (p.nmax + 31) / 32;  // atoms per lane: 1 to 4
+  const int hw = p.nmax > 32 ? (p.nmax + 31) / 32 : 1;  // atoms per lane: 1 to 4
   const void *const fns[3][4] = {
       {(const void *)refine_kernel<0, 1>, (const void *)refine_kernel<0, 2>, (const void *)refine_kernel<0, 3>,
        (const void *)refine_kernel<0, 4>},
