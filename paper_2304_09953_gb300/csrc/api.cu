@@ -346,7 +346,8 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
       mn = std::min(mn, x);
       mx = std::max(mx, x);
     }
-    const double ext = (mx - mn) * (1.0 + 1e-6) + 1e-3;
+    // a receptor thinner than the cutoff has one cell of that width
+    const double ext = std::max((mx - mn) * (1.0 + 1e-6) + 1e-3, 1.001 * cut_g);
     nc[a] = (int)std::max(1.0, std::min(16.0, std::floor(ext / (1.001 * cut_g))));
     lo[a] = mn;
     wd[a] = ext / nc[a];
