@@ -59,6 +59,19 @@ static cudaError_t dmalloc(T **p, size_t n) {
   return cudaMalloc((void **)p, n * sizeof(T));
 }
 
+// Several device arrays in one allocation: an allocation or a copy costs 10 to
+// 50 us of host time however small it is, which for a few hundred ligands was
+// most of setting up a batch or a plan.
+struct Arena {
+  size_t bytes = 0;
+  template <class T>
+  size_t add(size_t n) {  // the offset of n elements
+    const size_t at = bytes;
+    bytes += (n * sizeof(T) + 255) & ~(size_t)255;
+    return at;
+  }
+};
+
 static int pow2ceil(int v) {
   int p = 1;
   while (p < v) p <<= 1;
@@ -103,15 +116,17 @@ static HostPool &host_pool() {
   return *pool;
 }
 
-// fn(i) for every i in [0, n), handed out in blocks of 64 to `threads`
-// threads (the caller's included).
+// fn(i) for every i in [0, n), handed out in blocks to `threads` threads (the
+// caller's included): about four blocks each, of at most 64 (blocks of 64 gave
+// 301 ligands, about 6 us each to pack, to five of the threads).
 static void parallel_for(int n, int threads, const std::function<void(int)> &fn) {
   std::atomic<int> next(0);
+  const int block = std::max(1, std::min(64, n / (4 * std::max(threads, 1))));
   const std::function<void()> body = [&]() {
     for (;;) {
-      const int i0 = next.fetch_add(64);
+      const int i0 = next.fetch_add(block);
       if (i0 >= n) break;
-      for (int i = i0; i < std::min(n, i0 + 64); ++i) fn(i);
+      for (int i = i0; i < std::min(n, i0 + block); ++i) fn(i);
     }
   };
   if (threads <= 1) { body(); return; }
@@ -799,7 +814,7 @@ extern "C" ligate_status ligate_batch_create(const ligate_ligands *L, ligate_bat
   std::vector<ligate_status> st(n, LIGATE_OK);
   std::vector<std::string> errs(n);
   const unsigned nt = std::max(1u, std::min(64u, std::thread::hardware_concurrency()));
-  const int nthreads = n < 256 ? 1 : (int)nt;
+  const int nthreads = n < 64 ? 1 : (int)nt;
   parallel_for(n, nthreads, [&](int i) {
     char buf[256];
     buf[0] = 0;
@@ -859,19 +874,34 @@ extern "C" ligate_status ligate_batch_create(const ligate_ligands *L, ligate_bat
     std::copy(pk.cand.begin(), pk.cand.end(), d.h_cand.begin() + ld.cand_base);
     pk = LigPack();
   });
-  cudaError_t e;
-  if ((e = dmalloc(&d.lig, n)) != cudaSuccess || (e = dmalloc(&d.atoms, na)) != cudaSuccess ||
-      (e = dmalloc(&d.bonds, nb)) != cudaSuccess || (e = dmalloc(&d.elig, ne)) != cudaSuccess ||
-      (e = dmalloc(&d.cand, nc)) != cudaSuccess || (e = dmalloc(&d.order, na)) != cudaSuccess) {
+  Arena ar;
+  const size_t o_lig = ar.add<LigDesc>(n), o_atoms = ar.add<float4>(na), o_bonds = ar.add<BondRec>(nb),
+               o_elig = ar.add<uint32_t>(ne), o_cand = ar.add<uint16_t>(nc), o_order = ar.add<uint8_t>(na);
+  cudaError_t e = dmalloc(&B->arena, ar.bytes);
+  if (e != cudaSuccess) {
     ligate_batch_destroy(B);
     return cuda_fail(e, "batch allocation");
   }
-  if ((n && (e = cudaMemcpy(d.lig, d.h_lig.data(), sizeof(LigDesc) * n, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (na && (e = cudaMemcpy(d.atoms, atoms.data(), sizeof(float4) * na, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (nb && (e = cudaMemcpy(d.bonds, d.h_bonds.data(), sizeof(BondRec) * nb, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (ne && (e = cudaMemcpy(d.elig, d.h_elig.data(), 4 * ne, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (nc && (e = cudaMemcpy(d.cand, d.h_cand.data(), 2 * nc, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (na && (e = cudaMemcpy(d.order, d.h_order.data(), na, cudaMemcpyHostToDevice)) != cudaSuccess)) {
+  d.lig = reinterpret_cast<LigDesc *>(B->arena + o_lig);
+  d.atoms = reinterpret_cast<float4 *>(B->arena + o_atoms);
+  d.bonds = reinterpret_cast<BondRec *>(B->arena + o_bonds);
+  d.elig = reinterpret_cast<uint32_t *>(B->arena + o_elig);
+  d.cand = reinterpret_cast<uint16_t *>(B->arena + o_cand);
+  d.order = B->arena + o_order;
+  const struct { size_t at; const void *src; size_t bytes; } part[6] = {
+      {o_lig, d.h_lig.data(), sizeof(LigDesc) * n}, {o_atoms, atoms.data(), sizeof(float4) * na},
+      {o_bonds, d.h_bonds.data(), sizeof(BondRec) * nb}, {o_elig, d.h_elig.data(), sizeof(uint32_t) * ne},
+      {o_cand, d.h_cand.data(), sizeof(uint16_t) * nc}, {o_order, d.h_order.data(), (size_t)na}};
+  if (ar.bytes <= (4u << 20)) {  // put together here: one copy (larger ones: the copies' own time counts)
+    std::vector<unsigned char> stage(ar.bytes);
+    for (const auto &q : part)
+      if (q.bytes) memcpy(stage.data() + q.at, q.src, q.bytes);
+    if (ar.bytes) e = cudaMemcpy(B->arena, stage.data(), ar.bytes, cudaMemcpyHostToDevice);
+  } else {
+    for (const auto &q : part)
+      if (q.bytes && e == cudaSuccess) e = cudaMemcpy(B->arena + q.at, q.src, q.bytes, cudaMemcpyHostToDevice);
+  }
+  if (e != cudaSuccess) {
     ligate_batch_destroy(B);
     return cuda_fail(e, "batch upload");
   }
@@ -881,6 +911,11 @@ extern "C" ligate_status ligate_batch_create(const ligate_ligands *L, ligate_bat
 
 extern "C" void ligate_batch_destroy(ligate_batch *b) {
   if (!b) return;
+  if (b->arena) {  // holds all of them
+    cudaFree(b->arena);
+    delete b;
+    return;
+  }
   cudaFree(b->d.lig);
   cudaFree(b->d.atoms);
   cudaFree(b->d.bonds);
@@ -1065,13 +1100,15 @@ struct ligate_plan {
   size_t smem = 0;
   int n_ligands = 0;
   float *rot = nullptr, *anc = nullptr, *quat = nullptr;
-  uint16_t *visit = nullptr;  // anchor visiting order (DockParams::visit)
   // scratch of ligate_plan_best_quantile (grown on demand): best scores,
   // sort keys (two arrays) and sorted indices, q_cap entries each
   float *q_scores = nullptr;
   unsigned long long *q_keys = nullptr;
   int32_t *q_idx = nullptr;
   int q_cap = 0;
+  // one allocation: items, lig_items, lig_slot0, row_lig, stats (with the counters),
+  // partial, out, and DockParams' visiting order and clash tables
+  unsigned char *arena = nullptr;
   Item *items = nullptr;
   int *lig_items = nullptr, *lig_slot0 = nullptr, *counters = nullptr;
   PoseOut *partial = nullptr, *out = nullptr;
@@ -1108,15 +1145,12 @@ static void free_plan(ligate_plan *pl) {
   cudaFree(pl->sub_items); cudaFree(pl->sub_partial); cudaFree(pl->sub_count); cudaFree(pl->sub_lig_items);
   cudaFree(pl->sub_slot0); cudaFree(pl->rowmap); cudaFree(pl->sub_row_lig); cudaFree(pl->lig_by_cost);
   cudaFree(pl->lig_bucket);
-  cudaFree(pl->p.memo1); cudaFree(pl->p.tab);
   if (pl->exec) cudaGraphExecDestroy(pl->exec);
   if (pl->graph) cudaGraphDestroy(pl->graph);
   if (pl->cap_stream) cudaStreamDestroy(pl->cap_stream);
-  cudaFree(pl->rot); cudaFree(pl->anc); cudaFree(pl->quat); cudaFree(pl->visit);
+  cudaFree(pl->rot); cudaFree(pl->anc); cudaFree(pl->quat);
   cudaFree(pl->q_scores); cudaFree(pl->q_keys); cudaFree(pl->q_idx);
-  cudaFree(pl->items); cudaFree(pl->lig_items); cudaFree(pl->lig_slot0);
-  cudaFree(pl->partial); cudaFree(pl->out); cudaFree(pl->stats);  // counters: inside stats
-  cudaFree(pl->row_lig);
+  cudaFree(pl->arena);
   delete pl;
 }
 
@@ -1213,28 +1247,12 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
   pl->h = P->d.spacing;
   pl->pocket = P;
   pl->batch = B;
-  {
-    std::vector<int32_t> rl(pl->n_ligands);
-    for (int r = 0; r < pl->n_ligands; ++r) rl[r] = sel ? sel[r] : r;
-    cudaError_t e0;
-    if (!rl.empty() && ((e0 = dmalloc(&pl->row_lig, rl.size())) != cudaSuccess ||
-                        (e0 = cudaMemcpy(pl->row_lig, rl.data(), 4 * rl.size(), cudaMemcpyHostToDevice)) != cudaSuccess)) {
-      free_plan(pl);
-      return cuda_fail(e0, "plan allocation");
-    }
-  }
   st = base_params(P, B, s, mode, pl->p, &pl->rot, &pl->anc, &pl->quat, opt ? opt->rot : nullptr,
                    opt ? opt->anc : nullptr);
   if (st != LIGATE_OK) { free_plan(pl); return st; }
   DockParams &p = pl->p;
-  if (s->n_anchor <= 1024) {  // consecutive starts of a work item at nearby anchors (O(n^2) pairing)
-    const std::vector<uint16_t> order = anchor_visit_order(P->d.h_anchors.data(), s->n_anchor);
-    cudaError_t e = dmalloc(&pl->visit, order.size());
-    if (e == cudaSuccess)
-      e = cudaMemcpy(pl->visit, order.data(), sizeof(uint16_t) * order.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) { free_plan(pl); return cuda_fail(e, "plan allocation"); }
-    p.visit = pl->visit;
-  }
+  std::vector<uint16_t> visit;  // consecutive starts of a work item at nearby anchors (O(n^2) pairing)
+  if (s->n_anchor <= 1024) visit = anchor_visit_order(P->d.h_anchors.data(), s->n_anchor);
   const int sms = device_sms();
   memset(&pl->tile, 0, sizeof(pl->tile));
   if (tile) pl->tile = *tile;
@@ -1294,9 +1312,11 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
 
   // work queue: (ligand, start chunk) items, most expensive first
   const int n = pl->n_ligands;
-  std::vector<Item> items;
+  // (a row's items cost the same but for a shorter last one: sorted as two
+  // groups per row, then written out item by item)
   std::vector<int> lig_items(n), lig_slot0(n);
-  std::vector<double> cost;
+  std::vector<double> cost(2 * (size_t)n);  // per item of a row's whole chunks, of its last one
+  size_t ni = 0;
   double poses = 0, aev = 0, pev = 0;
   for (int r = 0; r < n; ++r) {
     const int i = sel ? sel[r] : r;
@@ -1306,20 +1326,12 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
     pev += q * p.n_starts;
     poses += (double)p.n_starts * (1.0 + (double)B->d.h_lig[i].n_rot * (p.S - 1));
     const int chunk = t.starts_per_item[bucket_of(B->d.h_lig[i])];
-    lig_slot0[r] = (int)items.size();
-    int c = 0;
-    for (int s0 = 0; s0 < p.n_starts; s0 += chunk, ++c) {
-      Item it;
-      memset(&it, 0, sizeof(it));
-      it.ligand = i;
-      it.row = r;
-      it.s0 = s0;
-      it.s1 = std::min(p.n_starts, s0 + chunk);
-      it.slot = (int)items.size();
-      items.push_back(it);
-      cost.push_back((a + 0.35 * q + 40.0) * (it.s1 - it.s0));
-    }
-    lig_items[r] = c;
+    const int whole = p.n_starts / chunk, rest = p.n_starts - whole * chunk;
+    lig_slot0[r] = (int)ni;
+    lig_items[r] = whole + (rest > 0);
+    ni += lig_items[r];
+    cost[2 * (size_t)r] = (a + 0.35 * q + 40.0) * chunk;
+    cost[2 * (size_t)r + 1] = (a + 0.35 * q + 40.0) * rest;
   }
   pl->work.poses = poses;
   pl->work.atom_evals = aev;
@@ -1329,9 +1341,9 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
   // sort of the complemented bit patterns (non-negative floats order like
   // their bit patterns), 8 bits per pass, passes whose byte is the same for
   // every item skipped
-  std::vector<uint32_t> key(items.size()), key2(items.size());
-  std::vector<uint32_t> order(items.size()), order2(items.size());
-  for (size_t i = 0; i < items.size(); ++i) {
+  std::vector<uint32_t> key(cost.size()), key2(cost.size());
+  std::vector<uint32_t> order(cost.size()), order2(cost.size());
+  for (size_t i = 0; i < cost.size(); ++i) {
     const float c = (float)cost[i];
     uint32_t bits;
     memcpy(&bits, &c, 4);
@@ -1351,42 +1363,70 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
     key.swap(key2);
     order.swap(order2);
   }
-  std::vector<Item> sorted(items.size());
-  for (size_t i = 0; i < order.size(); ++i) sorted[i] = items[order[i]];
-  const size_t ni = items.size();
-  cudaError_t e;
+  // clash tables: every row's, built once per run, while they stay within
+  // TAB_BUDGET; beyond it those of the pairs a single earlier bond separates,
+  // per resident warp
+  int m1 = 0;
+  for (int r = 0; r < n; ++r) {
+    const LigDesc &ld = B->d.h_lig[sel ? sel[r] : r];
+    m1 = std::max(m1, dock_memo1_tables(ld, B->d.h_bonds.data() + ld.bond_base, p.S));
+  }
+  p.m1max = m1;
+  const size_t stride = dock_tab_stride(p.S, p.rmax, m1);
+  const bool tab = n > 0 && p.rmax > 0 && stride * sizeof(float) * n <= TAB_BUDGET;
   // stats (64-bit), queue, done[n], lig_thr[n]: one array, reset at once
   pl->counter_bytes = sizeof(unsigned long long) * N_STATS + sizeof(int) * (2 * (size_t)n + 1);
-  if ((e = dmalloc(&pl->items, ni)) != cudaSuccess || (e = dmalloc(&pl->lig_items, n)) != cudaSuccess ||
-      (e = dmalloc(&pl->lig_slot0, n)) != cudaSuccess ||
-      (e = dmalloc(&pl->stats, pl->counter_bytes / sizeof(unsigned long long) + 1)) != cudaSuccess ||
-      (e = dmalloc(&pl->partial, ni * p.K)) != cudaSuccess ||
-      (e = dmalloc(&pl->out, (size_t)n * p.K)) != cudaSuccess) {
+  Arena ar;  // first what is uploaded
+  const size_t o_items = ar.add<Item>(ni), o_lig_items = ar.add<int>(n), o_lig_slot0 = ar.add<int>(n),
+               o_row_lig = ar.add<int32_t>(n), o_visit = ar.add<uint16_t>(visit.size()), uploaded = ar.bytes,
+               o_stats = ar.add<char>(pl->counter_bytes), o_partial = ar.add<PoseOut>(ni * p.K),
+               o_out = ar.add<PoseOut>((size_t)n * p.K),
+               o_tab = ar.add<float>(tab ? stride * n : (size_t)pl->grid * t.warps_per_cta * m1 * p.S * p.S);
+  cudaError_t e = dmalloc(&pl->arena, ar.bytes);
+  if (e != cudaSuccess) {
     free_plan(pl);
     return cuda_fail(e, "plan allocation");
   }
-  if ((ni && (e = cudaMemcpy(pl->items, sorted.data(), sizeof(Item) * ni, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (n && (e = cudaMemcpy(pl->lig_items, lig_items.data(), 4 * (size_t)n, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (n && (e = cudaMemcpy(pl->lig_slot0, lig_slot0.data(), 4 * (size_t)n, cudaMemcpyHostToDevice)) != cudaSuccess)) {
+  pl->items = reinterpret_cast<Item *>(pl->arena + o_items);
+  pl->lig_items = reinterpret_cast<int *>(pl->arena + o_lig_items);
+  pl->lig_slot0 = reinterpret_cast<int *>(pl->arena + o_lig_slot0);
+  pl->row_lig = reinterpret_cast<int32_t *>(pl->arena + o_row_lig);
+  pl->stats = reinterpret_cast<unsigned long long *>(pl->arena + o_stats);
+  pl->partial = reinterpret_cast<PoseOut *>(pl->arena + o_partial);
+  pl->out = reinterpret_cast<PoseOut *>(pl->arena + o_out);
+  if (!visit.empty()) p.visit = reinterpret_cast<const uint16_t *>(pl->arena + o_visit);
+  if (tab) {
+    p.tab = reinterpret_cast<float *>(pl->arena + o_tab);
+    p.tab_stride = (int)stride;
+  } else if (m1 > 0) {
+    p.memo1 = reinterpret_cast<float *>(pl->arena + o_tab);
+  }
+  std::vector<unsigned char> stage(uploaded);
+  Item *next = reinterpret_cast<Item *>(stage.data() + o_items);
+  for (const uint32_t q : order) {
+    const int r = (int)(q / 2), i = sel ? sel[r] : r, chunk = t.starts_per_item[bucket_of(B->d.h_lig[i])],
+              whole = p.n_starts / chunk;
+    for (int c = q & 1 ? whole : 0; c < (q & 1 ? lig_items[r] : whole); ++c) {
+      Item it;
+      memset(&it, 0, sizeof(it));
+      it.ligand = i;
+      it.row = r;
+      it.s0 = c * chunk;
+      it.s1 = c < whole ? it.s0 + chunk : p.n_starts;
+      it.slot = lig_slot0[r] + c;
+      *next++ = it;
+    }
+  }
+  int32_t *const row_lig = reinterpret_cast<int32_t *>(stage.data() + o_row_lig);
+  for (int r = 0; r < n; ++r) row_lig[r] = sel ? sel[r] : r;
+  if (n) {
+    memcpy(stage.data() + o_lig_items, lig_items.data(), sizeof(int) * (size_t)n);
+    memcpy(stage.data() + o_lig_slot0, lig_slot0.data(), sizeof(int) * (size_t)n);
+  }
+  if (!visit.empty()) memcpy(stage.data() + o_visit, visit.data(), sizeof(uint16_t) * visit.size());
+  if (uploaded && (e = cudaMemcpy(pl->arena, stage.data(), uploaded, cudaMemcpyHostToDevice)) != cudaSuccess) {
     free_plan(pl);
     return cuda_fail(e, "plan upload");
-  }
-  {  // clash tables: every row's, built once per run, while they stay within TAB_BUDGET;
-     // beyond it those of the pairs a single earlier bond separates, per resident warp
-    int m1 = 0;
-    for (int r = 0; r < n; ++r) {
-      const LigDesc &ld = B->d.h_lig[sel ? sel[r] : r];
-      m1 = std::max(m1, dock_memo1_tables(ld, B->d.h_bonds.data() + ld.bond_base, p.S));
-    }
-    p.m1max = m1;
-    const size_t stride = dock_tab_stride(p.S, p.rmax, m1);
-    if (n > 0 && p.rmax > 0 && stride * sizeof(float) * n <= TAB_BUDGET) {
-      if ((e = dmalloc(&p.tab, stride * n)) != cudaSuccess) { free_plan(pl); return cuda_fail(e, "plan allocation"); }
-      p.tab_stride = (int)stride;
-    } else if (m1 > 0) {
-      const size_t floats = (size_t)pl->grid * t.warps_per_cta * m1 * p.S * p.S;
-      if ((e = dmalloc(&p.memo1, floats)) != cudaSuccess) { free_plan(pl); return cuda_fail(e, "plan allocation"); }
-    }
   }
   pl->counters = reinterpret_cast<int *>(pl->stats + N_STATS);
   p.items = pl->items;

@@ -351,5 +351,6 @@ struct ligate_pocket {
 struct ligate_batch {
   ligate::BatchDev d;
   int max_type = 0;
+  unsigned char *arena = nullptr;  // one allocation with d's device arrays (else they are their own)
 };
 
