@@ -834,7 +834,7 @@ def main():
                   "poses_per_s": ws * work_plain.poses / (plain_ms / 1000),
                   "poses_evaluated_per_s": ws * (work_plain.starts + work_plain.done_bond_sweeps * (S - 1))
                   / (plain_ms / 1000), "ms_per_step": plain_ms,
-                  "form": "fp32 plain maps, default tile, no rescore",
+                  "form": "fp32 maps, default tile, no rescore",
                   "roofline_frac": plain_alg / (plain_ms / 1000) / 1e12 / peak,
                   "roofline_frac_executed": plain_flops / (plain_ms / 1000) / 1e12 / peak,
                   "gather": {"achieved": plain_gather_gbs, "peak": gather_peak_f32, "unit": "GB/s",

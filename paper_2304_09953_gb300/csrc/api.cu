@@ -2073,7 +2073,7 @@ extern "C" ligate_status ligate_plan_refine(const ligate_plan *pl, int iteration
 }
 
 // ===========================================================================
-// Exact rescoring (dock.cu).
+// Exact rescoring (rescore.cu).
 static ligate_status rec_params(const ligate_pocket *P, const ligate_batch *B, RecParams &r, const char *what) {
   if (!P->d.rec_pair) { set_error("%s: the pocket has no receptor (ligate_pocket_set_receptor)", what); return LIGATE_ERR_INVALID; }
   if (B->max_type >= P->d.rec_types) {
