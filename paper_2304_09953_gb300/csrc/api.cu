@@ -317,6 +317,75 @@ extern "C" void ligate_pocket_destroy(ligate_pocket *p) {
   delete p;
 }
 
+// The fine cells' lists (d.rec_fine, d.rec_list) of the receptor in d.rec and
+// d.rec_cell: fine cells of about 2 A (wider while the lists would exceed 16 Mi
+// entries) inside each coarse cell, one coarse cell beyond the grid included,
+// over the map box and three quarters of the cutoff around it (lists for every
+// cell of the neighbourhood gained nothing).  A fine cell's list holds the
+// receptor atoms of its coarse cell's 3 x 3 x 3 neighbourhood that can be within
+// the cutoff of a point in it, with a margin for FP32 rounding of the cell index
+// and the distance, in the column (lane, accumulator) that the kernel's
+// row-by-row sum over the neighbourhood gives them: position o of a row of three
+// cells is lane o % 32, accumulator o / 32 % 2.  Built on the device, counted,
+// then filled: the host's threads took 11 ms for 3,000 receptor atoms and 27 for
+// 8,000 in the large box.
+static cudaError_t build_fine_lists(PocketDev &d, int n, const int (&nc)[3], const double (&lo)[3],
+                                    const double (&wd)[3], double h, double cut_g, int (&fs)[3], int (&f0)[3],
+                                    int (&nf)[3]) {
+  const int dim[3] = {d.nx, d.ny, d.nz};
+  cudaError_t e;
+  std::vector<int> steps, fstart(1, 0);
+  int *counts = nullptr;
+  FineGrid g;
+  for (int a = 0; a < 3; ++a) { fs[a] = 1; f0[a] = nf[a] = 0; }
+  for (double width = 2.0; n > 0 && n < 0xffff; width *= 2.0) {
+    bool finest = true;
+    for (int a = 0; a < 3; ++a) {
+      fs[a] = (int)std::max(1.0, std::min(16.0, std::ceil(wd[a] * h / width)));
+      finest &= fs[a] == 1;
+      const double wf = wd[a] / fs[a];
+      const double rim = 0.75 * cut_g;  // poses reach out of the box by a few A
+      f0[a] = (int)std::max(-(double)fs[a], std::floor((-rim - lo[a]) / wf));
+      const int f1 = (int)std::min((double)(nc[a] + 1) * fs[a] - 1,
+                                   std::max(-1e6, std::floor((dim[a] - 1 + rim - lo[a]) / wf)));
+      nf[a] = std::max(0, f1 - f0[a] + 1);
+      g.nc[a] = nc[a]; g.fs[a] = fs[a]; g.f0[a] = f0[a]; g.nf[a] = nf[a];
+      g.lo[a] = lo[a]; g.wf[a] = wf;
+    }
+    const double reach = cut_g * (1.0 + 1e-5) + 0.02 + 1e-5 * std::max(dim[0], std::max(dim[1], dim[2]));
+    g.reach2 = reach * reach;
+    const long long nfc = (long long)nf[0] * nf[1] * nf[2];
+    long long total = 0;
+    if (nfc > 0 && nfc <= (1 << 18)) {
+      steps.resize((size_t)nfc);
+      if ((e = dmalloc(&counts, (size_t)nfc)) != cudaSuccess ||
+          (e = launch_fine_lists(g, d.rec, d.rec_cell, nullptr, counts, nullptr)) != cudaSuccess ||
+          (e = cudaMemcpy(steps.data(), counts, 4 * (size_t)nfc, cudaMemcpyDeviceToHost)) != cudaSuccess) {
+        cudaFree(counts);
+        return e;
+      }
+      cudaFree(counts);
+      for (const int k : steps) total += 64LL * k;
+    }
+    if (nfc > (1 << 18) || total > (16 << 20)) {
+      if (finest) { nf[0] = 0; break; }
+      continue;
+    }
+    fstart.assign((size_t)nfc + 1, 0);
+    for (size_t c = 0; c < (size_t)nfc; ++c) fstart[c + 1] = fstart[c] + steps[c];
+    break;
+  }
+  if ((e = dmalloc(&d.rec_fine, fstart.size())) != cudaSuccess ||
+      (e = cudaMemcpy(d.rec_fine, fstart.data(), 4 * fstart.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
+      (e = dmalloc(&d.rec_list, 64 * (size_t)fstart.back())) != cudaSuccess)
+    return e;
+  if (fstart.back() > 0 &&
+      ((e = launch_fine_lists(g, d.rec, d.rec_cell, d.rec_fine, nullptr, d.rec_list)) != cudaSuccess ||
+       (e = cudaStreamSynchronize(0)) != cudaSuccess))  // read by kernels on any stream
+    return e;
+  return cudaSuccess;
+}
+
 extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const float *xyz, const int32_t *type,
                                                     int n, const float *radius, const float *eps,
                                                     int n_types, float cutoff, float cap, float rmin) {
@@ -385,88 +454,6 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
     for (int j = 0; j < n; ++j) sorted[fill[cell_of[j]]++] = rec[j];  // stable: input order within a cell
     rec.swap(sorted);
   }
-  // fine cells of about 2 A (wider while the lists would exceed 16 Mi entries)
-  // inside each coarse cell, one coarse cell beyond the grid included, over the
-  // map box and three quarters of the cutoff around it (lists for every cell
-  // of the neighbourhood cost 17 ms more per receptor and gained nothing).  A
-  // fine cell's list holds the receptor atoms of its coarse cell's
-  // 3 x 3 x 3 neighbourhood that can be within the cutoff of a point in it,
-  // with a margin for FP32 rounding of the cell index and the distance, in the
-  // column (lane, accumulator) that the kernel's row-by-row sum over the
-  // neighbourhood gives them: position o of a row of three cells is lane o % 32,
-  // accumulator o / 32 % 2
-  const int dim[3] = {P->d.nx, P->d.ny, P->d.nz};
-  int fs[3] = {1, 1, 1}, f0[3] = {0, 0, 0}, nf[3] = {0, 0, 0};
-  std::vector<int> fstart(1, 0);
-  std::vector<uint16_t> flist;
-  for (double width = 2.0; n > 0 && n < 0xffff; width *= 2.0) {
-    bool finest = true;
-    for (int a = 0; a < 3; ++a) {
-      fs[a] = (int)std::max(1.0, std::min(16.0, std::ceil(wd[a] * h / width)));
-      finest &= fs[a] == 1;
-      const double wf = wd[a] / fs[a];
-      const double rim = 0.75 * cut_g;  // poses reach out of the box by a few A
-      f0[a] = (int)std::max(-(double)fs[a], std::floor((-rim - lo[a]) / wf));
-      const int f1 = (int)std::min((double)(nc[a] + 1) * fs[a] - 1,
-                                   std::max(-1e6, std::floor((dim[a] - 1 + rim - lo[a]) / wf)));
-      nf[a] = std::max(0, f1 - f0[a] + 1);
-    }
-    const long long nfc = (long long)nf[0] * nf[1] * nf[2];
-    if (nfc > (1 << 18)) {
-      if (finest) { nf[0] = 0; break; }
-      continue;
-    }
-    std::vector<std::vector<uint16_t>> lists((size_t)nfc);
-    std::atomic<long long> total(0);
-    const double reach = cut_g * (1.0 + 1e-5) + 0.02 + 1e-5 * std::max(dim[0], std::max(dim[1], dim[2]));
-    const long long most = (long long)16 << 20;
-    parallel_for((int)nfc, nfc < 256 ? 1 : (int)std::max(1u, std::min(64u, std::thread::hardware_concurrency())),
-                 [&](int c) {
-      if (total.load(std::memory_order_relaxed) > most) return;
-      const int fc[3] = {c % nf[0], c / nf[0] % nf[1], c / nf[0] / nf[1]};
-      int cc[3], k0[3], k1[3];
-      double b0[3], b1[3];
-      for (int a = 0; a < 3; ++a) {
-        const int f = f0[a] + fc[a] + fs[a];  // from the coarse cell before the grid
-        cc[a] = f / fs[a] - 1;
-        b0[a] = lo[a] + (f0[a] + fc[a]) * (wd[a] / fs[a]);
-        b1[a] = b0[a] + wd[a] / fs[a];
-        k0[a] = std::max(cc[a] - 1, 0);
-        k1[a] = std::min(cc[a] + 1, nc[a] - 1);
-      }
-      if (k0[0] > k1[0] || k0[1] > k1[1] || k0[2] > k1[2]) return;
-      std::vector<uint16_t> col[64];
-      size_t steps = 0;
-      for (int z = k0[2]; z <= k1[2]; ++z)
-        for (int y = k0[1]; y <= k1[1]; ++y) {
-          const int row = (z * nc[1] + y) * nc[0], s0 = start[row + k0[0]];
-          for (int j = s0; j < start[row + k1[0] + 1]; ++j) {
-            const double dx = std::max(0.0, std::max(b0[0] - rec[j].x, rec[j].x - b1[0])),
-                         dy = std::max(0.0, std::max(b0[1] - rec[j].y, rec[j].y - b1[1])),
-                         dz = std::max(0.0, std::max(b0[2] - rec[j].z, rec[j].z - b1[2]));
-            if (dx * dx + dy * dy + dz * dz > reach * reach) continue;
-            std::vector<uint16_t> &v = col[(j - s0) % 64];
-            v.push_back((uint16_t)j);
-            steps = std::max(steps, v.size());
-          }
-        }
-      std::vector<uint16_t> &L = lists[c];
-      L.assign(steps * 64, 0xffff);
-      for (int q = 0; q < 64; ++q)
-        for (size_t k = 0; k < col[q].size(); ++k) L[k * 64 + q] = col[q][k];
-      total += (long long)L.size();
-    });
-    if (total.load() > most) {
-      if (finest) { nf[0] = 0; break; }
-      continue;
-    }
-    fstart.assign((size_t)nfc + 1, 0);
-    for (size_t c = 0; c < lists.size(); ++c) fstart[c + 1] = fstart[c] + (int)(lists[c].size() / 64);
-    flist.resize((size_t)fstart.back() * 64);
-    for (size_t c = 0; c < lists.size(); ++c)
-      std::copy(lists[c].begin(), lists[c].end(), flist.begin() + (size_t)fstart[c] * 64);
-    break;
-  }
   std::vector<float2> pair((size_t)n_types * n_types);
   for (int t = 0; t < n_types; ++t)
     for (int u = 0; u < n_types; ++u) {
@@ -484,6 +471,7 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
   P->d.rec_pair = nullptr;
   P->d.rec_cell = nullptr;
   P->d.n_rec = 0;
+  int fs[3], f0[3], nf[3];
   cudaError_t e;
   if ((n && ((e = dmalloc(&P->d.rec, (size_t)n)) != cudaSuccess ||
              (e = cudaMemcpy(P->d.rec, rec.data(), 16 * (size_t)n, cudaMemcpyHostToDevice)) != cudaSuccess)) ||
@@ -491,11 +479,7 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
       (e = cudaMemcpy(P->d.rec_pair, pair.data(), 8 * pair.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = dmalloc(&P->d.rec_cell, start.size())) != cudaSuccess ||
       (e = cudaMemcpy(P->d.rec_cell, start.data(), 4 * start.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = dmalloc(&P->d.rec_fine, fstart.size())) != cudaSuccess ||
-      (e = cudaMemcpy(P->d.rec_fine, fstart.data(), 4 * fstart.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = dmalloc(&P->d.rec_list, flist.size())) != cudaSuccess ||
-      (!flist.empty() &&
-       (e = cudaMemcpy(P->d.rec_list, flist.data(), 2 * flist.size(), cudaMemcpyHostToDevice)) != cudaSuccess)) {
+      (e = build_fine_lists(P->d, n, nc, lo, wd, h, cut_g, fs, f0, nf)) != cudaSuccess) {
     cudaFree(P->d.rec); cudaFree(P->d.rec_pair); cudaFree(P->d.rec_cell);
     cudaFree(P->d.rec_fine); cudaFree(P->d.rec_list);
     P->d.rec_fine = nullptr; P->d.rec_list = nullptr;

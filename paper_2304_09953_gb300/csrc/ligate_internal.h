@@ -254,7 +254,19 @@ inline void fill_step_table(int S, float *tab) {
   }
 }
 
-// Exact rescoring (dock.cu): explicit poses (lig_idx, start_id, tors) or,
+// Fine cells of a receptor's cell grid (grid units): per axis the coarse cells,
+// fine cells per coarse one, first fine cell and their number, the receptor's
+// low corner and a fine cell's width.
+struct FineGrid {
+  int nc[3], fs[3], f0[3], nf[3];
+  double lo[3], wf[3], reach2;
+};
+// steps != NULL: each fine cell's list steps (64 entries each); else the lists,
+// cell c's from step first[c] to first[c + 1] (default stream).
+cudaError_t launch_fine_lists(const FineGrid &g, const float4 *rec, const int *cell, const int *first, int *steps,
+                              uint16_t *list);
+
+// Exact rescoring (rescore.cu): explicit poses (lig_idx, start_id, tors) or,
 // with poses != NULL, a plan's output [n_poses / K][K] with row_lig.
 size_t rescore_smem_bytes(const DockParams &p, const RecParams &r, int warps);
 cudaError_t launch_rescore(const DockParams &p, const RecParams &r, int n_poses, const int32_t *lig_idx,
@@ -262,7 +274,7 @@ cudaError_t launch_rescore(const DockParams &p, const RecParams &r, int n_poses,
                            const int32_t *row_lig, const StateSrc *states, ligate_rescored *out,
                            cudaStream_t s);
 
-// Per-pose selector features (dock.cu), [n_poses][256] FP32; explicit
+// Per-pose selector features (rescore.cu), [n_poses][256] FP32; explicit
 // poses or a plan's output as for launch_rescore.
 cudaError_t launch_pose_features(const DockParams &p, int n_poses, const int32_t *lig_idx,
                                  const int32_t *start_id, const uint8_t *tors, const ligate_pose *poses,

@@ -83,6 +83,55 @@ __device__ __noinline__ float receptor_cells(const RecParams &r, const float2 *p
   return warp_sum(acc[0] + acc[1]);
 }
 
+// The fine cells' lists, a warp per cell: lane l has the columns l and l + 32
+// (positions l, l + 32, l + 64, ... of a row of cells, in turn).  Steps of the
+// longest column, or the entries themselves, 0xffff where a column has ended.
+__global__ void __launch_bounds__(256) fine_lists_kernel(const FineGrid g, const float4 *__restrict__ rec,
+                                                        const int *__restrict__ cell, const int *__restrict__ first,
+                                                        int *__restrict__ steps, uint16_t *__restrict__ list) {
+  const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (c >= g.nf[0] * g.nf[1] * g.nf[2]) return;
+  const int fc[3] = {c % g.nf[0], c / g.nf[0] % g.nf[1], c / g.nf[0] / g.nf[1]};
+  int k0[3], k1[3];
+  double b0[3], b1[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int cc = (g.f0[a] + fc[a] + g.fs[a]) / g.fs[a] - 1;  // from the coarse cell before the grid
+    b0[a] = g.lo[a] + (g.f0[a] + fc[a]) * g.wf[a];
+    b1[a] = b0[a] + g.wf[a];
+    k0[a] = max(cc - 1, 0);
+    k1[a] = min(cc + 1, g.nc[a] - 1);
+  }
+  const int total = steps ? 0 : first[c + 1] - first[c];
+  uint16_t *const out = steps ? nullptr : list + 64 * (size_t)first[c];
+  int n[2] = {0, 0};
+  if (k0[0] <= k1[0])
+    for (int z = k0[2]; z <= k1[2]; ++z)
+      for (int y = k0[1]; y <= k1[1]; ++y) {
+        const int row = (z * g.nc[1] + y) * g.nc[0], j1 = cell[row + k1[0] + 1];
+        for (int j0 = cell[row + k0[0]] + lane; j0 < j1; j0 += 64)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int j = j0 + 32 * q;
+            if (j >= j1) continue;
+            const float4 v = rec[j];
+            const double dx = fmax(0.0, fmax(b0[0] - v.x, v.x - b1[0])), dy = fmax(0.0, fmax(b0[1] - v.y, v.y - b1[1])),
+                         dz = fmax(0.0, fmax(b0[2] - v.z, v.z - b1[2]));
+            if (dx * dx + dy * dy + dz * dz > g.reach2) continue;
+            if (out && n[q] < total) out[64 * n[q] + lane + 32 * q] = (uint16_t)j;
+            ++n[q];
+          }
+      }
+  if (steps) {
+    const int most = (int)__reduce_max_sync(FULL, (unsigned)max(n[0], n[1]));
+    if (lane == 0) steps[c] = most;
+  } else {
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      for (int k = n[q]; k < total; ++k) out[64 * k + lane + 32 * q] = 0xffff;
+  }
+}
+
 constexpr int POSE_RUN = 4;  // consecutive poses a warp takes at a time
 
 __global__ void __launch_bounds__(256) rescore_kernel(const __grid_constant__ DockParams p,
@@ -538,6 +587,14 @@ cudaError_t launch_selector_labels(const ligate_rescored *rec, long long n, floa
                                    cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   selector_labels_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(rec, n, fail_label, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fine_lists(const FineGrid &g, const float4 *rec, const int *cell, const int *first, int *steps,
+                              uint16_t *list) {
+  const int cells = g.nf[0] * g.nf[1] * g.nf[2];
+  if (cells <= 0) return cudaSuccess;
+  fine_lists_kernel<<<(cells + 7) / 8, 256>>>(g, rec, cell, first, steps, list);
   return cudaGetLastError();
 }
 
