@@ -523,6 +523,7 @@ __global__ void __launch_bounds__(1024) sort_tile_kernel(const float *__restrict
   const int len = min(SORT_TILE, n - base);
   int size = 2;
   while (size < len) size <<= 1;
+  pdl_wait();
   for (int q = threadIdx.x; q < size; q += blockDim.x) {
     unsigned long long key = ~0ull;
     if (q < len) {
@@ -580,6 +581,7 @@ __global__ void __launch_bounds__(1024) sort_tile_kernel(const float *__restrict
 __global__ void __launch_bounds__(256) merge_kernel(const unsigned long long *__restrict__ in, int n, int R, int k,
                                                     unsigned long long *__restrict__ out,
                                                     int32_t *__restrict__ idx) {
+  pdl_wait();
   const int per = min(R, k);
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int run = (int)(t / per), p = (int)(t % per);
@@ -631,21 +633,23 @@ __global__ void __launch_bounds__(256) merge_kernel(const unsigned long long *__
 cudaError_t sort_select(const float *pred, int n, int k, unsigned long long *keys, int32_t *idx, cudaStream_t s) {
   if (n <= 0 || k <= 0) return cudaSuccess;
   const int tiles = (n + SORT_TILE - 1) / SORT_TILE;
-  sort_tile_kernel<<<tiles, 1024, 0, s>>>(pred, n, k, keys, tiles == 1 ? idx : nullptr);
+  cudaError_t e = launch_pdl(sort_tile_kernel, dim3(tiles), dim3(1024), 0, s, pred, n, k, keys, tiles == 1 ? idx : nullptr);
   unsigned long long *in = keys, *out = keys + n;
   long long runs = tiles;
-  for (long long R = SORT_TILE; runs > 1; R *= MERGE_WAYS) {
+  for (long long R = SORT_TILE; runs > 1 && e == cudaSuccess; R *= MERGE_WAYS) {
     const long long threads = runs * std::min<long long>(R, k);
     runs = (runs + MERGE_WAYS - 1) / MERGE_WAYS;
-    merge_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(in, n, (int)R, k, out, runs == 1 ? idx : nullptr);
+    e = launch_pdl(merge_kernel, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, s, in, n, (int)R, k, out,
+                   runs == 1 ? idx : nullptr);
     std::swap(in, out);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 // Mean prediction of an ensemble, accumulated in network order.
 __global__ void mean_pred_kernel(const float *__restrict__ pred, int n_nets, int n, float a, float *__restrict__ mean) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
   if (i >= n) return;
   float v = a * pred[i];
   for (int m = 1; m < n_nets; ++m) v = fmaf(a, pred[(size_t)m * n + i], v);
@@ -653,8 +657,7 @@ __global__ void mean_pred_kernel(const float *__restrict__ pred, int n_nets, int
 }
 cudaError_t mean_pred(const float *pred, int n_nets, int n, float *mean, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  mean_pred_kernel<<<(n + 255) / 256, 256, 0, s>>>(pred, n_nets, n, 1.f / (float)n_nets, mean);
-  return cudaGetLastError();
+  return launch_pdl(mean_pred_kernel, dim3((n + 255) / 256), dim3(256), 0, s, pred, n_nets, n, 1.f / (float)n_nets, mean);
 }
 
 // Launch helpers used by the surrogate object.

@@ -8,11 +8,11 @@
 namespace ligate {
 namespace mlp {
 
-// The kernels of a training step follow one another on one stream, each a few
-// microseconds long, so a launch's own latency counts: they are launched with
-// programmatic stream serialisation.  A kernel's CTAs may start while the one
-// before it drains, and pdl_wait (before the first access to memory that
-// another kernel writes or reads) holds them until it has finished.
+// The kernels of a training step, and those of a ranking, follow one another on
+// one stream, each a few microseconds long, so a launch's own latency counts:
+// they are launched with programmatic stream serialisation.  A kernel's CTAs may
+// start while the one before it drains, and pdl_wait (before the first access to
+// memory that another kernel writes or reads) holds them until it has finished.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
