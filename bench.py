@@ -868,7 +868,7 @@ def main():
         "triage": triage, "refine": refine, "rescore": rescore, "pose_selector": selector,
         "model_tile": model,
         "cpu_baseline": cpu, "e2e": e2e, "clocks": clock_info,
-        "gpu_launches": launches_per_run * args.steps,
+        "gpu_launches": launches_per_run * args.steps,  # docking kernel; each run builds its clash tables before it
     }
     if rank == 0:
         print(json.dumps(line), flush=True)
