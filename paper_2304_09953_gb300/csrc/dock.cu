@@ -193,8 +193,11 @@ cudaError_t launch_dock(int mode, int reg_cap, const DockParams &p, int grid, in
 
 cudaError_t launch_clash_tables(const DockParams &p, const int32_t *row_lig, int rows, cudaStream_t s) {
   if (rows <= 0 || !p.tab || p.rmax == 0) return cudaSuccess;
-  const int warps = 4;
-  const size_t smem = (size_t)warps * smem_bytes_per_warp(p.nmax, 0, p.G, 0);
+  // four warps per CTA, fewer where their slots exceed a CTA's shared memory
+  // (G = 32 start groups, S = 1, with more than 64 atoms: 79 or 104 KB a warp)
+  const size_t per_warp = smem_bytes_per_warp(p.nmax, 0, p.G, 0);
+  const int warps = (int)std::min<size_t>(4, (size_t)(227 * 1024) / per_warp);
+  const size_t smem = (size_t)warps * per_warp;
   cudaError_t e = cudaFuncSetAttribute(clash_tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e != cudaSuccess) return e;
   // rounds of a table side by side while that makes few warps per SM

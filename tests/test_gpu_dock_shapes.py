@@ -8,7 +8,7 @@ import pytest
 
 from paper_2304_09953_gb300 import docking as D
 from paper_2304_09953_gb300 import native as N
-from paper_2304_09953_gb300.workload import Sampling
+from paper_2304_09953_gb300.workload import Sampling, make_ligands
 from tests.parity import Stats, compare_ligand
 
 pytestmark = pytest.mark.gpu
@@ -48,4 +48,29 @@ def test_shapes_agree_and_match_the_oracle(batched_small, S, K, orient, anchor):
     for r in range(0, len(idx), 4):
         if K <= samp.n_starts:
             compare_ligand(ligs.ligand(r), w.pocket, samp, ref[r], K=K, stats=st)
+    print(st.line())
+
+
+@pytest.mark.parametrize("n_atoms", [64, 65, 96, 128])
+@pytest.mark.parametrize("S", [1, 2])
+def test_large_ligands_at_few_torsion_steps(batched_small, S, n_atoms):
+    """The most start groups per warp with the largest ligands, whose slots
+    limit the warps of a CTA: a full run, a selection and the one-call docking
+    give the oracle's poses."""
+    torch = pytest.importorskip("torch")
+    w = batched_small
+    ligs = make_ligands(17, np.array([n_atoms, 24, n_atoms], np.int32), np.array([8, 3, 16], np.int32),
+                        w.pocket.n_types)
+    samp = Sampling(w.sampling.quats[:8], 8, S, 4)
+    ph, bh = D.PocketHandle(w.pocket), D.BatchHandle(ligs)
+    pl = D.Plan(ph, bh, samp, mode="fp32")
+    res = pl.result()
+    sel = torch.tensor([2, 0], dtype=torch.int32, device="cuda")
+    assert np.array_equal(pl.run_subset(sel, result=True), res[[2, 0]])
+    out = np.zeros((ligs.n, 4), N.POSE_DTYPE)
+    N.ligate_dock_batch(ph.h, ligs, N.make_sampling(samp, *D.MODES["fp32"], False), out)
+    assert np.array_equal(out, res)
+    st = Stats()
+    for r in range(ligs.n):
+        compare_ligand(ligs.ligand(r), w.pocket, samp, res[r], K=4, stats=st)
     print(st.line())
