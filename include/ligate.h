@@ -667,8 +667,11 @@ int ligate_surrogate_engine(const ligate_surrogate *s);
  * of a tcgen05 contraction on the current device issues none of its tensor
  * loads, so its bounded wait on the first stage runs out (after 2 s); the
  * kernel records the timeout, releases its tensor memory and returns, and
- * the surrogate call that launched it returns LIGATE_ERR_TIMEOUT.  Nothing
- * hangs and the context stays usable.  Other kinds: INVALID. */
+ * the surrogate call that launched it returns LIGATE_ERR_TIMEOUT.  kind 2:
+ * one warp of the next CTA of the inference kernel (predict, rank) takes its
+ * last layer's wait as run out while the warps beside it go on; the CTA leaves
+ * its remaining rows with the same status.  Nothing hangs and the context
+ * stays usable.  Other kinds: INVALID. */
 ligate_status ligate_debug_inject_fault(int kind);
 
 #if defined(__GNUC__)

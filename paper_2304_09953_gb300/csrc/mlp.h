@@ -103,9 +103,11 @@ struct FwdSpec {
 cudaError_t forward_tc05(const FwdSpec *nets, int n_nets, const float *desc, int n, cudaStream_t s);
 // mean[i] = sum_m (1 / n_nets) pred[m][i], accumulated in network order.
 cudaError_t mean_pred(const float *pred, int n_nets, int n, float *mean, cudaStream_t s);
-// Test hook: the next CTA of a tcgen05 contraction issues no loads, so its
-// bounded wait runs out (err set, LIGATE_ERR_TIMEOUT at the next check).
-cudaError_t inject_skip_loads_once();
+// Test hook (err set, LIGATE_ERR_TIMEOUT at the next check): kind 1, the next
+// CTA of a tcgen05 contraction issues no loads, so its bounded wait runs out;
+// kind 2, one warp of the next forward_tc05 CTA takes its last layer's wait as
+// run out while the warps beside it go on.
+cudaError_t inject_fault_once(int kind);
 // wt[n][k] = bf16(w[k][n]) for row-major FP32 w [K][N].
 cudaError_t transpose_bf16(const float *w, int K, int N, __nv_bfloat16 *wt, cudaStream_t s);
 

@@ -111,9 +111,9 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
                : "memory");
 }
 
-// Fault flag for tests of the timeout path (ligate_debug_inject_fault):
-// nothing in normal operation sets it.
-__device__ int g_fault_skip_loads = 0;
+// Fault for tests of the timeout path (ligate_debug_inject_fault's kind; the
+// CTA that takes it resets it): nothing in normal operation sets it.
+__device__ int g_fault = 0;
 
 template <int TN, int STAGES>
 struct __align__(1024) Smem {
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(128, 1)
     int issued = 0;  // K slices whose loads were issued
     // test hook: a CTA that takes the fault flag issues no loads, so its
     // bounded wait on the first stage runs out and the error path runs
-    const bool skip_loads = atomicExch(&g_fault_skip_loads, 0) != 0;
+    const bool skip_loads = atomicCAS(&g_fault, 1, 0) == 1;
     for (int kb = 0; kb < nk && kb < STAGES && !skip_loads; ++kb, ++issued) {
       mbar_expect_tx(&s.full[kb], A_BYTES + B_BYTES);
       tma_load_2d(s.a[kb], &tm_a, &s.full[kb], kb * TK, m0);
@@ -299,6 +299,7 @@ struct __align__(1024) FwdSmem {
   __nv_bfloat16 w4[512];
   uint64_t full[FW_STAGES], empty[FW_STAGES], in[2], acc[2], drain;
   uint32_t tmem_base;
+  volatile int fault;  // test hook: warp 1 takes its last wait as run out
 };
 static_assert(sizeof(FwdSmem) + 1024 <= 227 * 1024, "one CTA's shared memory");
 
@@ -323,6 +324,17 @@ __device__ __forceinline__ void warp_arrive(uint64_t *bar, int lane) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncwarp();
   if (lane == 0) mbar_arrive(bar);
+}
+// Whether all 128 threads of warps 0-3 are `ok`; a barrier among them.
+__device__ __forceinline__ bool all_of_half(bool ok) {
+  unsigned r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, 1, 128, p;\n"
+      " selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"(ok ? 1u : 0u)
+      : "memory");
+  return r != 0;
 }
 // mbar_wait by a whole warp, the same answer in every lane.
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, unsigned parity) {
@@ -421,6 +433,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid
     mbar_init(&s.acc[0], 1);
     mbar_init(&s.acc[1], 1);
     mbar_init(&s.drain, 1);
+    s.fault = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 8) {  // the whole tensor memory: 512 columns
@@ -438,7 +451,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     if (warp == 9) {  // the weight stream of all items, one thread
-      if (lane == 0 && atomicExch(&g_fault_skip_loads, 0) == 0) {  // test hook (see gemm_tc05_kernel)
+      const int fault = lane == 0 ? atomicExch(&g_fault, 0) : 1;  // test hook (see gemm_tc05_kernel)
+      if (fault == 2) s.fault = 1;
+      if (fault != 1) {
         int loaded = 0;
         bool go = true;
         for (int item = first_item; item < a.items && go; item += step) {
@@ -513,6 +528,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid
       const FwdNet &net = a.net[item / a.tiles];
       const int row0 = item % a.tiles * TM, next = item + step;
       if (half == 0) {
+        // Warps 0-3 wait for the tensor core each by itself, and one's wait may run
+        // out just before another's succeeds: each meets the others at the tile's
+        // last barrier (all_of_half) all the same, and they leave together.
         for (int q = tid; q < 512; q += 128) s.w4[q] = net.w4[q];
         asm volatile("bar.sync 1, 128;" ::: "memory");
 #pragma unroll 1
@@ -524,7 +542,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid
           fw_store_half(s, 0, row, x);
           warp_arrive(&s.in[0], lane);
         }
-        if (!ok || !(ok = warp_wait(&s.acc[0], layer & 1u))) break;
+        if (!ok || !(ok = warp_wait(&s.acc[0], layer & 1u) && !(warp == 1 && s.fault))) {
+          all_of_half(false);
+          break;
+        }
         // head: chain c of 32 sums the columns c, c + 32, ..., then the
         // butterfly's tree
         float acc[32];
@@ -555,7 +576,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid
             }
           }
         }
-        if (!ok) break;
+        if (!ok) {
+          all_of_half(false);
+          break;
+        }
         ++layer;
         warp_arrive(&s.in[1], lane);
 #pragma unroll
@@ -563,7 +587,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) mlp_forward_kernel(const __grid
 #pragma unroll
           for (int c = 0; c < o; ++c) acc[c] += acc[c + o];
         if (row0 + row < a.n) net.pred[row0 + row] = fmaf(acc[0] + __ldg(net.b4), net.ly_sd, net.ly_mu);
-        asm volatile("bar.sync 1, 128;" ::: "memory");  // w4 is read
+        ok = all_of_half(true);  // w4 is read
       } else {
         const int nrow0 = next % a.tiles * TM;
         if (next < a.items)  // the next tile's rows towards L2
@@ -711,10 +735,7 @@ cudaError_t forward_tc05(const FwdSpec *nets, int n_nets, const float *desc, int
   return cudaSuccess;
 }
 
-cudaError_t inject_skip_loads_once() {
-  const int one = 1;
-  return cudaMemcpyToSymbol(g_fault_skip_loads, &one, sizeof(int));
-}
+cudaError_t inject_fault_once(int kind) { return cudaMemcpyToSymbol(g_fault, &kind, sizeof(int)); }
 
 // Wt[n][k] = bf16(W[k][n]) for a row-major [K][N] FP32 weight matrix.
 __global__ void transpose_bf16_kernel(const float *__restrict__ w, int K, int N,

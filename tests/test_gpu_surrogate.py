@@ -313,6 +313,28 @@ def test_tcgen05_wait_timeout_is_reported_and_recoverable(monkeypatch):
         N.ligate_debug_inject_fault(7)
 
 
+@pytest.mark.parametrize("n", [1000, 40000])
+def test_one_warp_alone_runs_out_of_time(n):
+    """One warp of an inference CTA gives up its wait while the warps beside
+    it see the same wait succeed: all leave together (one row tile, or with
+    tiles left), the call reports the timeout, and the next one is right."""
+    desc = torch.from_numpy(np.random.default_rng(12).normal(size=(n, 256)).astype(np.float32)).cuda()
+    s = N.ligate_surrogate_create(None, 12)
+    try:
+        if N.ligate_surrogate_engine(s) != 1:
+            pytest.skip("tcgen05 engine")
+        ref, bad, again = (torch.zeros(n, dtype=torch.float32, device="cuda") for _ in range(3))
+        N.ligate_surrogate_predict(s, desc, n, ref)
+        N.ligate_debug_inject_fault(2)
+        with pytest.raises(N.LigateError) as ei:
+            N.ligate_surrogate_predict(s, desc, n, bad)
+        assert ei.value.status == N.LIGATE_ERR_TIMEOUT
+        N.ligate_surrogate_predict(s, desc, n, again)
+        assert torch.equal(again, ref)
+    finally:
+        N.ligate_surrogate_destroy(s)
+
+
 def test_checkpoint_resumes_training_exactly(tmp_path):
     """Save after one epoch, load into a new object, train both one more
     epoch with the same seed: identical weights (Adam moments, step and
