@@ -228,6 +228,10 @@ typedef struct {
  * kernel, per-ligand merge and optional FP32 rescoring) into one CUDA graph
  * on first run.  tile == NULL picks the autotuner's cached shape for this
  * device (LIGATE_TUNE_CACHE file, see ligate_autotune) or the default.
+ * Device memory: beside the items and lists the clash tables of its ligands
+ * (about 12 KB each at S = 16 and 12 rotatable bonds), or, beyond 1 GiB of them
+ * or when there is no room for them, tables per resident warp (about 30 MB;
+ * the same results, slower).
  * The plan borrows pocket and batch: keep both alive until it is
  * destroyed.  Errors: INVALID, UNSUPPORTED (S, K or layout outside the
  * limits, BF16/FP16 without the matching pocket copy), OOM, CUDA. */

@@ -1357,16 +1357,21 @@ static ligate_status plan_create_impl(const ligate_pocket *P, const ligate_batch
   }
   p.m1max = m1;
   const size_t stride = dock_tab_stride(p.S, p.rmax, m1);
-  const bool tab = n > 0 && p.rmax > 0 && stride * sizeof(float) * n <= TAB_BUDGET;
+  bool tab = n > 0 && p.rmax > 0 && stride * sizeof(float) * n <= TAB_BUDGET;
   // stats (64-bit), queue, done[n], lig_thr[n]: one array, reset at once
   pl->counter_bytes = sizeof(unsigned long long) * N_STATS + sizeof(int) * (2 * (size_t)n + 1);
   Arena ar;  // first what is uploaded
   const size_t o_items = ar.add<Item>(ni), o_lig_items = ar.add<int>(n), o_lig_slot0 = ar.add<int>(n),
                o_row_lig = ar.add<int32_t>(n), o_visit = ar.add<uint16_t>(visit.size()), uploaded = ar.bytes,
                o_stats = ar.add<char>(pl->counter_bytes), o_partial = ar.add<PoseOut>(ni * p.K),
-               o_out = ar.add<PoseOut>((size_t)n * p.K),
-               o_tab = ar.add<float>(tab ? stride * n : (size_t)pl->grid * t.warps_per_cta * m1 * p.S * p.S);
-  cudaError_t e = dmalloc(&pl->arena, ar.bytes);
+               o_out = ar.add<PoseOut>((size_t)n * p.K), o_tab = ar.bytes;
+  auto tables = [&]() { return sizeof(float) * (tab ? stride * n : (size_t)pl->grid * t.warps_per_cta * m1 * p.S * p.S); };
+  cudaError_t e = dmalloc(&pl->arena, o_tab + tables());
+  if (e == cudaErrorMemoryAllocation && tab) {  // no room for the rows' tables: per warp, as beyond TAB_BUDGET
+    cudaGetLastError();  // not for the next check to find
+    tab = false;
+    e = dmalloc(&pl->arena, o_tab + tables());
+  }
   if (e != cudaSuccess) {
     free_plan(pl);
     return cuda_fail(e, "plan allocation");

@@ -3,12 +3,15 @@
 a plain-layout plan (which searches the pocket's FP32 corner copy) against
 one whose pocket has no copy, at torsion steps around the group sizes and
 list lengths from one to the limit; and the result is the oracle's."""
+import contextlib
+
 import numpy as np
 import pytest
 
 from paper_2304_09953_gb300 import docking as D
 from paper_2304_09953_gb300 import native as N
 from paper_2304_09953_gb300.workload import Sampling, make_ligands
+from tests.device_memory import all_but
 from tests.parity import Stats, compare_ligand
 
 pytestmark = pytest.mark.gpu
@@ -74,3 +77,25 @@ def test_large_ligands_at_few_torsion_steps(batched_small, S, n_atoms):
     for r in range(ligs.n):
         compare_ligand(ligs.ligand(r), w.pocket, samp, res[r], K=4, stats=st)
     print(st.line())
+
+
+def test_clash_tables_give_way_to_memory(batched_small):
+    """A plan whose ligands' clash tables (96 MB here) find no room takes
+    tables per warp (32 MB) and gives the same bits."""
+    torch = pytest.importorskip("torch")
+    w = batched_small
+    ligs = w.ligands.subset([i % w.ligands.n for i in range(8000)])
+    samp = Sampling(w.sampling.quats[:16], 8, 16, 1)
+    ph, bh = D.PocketHandle(w.pocket), D.BatchHandle(ligs)
+    D.Plan(ph, bh, samp, mode="bf16").result()  # what the first run loads
+    torch.cuda.empty_cache()
+    res, used = [], []
+    for short in (False, True):
+        with all_but(64 << 20) if short else contextlib.nullcontext():
+            before = torch.cuda.mem_get_info()[0]
+            pl = D.Plan(ph, bh, samp, mode="bf16")
+            used.append(before - torch.cuda.mem_get_info()[0])
+            res.append(pl.result())
+            pl.close()
+    assert used[0] > 64 << 20 > used[1]
+    assert np.array_equal(res[0], res[1])
