@@ -283,7 +283,8 @@ ligate_status ligate_plan_best_scores(const ligate_plan *plan, float *out, int s
  *
  * ligate_plan_best_quantile: the k-th smallest of the last run's best
  * scores, k = ceil(frac * rows) (1 <= k <= rows), into DEVICE out[0]
- * (enqueues; the first call for a plan of a new size allocates scratch).
+ * (enqueues; a plan's first call allocates scratch, for runs of any
+ * selection of its ligands).
  * Run on a plan whose starts are a subset of another plan's (the same
  * pocket, precision, torsion steps and ligands; the first orientations and
  * anchors of the same lists), it gives a value at or above the k-th best

@@ -1084,7 +1084,7 @@ struct ligate_plan {
   size_t smem = 0;
   int n_ligands = 0;
   float *rot = nullptr, *anc = nullptr, *quat = nullptr;
-  // scratch of ligate_plan_best_quantile (grown on demand): best scores,
+  // scratch of ligate_plan_best_quantile (made on first use): best scores,
   // sort keys (two arrays) and sorted indices, q_cap entries each
   float *q_scores = nullptr;
   unsigned long long *q_keys = nullptr;
@@ -1953,13 +1953,14 @@ extern "C" ligate_status ligate_plan_best_quantile(ligate_plan *pl, double frac,
   if (n == 0) { set_error("plan_best_quantile: the plan has no rows"); return LIGATE_ERR_INVALID; }
   const int k = std::min(n, std::max(1, (int)std::ceil(frac * n - 1e-9)));
   cudaError_t e = cudaSuccess;
-  if (pl->q_cap < n) {  // grown once per size (allocates: not inside a capture)
+  if (pl->q_cap < n) {  // once, for a run of all the plan's ligands (allocates: not inside a capture)
+    const int cap = std::max(n, pl->n_ligands);
     cudaFree(pl->q_scores); cudaFree(pl->q_keys); cudaFree(pl->q_idx);
     pl->q_scores = nullptr; pl->q_keys = nullptr; pl->q_idx = nullptr; pl->q_cap = 0;
-    if ((e = dmalloc(&pl->q_scores, n)) != cudaSuccess || (e = dmalloc(&pl->q_keys, 2 * (size_t)n)) != cudaSuccess ||
-        (e = dmalloc(&pl->q_idx, n)) != cudaSuccess)
+    if ((e = dmalloc(&pl->q_scores, cap)) != cudaSuccess || (e = dmalloc(&pl->q_keys, 2 * (size_t)cap)) != cudaSuccess ||
+        (e = dmalloc(&pl->q_idx, cap)) != cudaSuccess)
       return cuda_fail(e, "plan_best_quantile");
-    pl->q_cap = n;
+    pl->q_cap = cap;
   }
   cudaStream_t st = (cudaStream_t)stream;
   best_scores_kernel<<<(n + 255) / 256, 256, 0, st>>>(pl->out, n, pl->p.K, pl->q_scores, 1, 0);

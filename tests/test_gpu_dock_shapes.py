@@ -99,3 +99,22 @@ def test_clash_tables_give_way_to_memory(batched_small):
             pl.close()
     assert used[0] > 64 << 20 > used[1]
     assert np.array_equal(res[0], res[1])
+
+
+def test_quantile_captured_after_a_smaller_selection(batched_small):
+    """The quantile's scratch, made at its first call on a selection, serves a
+    full run: nothing is allocated inside a stream capture."""
+    torch = pytest.importorskip("torch")
+    w = batched_small
+    ph, bh = D.PocketHandle(w.pocket), D.BatchHandle(w.ligands)
+    pl = D.Plan(ph, bh, Sampling(w.sampling.quats[:8], 8, 8, 1), mode="fp32")
+    cut = torch.zeros(1, dtype=torch.float32, device="cuda")
+    pl.run_subset(torch.arange(3, dtype=torch.int32, device="cuda"))
+    pl.best_quantile(1.0, cut)
+    best = np.sort(pl.result()[:, 0]["score"])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pl.best_quantile(0.5, cut, torch.cuda.current_stream().cuda_stream)
+    graph.replay()
+    assert cut.item() == best[w.ligands.n // 2 - 1]
