@@ -324,7 +324,8 @@ extern "C" void ligate_pocket_destroy(ligate_pocket *p) {
 // cell of the neighbourhood gained nothing).  A fine cell's list holds the
 // receptor atoms of its coarse cell's 3 x 3 x 3 neighbourhood that can be within
 // the cutoff of a point in it, with a margin for FP32 rounding of the cell index
-// and the distance, in the column (lane, accumulator) that the kernel's
+// (2.4e-7 of the cell grid's extent per axis at most: the subtraction, the inverse
+// width, the products) and of the distance, in the column (lane, accumulator) that the kernel's
 // row-by-row sum over the neighbourhood gives them: position o of a row of three
 // cells is lane o % 32, accumulator o / 32 % 2.  Built on the device, counted,
 // then filled: the host's threads took 11 ms for 3,000 receptor atoms and 27 for
@@ -345,14 +346,15 @@ static cudaError_t build_fine_lists(PocketDev &d, int n, const int (&nc)[3], con
       finest &= fs[a] == 1;
       const double wf = wd[a] / fs[a];
       const double rim = 0.75 * cut_g;  // poses reach out of the box by a few A
-      f0[a] = (int)std::max(-(double)fs[a], std::floor((-rim - lo[a]) / wf));
+      f0[a] = (int)std::min((double)(nc[a] + 1) * fs[a], std::max(-(double)fs[a], std::floor((-rim - lo[a]) / wf)));
       const int f1 = (int)std::min((double)(nc[a] + 1) * fs[a] - 1,
                                    std::max(-1e6, std::floor((dim[a] - 1 + rim - lo[a]) / wf)));
       nf[a] = std::max(0, f1 - f0[a] + 1);
       g.nc[a] = nc[a]; g.fs[a] = fs[a]; g.f0[a] = f0[a]; g.nf[a] = nf[a];
       g.lo[a] = lo[a]; g.wf[a] = wf;
     }
-    const double reach = cut_g * (1.0 + 1e-5) + 0.02 + 1e-5 * std::max(dim[0], std::max(dim[1], dim[2]));
+    double reach = cut_g * (1.0 + 1e-5) + 0.02 + 1e-5 * std::max(dim[0], std::max(dim[1], dim[2]));
+    for (int a = 0; a < 3; ++a) reach += 1e-6 * (nc[a] + 1) * wd[a];
     g.reach2 = reach * reach;
     const long long nfc = (long long)nf[0] * nf[1] * nf[2];
     long long total = 0;

@@ -126,3 +126,46 @@ def test_docking_many_starts_or_rows(batched_small, n_lig, orient, anchor, S, K)
     assert np.array_equal(D.Plan(ph, bh, samp, mode="fp32").result(), ref)
     bh.close()
     ph.close()
+
+
+@pytest.mark.parametrize("length", [1e3, 3e5, 1e6, 3e6])
+def test_rescoring_beside_a_receptor_atom_far_away(tiny, length):
+    """A receptor atom far from the box makes the cells wide, and a point's
+    cell index rounds by up to 1e-7 of the receptor's length: a one-atom
+    ligand stepped across the cell boundary beside the receptor's near end
+    still sees every receptor atom within the cutoff (FP64 sum)."""
+    P0, h, cut = tiny.pocket, tiny.pocket.spacing, 8.0
+    near = 0.75 * (P0.dims[0] - 1) * h  # the near end
+    worst = 0.0
+    for k in range(8):
+        far = np.float32(-length * (1 + 0.003 * k))
+        lo, mx = np.float32(float(far) / h), np.float32(near / h)
+        end = (float(lo) + (float(mx) - float(lo)) * (1 + 1e-6) + 1e-3) * h  # the last cell's boundary
+        # a ladder of receptor atoms about the cutoff before the boundary, 0.6 mA apart
+        x = np.float32(end - cut - 0.06 + 6e-4 * np.arange(200))
+        y = np.full(201, 4.0, np.float32)
+        xyz = np.stack([np.append(x, np.float32(near)), y, y], 1)
+        xyz = np.vstack([xyz, [[far, 4.0, 4.0]]]).astype(np.float32)
+        xyz[-2, 1] = 100.0  # the near end's own atom sits beyond the cutoff
+        T = P0.maps.shape[0]
+        rad, eps = np.full(T, 1.8), np.full(T, 0.2)
+        P = Pocket(P0.maps, np.zeros(3), h, P0.anchors, xyz, np.zeros(len(xyz), np.int32), rad, eps)
+        lig = make_ligands(1, np.array([1], np.int32), np.array([0], np.int32), T)
+        px = np.float32(end - 0.06 + 6e-4 * np.arange(200) + 3e-4)
+        st = np.zeros(len(px), N.STATE_DTYPE)
+        st["rot"][:] = np.eye(3, dtype=np.float32).reshape(-1)
+        st["trans"][:] = np.stack([px, np.full_like(px, 4.0), np.full_like(px, 4.0)], 1)
+        ph, bh = D.PocketHandle(P), D.BatchHandle(lig)
+        out = torch.zeros(len(px) * N.RESCORED_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+        N.ligate_rescore_states(ph.h, bh.h, N.make_sampling(tiny.sampling), len(px),
+                                torch.zeros(len(px), dtype=torch.int32, device="cuda"), to_dev(st), out)
+        got = out.cpu().numpy().view(N.RESCORED_DTYPE)["e_inter"].astype(np.float64)
+        bh.close()
+        ph.close()
+        d = np.abs(px.astype(np.float64)[:, None] - x.astype(np.float64))
+        q = (3.6 / d) ** 6
+        want = np.where(d <= cut, 0.2 * (q * q - 2 * q), 0.0).sum(1)
+        worst = max(worst, np.abs(got - want).max())
+    # one atom at the cutoff counts 0.0033: positions are half a step off the ladder,
+    # so FP32 rounding moves none across it
+    assert worst < 5e-4, worst
