@@ -474,6 +474,16 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
   P->d.rec_cell = nullptr;
   P->d.n_rec = 0;
   int fs[3], f0[3], nf[3];
+  auto lists = [&]() {
+    const cudaError_t e = build_fine_lists(P->d, n, nc, lo, wd, h, cut_g, fs, f0, nf);
+    if (e != cudaErrorMemoryAllocation) return e;
+    // no room for the lists (up to 34 MB): rescoring sums over the coarse cells
+    cudaGetLastError();  // not for the next check to find
+    cudaFree(P->d.rec_fine); cudaFree(P->d.rec_list);
+    P->d.rec_fine = nullptr; P->d.rec_list = nullptr;
+    nf[0] = nf[1] = nf[2] = 0;
+    return cudaSuccess;
+  };
   cudaError_t e;
   if ((n && ((e = dmalloc(&P->d.rec, (size_t)n)) != cudaSuccess ||
              (e = cudaMemcpy(P->d.rec, rec.data(), 16 * (size_t)n, cudaMemcpyHostToDevice)) != cudaSuccess)) ||
@@ -481,7 +491,7 @@ extern "C" ligate_status ligate_pocket_set_receptor(ligate_pocket *P, const floa
       (e = cudaMemcpy(P->d.rec_pair, pair.data(), 8 * pair.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = dmalloc(&P->d.rec_cell, start.size())) != cudaSuccess ||
       (e = cudaMemcpy(P->d.rec_cell, start.data(), 4 * start.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = build_fine_lists(P->d, n, nc, lo, wd, h, cut_g, fs, f0, nf)) != cudaSuccess) {
+      (e = lists()) != cudaSuccess) {
     cudaFree(P->d.rec); cudaFree(P->d.rec_pair); cudaFree(P->d.rec_cell);
     cudaFree(P->d.rec_fine); cudaFree(P->d.rec_list);
     P->d.rec_fine = nullptr; P->d.rec_list = nullptr;

@@ -3,6 +3,8 @@ sizes where their kernels change shape: atoms around multiples of 32 and pair
 distances on the bins' edges, 1 to 4 atoms per lane, receptors from one atom
 to several list steps that reach beyond the box, and rows at a 4-byte
 alignment."""
+import contextlib
+
 import numpy as np
 import pytest
 
@@ -10,6 +12,7 @@ import oracle
 from paper_2304_09953_gb300 import docking as D
 from paper_2304_09953_gb300 import native as N
 from paper_2304_09953_gb300.workload import Pocket, Sampling, make_ligands
+from tests.device_memory import all_but
 from tests.parity import Geometry, Stats, rescore_check
 from tests.test_gpu_refine import seeded_states, to_dev
 from tests.test_gpu_rescore import explicit
@@ -169,3 +172,43 @@ def test_rescoring_beside_a_receptor_atom_far_away(tiny, length):
     # one atom at the cutoff counts 0.0033: positions are half a step off the ladder,
     # so FP32 rounding moves none across it
     assert worst < 5e-4, worst
+
+
+def test_listed_and_coarse_cells_give_the_same_bits(batched_small):
+    """A receptor set while there is no room for its fine cells' lists is
+    summed over the coarse cells: poses inside the lists, across their rim and
+    outside them (atoms of both kinds side by side) get the same bits."""
+    w, P0 = batched_small, batched_small.pocket
+    rng = np.random.default_rng(8)
+    lo, hi = np.asarray(P0.origin), np.asarray(P0.origin) + (np.array(P0.dims) - 1) * P0.spacing
+    n_types = P0.maps.shape[0]
+    bare = Pocket(P0.maps, P0.origin, P0.spacing, P0.anchors)
+    rec = (rng.uniform(lo - 14.0, hi + 14.0, size=(11000, 3)).astype(np.float32),
+           rng.integers(0, n_types, size=11000).astype(np.int32), np.linspace(1.5, 2.0, n_types),
+           np.linspace(0.1, 0.3, n_types), 8.0, 10.0, 0.5)
+
+    class W:
+        pocket, ligands, sampling = P0, w.ligands, w.sampling
+
+    lig, st, _ = seeded_states(W, np.arange(w.ligands.n), rng, 40, spread=10.0)
+    st["trans"][::50] += np.float32(300.0)
+    bh, s = D.BatchHandle(w.ligands), N.make_sampling(w.sampling)
+    dev = torch.from_numpy(lig).cuda(), to_dev(st)
+    outs, used = [], []
+    N.ligate_pocket_set_receptor(D.PocketHandle(bare, mask=0).h, *rec)  # what the first call loads
+    for short in (False, True):
+        ph = D.PocketHandle(bare, mask=0)
+        torch.cuda.empty_cache()
+        with all_but(4 << 20) if short else contextlib.nullcontext():
+            before = torch.cuda.mem_get_info()[0]
+            N.ligate_pocket_set_receptor(ph.h, *rec)
+            used.append(before - torch.cuda.mem_get_info()[0])
+        out = torch.zeros(len(lig) * N.RESCORED_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+        N.ligate_rescore_states(ph.h, bh.h, s, len(lig), *dev, out)
+        outs.append(out.cpu().numpy().view(N.RESCORED_DTYPE))
+        ph.close()
+    bh.close()
+    assert used[0] > 6 << 20 > used[1], used
+    assert np.array_equal(outs[0], outs[1])
+    e = outs[0]["e_inter"]
+    assert (e == 0).any() and (np.abs(e) > 1).sum() > len(e) // 2
