@@ -95,6 +95,9 @@ __device__ __noinline__ float receptor_cells(const RecParams &r, const float2 *p
 // The fine cells' lists, a warp per cell: lane l has the columns l and l + 32
 // (positions l, l + 32, l + 64, ... of a row of cells, in turn).  Steps of the
 // longest column, or the entries themselves, 0xffff where a column has ended.
+// Bound by issue on the distance tests, in FP32 (the reach's margin covers their
+// rounding): in FP64, which this device runs at a sixty-fourth of the rate, the
+// two passes over 3,000 receptor atoms and 12,167 cells took 360 us each.
 __global__ void __launch_bounds__(256) fine_lists_kernel(const FineGrid g, const float4 *__restrict__ rec,
                                                         const int *__restrict__ cell, const int *__restrict__ first,
                                                         int *__restrict__ steps, uint16_t *__restrict__ list) {
@@ -102,17 +105,18 @@ __global__ void __launch_bounds__(256) fine_lists_kernel(const FineGrid g, const
   if (c >= g.nf[0] * g.nf[1] * g.nf[2]) return;
   const int fc[3] = {c % g.nf[0], c / g.nf[0] % g.nf[1], c / g.nf[0] / g.nf[1]};
   int k0[3], k1[3];
-  double b0[3], b1[3];
+  float b0[3], b1[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const int cc = (g.f0[a] + fc[a] + g.fs[a]) / g.fs[a] - 1;  // from the coarse cell before the grid
-    b0[a] = g.lo[a] + (g.f0[a] + fc[a]) * g.wf[a];
-    b1[a] = b0[a] + g.wf[a];
+    b0[a] = (float)(g.lo[a] + (g.f0[a] + fc[a]) * g.wf[a]);
+    b1[a] = (float)(g.lo[a] + (g.f0[a] + fc[a] + 1) * g.wf[a]);
     k0[a] = max(cc - 1, 0);
     k1[a] = min(cc + 1, g.nc[a] - 1);
   }
   const int total = steps ? 0 : first[c + 1] - first[c];
   uint16_t *const out = steps ? nullptr : list + 64 * (size_t)first[c];
+  const float reach2 = (float)g.reach2;
   int n[2] = {0, 0};
   if (k0[0] <= k1[0])
     for (int z = k0[2]; z <= k1[2]; ++z)
@@ -124,9 +128,9 @@ __global__ void __launch_bounds__(256) fine_lists_kernel(const FineGrid g, const
             const int j = j0 + 32 * q;
             if (j >= j1) continue;
             const float4 v = rec[j];
-            const double dx = fmax(0.0, fmax(b0[0] - v.x, v.x - b1[0])), dy = fmax(0.0, fmax(b0[1] - v.y, v.y - b1[1])),
-                         dz = fmax(0.0, fmax(b0[2] - v.z, v.z - b1[2]));
-            if (dx * dx + dy * dy + dz * dz > g.reach2) continue;
+            const float dx = fmaxf(0.f, fmaxf(b0[0] - v.x, v.x - b1[0])), dy = fmaxf(0.f, fmaxf(b0[1] - v.y, v.y - b1[1])),
+                        dz = fmaxf(0.f, fmaxf(b0[2] - v.z, v.z - b1[2]));
+            if (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > reach2) continue;
             if (out && n[q] < total) out[64 * n[q] + lane + 32 * q] = (uint16_t)j;
             ++n[q];
           }
