@@ -217,8 +217,9 @@ typedef struct {
   int ctas_per_sm;
   int starts_per_item[LIGATE_N_BUCKETS];
   int reg_cap;         /* registers per thread: 1: at most 85 (6 CTAs of 128 threads per SM), 2: at most
-                          102 (5 CTAs), 3: at most 128 (4 CTAs), 0: default (128 for the plain FP32
-                          layout, 102 for the corner layouts) */
+                          102 (5 CTAs), 3: at most 128 (4 CTAs), 0: default (102 for the corner
+                          layouts, 128 for the plain one and where shared memory
+                          keeps no more CTAs resident at 102) */
 } ligate_tile;
 
 /* ------------------------------------------------------------------------
@@ -496,8 +497,8 @@ typedef struct {
 } ligate_rescored;
 /* Explicit poses (DEVICE lig_idx, start_id, tors[n][LIGATE_MAX_ROT]; out
  * DEVICE [n]).  Errors: INVALID without a receptor or with ligand types
- * beyond it; UNSUPPORTED when the receptor (16 B per atom) does not fit in
- * shared memory (about 12,000 atoms).  Synchronises stream. */
+ * beyond it; UNSUPPORTED for receptors above about 12,000 atoms (16 B per
+ * atom, with the pair and cell tables, within 227 KB).  Synchronises stream. */
 ligate_status ligate_rescore_poses(const ligate_pocket *pocket, const ligate_batch *batch,
                                    const ligate_sampling *sampling, int n, const int32_t *lig_idx,
                                    const int32_t *start_id, const uint8_t *tors, ligate_rescored *out,
@@ -578,13 +579,15 @@ ligate_status ligate_autotune(const ligate_pocket *pocket, const ligate_batch *b
  * chosen without timing anything.  Shape: the CTA size and register cap
  * that keep the most warps resident on one SM under the register file and
  * shared-memory limits, among the kernel instances that do not spill
- * registers to local memory (for the plain FP32 layout only the
- * 128-register instances: its eight scalar gathers per interpolation need
+ * registers to local memory (with the present kernel the 128-register
+ * instances; for the plain FP32 layout, read when the pocket has no FP32
+ * corner copy, always those: its eight scalar gathers per interpolation need
  * registers for loads in flight).  Chunk of size bucket b (the work model, also used by
  * every plan for zero chunk fields): starts_per_item[b] = W / (8 P c_b)
  * clamped to [lo, 2048] and rounded down to the start group, with lo = 32 (8
  * to 32 for a run with fewer than 32 starts per resident warp; at least 2
- * top_k), W the
+ * top_k; for a run with fewer than 4 starts per resident warp those, or a
+ * 512th of a ligand's starts if that is more, down to one start group), W the
  * run's total work (sum over ligands of starts x per-start cost atoms +
  * 0.35 clash pairs + 40), P the resident warps of the whole GPU and c_b the
  * bucket's mean per-start cost: the largest item stays under an eighth of a

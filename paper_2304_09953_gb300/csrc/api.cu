@@ -1014,7 +1014,10 @@ ligate_status check_sampling(const ligate_pocket *P, const ligate_batch *B, cons
 // pocket's FP32 corner copy when it has one.  The corners hold the plain map's
 // values, so the results are the same bits, and one 32-byte gather takes the
 // place of eight scalar ones: 1,000 batched ligands (64^3 maps) 50.7 -> 27.1
-// ms, 1,000 of the large target's (96^3, a 220 MB copy) 69.1 -> 38.8 ms.
+// ms, 1,000 of the large target's (96^3, a 220 MB copy) 69.1 -> 38.8 ms.  On
+// larger maps too, where the plain ones still fit L2 and the copy does not: 500
+// ligands with 8,192 starts, 128^3 (537 MB) 38.2 -> 24.1 ms, 160^3 (1 GB) 40.2
+// -> 27.5, 200^3 (2 GB) 40.6 -> 30.4.
 int search_mode(const PocketDev &d, int mode) {
   return mode == MODE_F32_PLAIN && d.map_f32c ? (int)MODE_F32_CORNER : mode;
 }
@@ -1167,12 +1170,16 @@ static void default_tile(ligate_tile *t) {
 // small to give every warp 32 (at least 8), but no fewer than 2 K: an item
 // pays for loading its ligand, and has no K-th best of its own to stop starts
 // with before its K-th start.  A run of fewer than 4 starts per resident warp
-// spreads over all of them, in at most 512 items per ligand (their lists are
-// merged by one warp): every start is under way before a K-th best could stop
-// one (measured, lo = 128, 64, 32, 16, 8: one 24-atom
-// ligand with 512 starts and K = 4 372, 213, 135, 99 and 88 us; 301 ligands
-// with 1,717 starts and K = 5 4.9, 3.44, 3.19, 3.49 and 3.62 ms; 8 P in the
-// model against 12 P and 16 P: 1,000 ligands 24.1, 24.5, 25.1 ms).
+// spreads over all of them, in fewer than 1,024 items per ligand (their lists
+// are merged by one warp): every start is under way before a K-th best could
+// stop one (measured with the tables' kernel in place, lo = 128, 64, 32, 16, 8:
+// one 24-atom ligand with 512 starts and K = 4 372, 213, 135, 99 and 88 us; 301
+// ligands with 1,717 starts and K = 5 4.9, 3.44, 3.19, 3.49 and 3.62 ms; 8 P in
+// the model against 12 P and 16 P: 1,000 ligands 24.1, 24.5, 25.1 ms; n_starts
+// / 512 rounded up to whole start groups instead of down, for at most 512
+// items: one ligand at S = 32 with 1,000, 1,100 and 2,000 starts 238 -> 218, 227
+// -> 247 and 288 -> 309 us, at S = 16 with 1,100 and 1,500 180 -> 185 and 208 ->
+// 198).
 // Buckets without ligands get 512.  Ligands: sel[0..n) or all of B.
 static double least_chunk(double n, int n_starts, double P_warps, int K) {
   const double each = n * n_starts / std::max(P_warps, 1.0);
@@ -2116,7 +2123,7 @@ extern "C" ligate_status ligate_rescore_poses(const ligate_pocket *P, const liga
   st = base_params(P, B, s, mode, p, &rot, &anc, &quat);
   cudaError_t e = cudaSuccess;
   if (st == LIGATE_OK && rescore_smem_bytes(p, r, 1) > 227 * 1024) {
-    set_error("rescore_poses: %d receptor atoms do not fit in shared memory", r.n_rec);
+    set_error("rescore_poses: %d receptor atoms are more than rescoring takes", r.n_rec);
     st = LIGATE_ERR_UNSUPPORTED;
   }
   if (st == LIGATE_OK) {
@@ -2138,7 +2145,7 @@ extern "C" ligate_status ligate_plan_rescore(const ligate_plan *pl, ligate_resco
   const int n = pl->rows * pl->p.K;
   if (n == 0) return LIGATE_OK;
   if (rescore_smem_bytes(pl->p, r, 1) > 227 * 1024) {
-    set_error("plan_rescore: %d receptor atoms do not fit in shared memory", r.n_rec);
+    set_error("plan_rescore: %d receptor atoms are more than rescoring takes", r.n_rec);
     return LIGATE_ERR_UNSUPPORTED;
   }
   cudaError_t e = launch_rescore(pl->p, r, n, nullptr, nullptr, nullptr,
@@ -2167,7 +2174,7 @@ extern "C" ligate_status ligate_rescore_states(const ligate_pocket *P, const lig
   st = base_params(P, B, s, mode, p, &rot, &anc, &quat);
   cudaError_t e = cudaSuccess;
   if (st == LIGATE_OK && rescore_smem_bytes(p, r, 1) > 227 * 1024) {
-    set_error("rescore_states: %d receptor atoms do not fit in shared memory", r.n_rec);
+    set_error("rescore_states: %d receptor atoms are more than rescoring takes", r.n_rec);
     st = LIGATE_ERR_UNSUPPORTED;
   }
   if (st == LIGATE_OK) {
@@ -2195,7 +2202,7 @@ extern "C" ligate_status ligate_plan_rescore_refined(const ligate_plan *pl, cons
   const int n = pl->rows * pl->p.K;
   if (n == 0) return LIGATE_OK;
   if (rescore_smem_bytes(pl->p, r, 1) > 227 * 1024) {
-    set_error("plan_rescore_refined: %d receptor atoms do not fit in shared memory", r.n_rec);
+    set_error("plan_rescore_refined: %d receptor atoms are more than rescoring takes", r.n_rec);
     return LIGATE_ERR_UNSUPPORTED;
   }
   StateSrc ss;

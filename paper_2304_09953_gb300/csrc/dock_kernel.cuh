@@ -46,7 +46,7 @@ __device__ __forceinline__ float clash_sweep(const DockParams &p, const WarpSmem
                                              bool alive = true) {
   if (br.n_cand == 0) return 0.f;  // warp-uniform: every pair was memoised
   float ac = 0.f;
-  const int cap = PAIR_WARP / G;  // = 6 L
+  const int cap = PAIR_WARP / G;  // nearly 6 L
   float4 *list = w.list + g * cap;
   float2 *cab = w.cab + g * p.nmax;  // (axial a, radial distance b) of each atom
   const unsigned lmask = L == 32 ? FULL : ((1u << L) - 1u);
@@ -329,7 +329,9 @@ __device__ __forceinline__ bool beyond_bound(float lb, float thr) {
 // ---------------------------------------------------------------------------
 // CTAs of at most 128 threads; MINB of them must fit on one SM: 4 caps the
 // registers at 128 (16 resident warps), 5 at 102 (20 warps), 6 at 85 (24
-// warps, a few spills).
+// warps).  Bytes of frame, spill stores and spill loads: BF16 with 16 lanes per
+// start 16/0/0 at 128 registers and 80/52/92 at 96 (the call of build_memo holds
+// registers across it), generic 128/164/296 at 80.
 // Latency of the map gathers is covered by resident warps, so occupancy
 // matters more than per-thread registers here.
 template <int MODE, int MINB, int LT>

@@ -468,6 +468,9 @@ cudaError_t launch_pose_features(const DockParams &p, int n_poses, const int32_t
   return cudaGetLastError();
 }
 
+// Size by which rescoring accepts a receptor: 16 B per atom, the pair table, the
+// cell table and a warp's slot within a CTA's 227 KB, about 12,000 atoms.  The
+// kernel stages none of the receptor; the limit is the entry points' own.
 size_t rescore_smem_bytes(const DockParams &p, const RecParams &r, int warps) {
   const int ncells = r.ncx * r.ncy * r.ncz;
   return (size_t)r.n_rec * 16 + (size_t)((r.n_types * r.n_types + 1) & ~1) * 8 +
