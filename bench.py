@@ -84,7 +84,7 @@ def algorithmic_flops(work, S, n_starts, total_atoms):
 # valid only for the kernel revision it was captured on (sha1 prefix of
 # the docking kernel's files); any other revision reports null until it is
 # captured again.
-TRAFFIC_BYTES = {("cf4358d5f3d0", "batched", 10000): 104403456 + 24783104}
+TRAFFIC_BYTES = {("3f87d24975b7", "batched", 10000): 175107328 + 24531968}
 
 
 def kernel_source_sha():

@@ -25,7 +25,8 @@ namespace ligate {
 // builds each and sums the receptor term atom by atom (receptor_cells defines
 // the sum).
 //
-// What bounds it: instruction issue on the distance tests.  The 27 cells
+// What bounds it: issue and latency of the distance tests (65% of active cycles
+// issue; waits on fixed latency, L1 and branches).  The 27 cells
 // around an atom hold 6.4 times the atoms within the cutoff.  So each coarse
 // cell is split into fine cells about 2 A wide, and a fine cell has the
 // receptor atoms that can be within the cutoff of a point in it (1.8 times),
@@ -330,8 +331,9 @@ __global__ void __launch_bounds__(256) rescore_kernel(const __grid_constant__ Do
 // v >= 9); rest 0.  One warp per pose; the histogram lives in the warp's
 // pair-list slot.  An empty or invalid pose gives all zeros.
 //
-// What bounds it: instruction issue (about 2,500 warp instructions per pose
-// before, against 1 KB written).  Counts come from ballots, the per-type sums
+// What bounds it: instruction issue and the map gathers' latency (67% of active
+// cycles issue; about 2,500 warp instructions per pose before, against 1 KB
+// written).  Counts come from ballots, the per-type sums
 // share one butterfly, log1p of the counts comes from a table made by the same
 // function, the row is put together in shared memory and stored in 16-byte
 // pieces, and a warp takes consecutive poses, mostly of one ligand: 32,000
