@@ -2,7 +2,6 @@
 import contextlib
 import ctypes
 import glob
-import os
 
 
 def _cudart():

@@ -118,3 +118,18 @@ def test_quantile_captured_after_a_smaller_selection(batched_small):
         pl.best_quantile(0.5, cut, torch.cuda.current_stream().cuda_stream)
     graph.replay()
     assert cut.item() == best[w.ligands.n // 2 - 1]
+
+
+@pytest.mark.parametrize("S", [4, 8, 16, 18, 32])
+def test_small_runs_stay_below_1024_items(batched_small, S):
+    """A run of one ligand spreads its starts over the resident warps in fewer
+    than 1,024 items, whose lists one warp merges."""
+    w = batched_small
+    bh, ph = D.BatchHandle(w.ligands.subset([0])), D.PocketHandle(w.pocket)
+    for orient, anchor in ((20, 30), (31, 33), (33, 31), (48, 32), (64, 31), (128, 31)):
+        q = np.random.default_rng(orient).normal(size=(orient, 4))
+        samp = Sampling(q / np.linalg.norm(q, axis=1, keepdims=True), min(anchor, len(w.pocket.anchors)), S, 4)
+        pl = D.Plan(ph, bh, samp, mode="fp32c")
+        least = min(pl.tile()[0].starts_per_item)
+        assert least > 0 and -(-samp.n_starts // least) < 1024, (samp.n_starts, least)
+        pl.close()
