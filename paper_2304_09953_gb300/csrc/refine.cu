@@ -43,6 +43,13 @@ namespace {
 constexpr unsigned FULLM = 0xffffffffu;
 constexpr int NG = 6 + LIGATE_MAX_ROT;  // gradient components
 constexpr int NI = 1 + LIGATE_MAX_ROT;  // moments
+// Squared clash cutoff (A^2), by atoms per lane, from which enough pairs of a
+// ligand touch that finding them costs more than it saves (us with the search
+// and without, 16 iterations: 4,800 poses of the batched library at cutoffs of 3,
+// 4 and 8 A 342/358, 376/362, 481/362; 2,400 poses of 80 atoms at 4, 4.5 and 8 A
+// 482/502, 516/504, 632/506; of 120 atoms at 4, 5 and 8 A 768/870, 895/874,
+// 1085/876).
+constexpr float NEAR2_ALL[4] = {16.f, 16.f, 20.f, 25.f};
 constexpr uint32_t SEG_IDLE = 1u << 31;  // bond segment entry of a lane without a bond
 
 struct State {
@@ -152,8 +159,10 @@ struct RefineArgs {
 };
 
 // Energy and generalised gradient of state w.q[s] into w.G[s], w.I[s].  HW:
-// atoms per lane (n_atoms <= 32 HW).
-template <int HW>
+// atoms per lane (n_atoms <= 32 HW).  FIND: the pairs that may touch are found
+// first (clash cutoffs below NEAR2_ALL's), else every pair is visited; pairs that
+// do not touch add nothing, so the values are the same.
+template <int HW, bool FIND>
 __device__ float eval_state(const RefineArgs &a, const RSmem &w, const LigDesc &d, int s, int lane) {
   const DockParams &p = a.p;
   const State &q = w.q[s];
@@ -167,8 +176,8 @@ __device__ float eval_state(const RefineArgs &a, const RSmem &w, const LigDesc &
 #pragma unroll
   for (int h = 0; h < HW; ++h)
 #pragma unroll
-    for (int wd = 0; wd < HW; ++wd) hit[h][wd] = 0u;
-  {
+    for (int wd = 0; wd < HW; ++wd) hit[h][wd] = FIND || wd >= d.n_words ? 0u : ~0u;
+  if (FIND) {
     float4 own[HW];
 #pragma unroll
     for (int h = 0; h < HW; ++h)
@@ -336,7 +345,7 @@ __device__ void make_trial(const RSmem &w, int c, int n_atoms, int n_rot, float 
 
 // MODE 0: energy + gradient of explicit states; 1: refine explicit states;
 // 2: refine the plan's top-K poses.
-template <int MODE, int HW>
+template <int MODE, int HW, bool FIND>
 __global__ void __launch_bounds__(128) refine_kernel(const __grid_constant__ RefineArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -403,7 +412,7 @@ __global__ void __launch_bounds__(128) refine_kernel(const __grid_constant__ Ref
   __syncwarp();
   w.passes = bond_segments(w, d, lane);
 
-  float E = eval_state<HW>(a, w, d, 0, lane);
+  float E = eval_state<HW, FIND>(a, w, d, 0, lane);
   if (MODE == 0) {
     if (lane == 0) a.energy[pi] = E;
     for (int k = lane; k < NG; k += 32) a.grad[(size_t)pi * NG + k] = w.G[k];
@@ -416,7 +425,7 @@ __global__ void __launch_bounds__(128) refine_kernel(const __grid_constant__ Ref
   for (int it = 0; it < a.iters; ++it) {
     make_trial(w, cur, d.n_atoms, d.n_rot, eta, lane);
     __syncwarp();
-    const float Et = eval_state<HW>(a, w, d, 1 - cur, lane);
+    const float Et = eval_state<HW, FIND>(a, w, d, 1 - cur, lane);
     if (Et < E) {
       cur = 1 - cur;
       E = Et;
@@ -442,6 +451,20 @@ __global__ void __launch_bounds__(128) refine_kernel(const __grid_constant__ Ref
 
 size_t refine_smem_bytes(int nmax) { return refine_smem_per_warp(nmax); }
 
+namespace {
+template <bool FIND>
+const void *refine_fn(int mode, int hw) {
+  const void *const fns[3][4] = {
+      {(const void *)refine_kernel<0, 1, FIND>, (const void *)refine_kernel<0, 2, FIND>,
+       (const void *)refine_kernel<0, 3, FIND>, (const void *)refine_kernel<0, 4, FIND>},
+      {(const void *)refine_kernel<1, 1, FIND>, (const void *)refine_kernel<1, 2, FIND>,
+       (const void *)refine_kernel<1, 3, FIND>, (const void *)refine_kernel<1, 4, FIND>},
+      {(const void *)refine_kernel<2, 1, FIND>, (const void *)refine_kernel<2, 2, FIND>,
+       (const void *)refine_kernel<2, 3, FIND>, (const void *)refine_kernel<2, 4, FIND>}};
+  return fns[mode][hw - 1];
+}
+}  // namespace
+
 cudaError_t launch_refine(int mode, const DockParams &p, const double origin[3], double h, int n,
                           const int32_t *lig_idx, const ligate_pose_state *init, const ligate_pose *poses,
                           const int32_t *row_lig, int iters, float eta0, ligate_refined *out,
@@ -465,14 +488,8 @@ cudaError_t launch_refine(int mode, const DockParams &p, const double origin[3],
   const int warps = 4;
   const size_t smem = refine_smem_per_warp(p.nmax) * warps;
   const int hw = p.nmax > 32 ? (p.nmax + 31) / 32 : 1;  // atoms per lane: 1 to 4
-  const void *const fns[3][4] = {
-      {(const void *)refine_kernel<0, 1>, (const void *)refine_kernel<0, 2>, (const void *)refine_kernel<0, 3>,
-       (const void *)refine_kernel<0, 4>},
-      {(const void *)refine_kernel<1, 1>, (const void *)refine_kernel<1, 2>, (const void *)refine_kernel<1, 3>,
-       (const void *)refine_kernel<1, 4>},
-      {(const void *)refine_kernel<2, 1>, (const void *)refine_kernel<2, 2>, (const void *)refine_kernel<2, 3>,
-       (const void *)refine_kernel<2, 4>}};
-  const void *fn = fns[mode == 0 ? 0 : mode == 1 ? 1 : 2][hw - 1];
+  const int m = mode == 0 ? 0 : mode == 1 ? 1 : 2;
+  const void *fn = 1.f / p.inv_dc2_ang < NEAR2_ALL[hw - 1] ? refine_fn<true>(m, hw) : refine_fn<false>(m, hw);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   void *args[] = {&a};

@@ -13,7 +13,7 @@ from paper_2304_09953_gb300 import docking as D
 from paper_2304_09953_gb300 import native as N
 from paper_2304_09953_gb300.workload import Pocket, Sampling, make_ligands
 from tests.device_memory import all_but
-from tests.parity import Geometry, Stats, rescore_check
+from tests.parity import Geometry, Stats, check_state_energies, rescore_check
 from tests.test_gpu_refine import seeded_states, to_dev
 from tests.test_gpu_rescore import explicit
 
@@ -212,3 +212,36 @@ def test_listed_and_coarse_cells_give_the_same_bits(batched_small):
     assert np.array_equal(outs[0], outs[1])
     e = outs[0]["e_inter"]
     assert (e == 0).any() and (np.abs(e) > 1).sum() > len(e) // 2
+
+
+@pytest.mark.parametrize("cutoff", [3.99, 4.01, 4.48, 5.01, 30.0])
+def test_gradient_at_wide_clash_cutoffs(tiny, cutoff):
+    """Cutoffs from which the pairs that touch are not looked for, which depends
+    on the batch's largest ligand: energy and gradient are the same bits beside
+    a ligand that takes more atoms per lane, and the oracle's."""
+    own = make_ligands(8, np.array([20, 33, 64, 128], np.int32), np.array([3, 5, 6, 16], np.int32), 4)
+    samp = Sampling(tiny.sampling.quats, tiny.sampling.n_anchor, tiny.sampling.torsion_steps, tiny.sampling.top_k,
+                    clash_cutoff=cutoff)
+
+    class W:
+        pocket, ligands, sampling = tiny.pocket, own, samp
+
+    ph = D.PocketHandle(tiny.pocket)
+    s = N.make_sampling(samp, N.LIGATE_FP32, N.LIGATE_LAYOUT_PLAIN, False, None)
+    for li in range(3):
+        lig, rec, st64 = seeded_states(W, [li], np.random.default_rng(li), 17)
+        res = []
+        for ligs, at in ((own.subset([li]), 0), (own, li)):
+            bh = D.BatchHandle(ligs)
+            e = torch.zeros(len(lig), dtype=torch.float32, device="cuda")
+            g = torch.zeros((len(lig), N.LIGATE_GRAD_DIM), dtype=torch.float32, device="cuda")
+            N.ligate_pose_gradient(ph.h, bh.h, s, len(lig), torch.full((len(lig),), at, dtype=torch.int32,
+                                                                     device="cuda"), to_dev(rec), e, g)
+            res.append((e.cpu().numpy(), g.cpu().numpy()))
+            bh.close()
+        assert np.array_equal(res[0][0], res[1][0]) and np.array_equal(res[0][1], res[1][1])
+        e64, g64, sc, _, face = oracle.pose_grad(own.ligand(li), tiny.pocket, samp, np.array(st64))
+        check_state_energies(Geometry(tiny.pocket), own.ligand(li), tiny.pocket, samp, rec, st64, res[0][0], e64)
+        for k in np.nonzero(face >= 1e-4)[0]:  # the bar of the gradient's own test
+            np.testing.assert_array_less(np.abs(res[0][1][k, :g64.shape[1]] - g64[k]), 2e-4 * np.maximum(sc[k, 1:], 1.0))
+    ph.close()
